@@ -118,6 +118,7 @@ hydra_status lora_linear_impl(const void* x_off, const void* x_on, int64_t M, in
   g.err = err;
   g.epi = epi;
   g.single_cta = algo == 3;
+  g.x_settled = lora && !u_given;
   if (epi == kEpiRope) {
     g.rope_P = rope->P;
     g.rope_cols = rope->cols;
@@ -351,6 +352,7 @@ hydra_status hydra_lora_linear_tri(const void* x_off, const void* x_act, const v
   g.y_off = y_off;
   g.y_on = y_act;
   g.y_crit = y_crit;
+  g.x_settled = lora_a || lora_c;
   g.out_f32 = out_dtype == HYDRA_F32 ? 1 : 0;
   g.err = err;
   return hydra::launch_dual_lora_gemm_tc(g, st) == 0 ? HYDRA_OK : HYDRA_ERR_CUDA;
@@ -413,6 +415,7 @@ hydra_status hydra_lm_head_logprobs(const void* h_off, const void* h_on, int64_t
   g.out_f32 = 1;
   g.err = err;
   g.epi = 4;
+  g.x_settled = r > 0;
   g.lsm_target = tgt;
   g.lsm_ids = ids;
   g.lsm_L = L;

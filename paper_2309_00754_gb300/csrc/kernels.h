@@ -54,6 +54,9 @@ struct GemmArgs {
   int epi = 0;        // tcgen05 epilogue: 0 store, 1 SwiGLU, 2 residual add (fp32), 3 rotary,
                       // 4 log-softmax partials
   bool single_cta = false;  // tcgen05: never use the CTA-pair (cta_group::2) kernel
+  // the kernel launched just before on the stream is this call's lora_down: the inputs x were
+  // final before it let its dependents start (only u is still being written)
+  bool x_settled = false;
   // epi 3 (rotary): columns [0, rope_cols) rotate in heads of 128 at position row % rope_P,
   // by the (cos, sin) pairs of rope_table [rope_P][64] (launch_rope_table)
   int64_t rope_P = 1;
@@ -71,6 +74,10 @@ struct GemmArgs {
 int* device_error_word();
 
 int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream);
+// The same linear for few token rows per stream (lora_gemm_small.cu), which
+// launch_dual_lora_gemm_tc takes where small_gemm_wanted.
+bool small_gemm_wanted(int64_t M, int64_t K, int64_t N);
+int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream);
 // TMA map over a row-major [rows, cols] bf16 (or fp32) matrix with row stride ld elements:
 // 128-byte swizzle, boxes of [box_rows x 128 bytes], zero fill out of bounds
 bool make_tma_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld,

@@ -1,0 +1,889 @@
+// The dual-output LoRA linear (see lora_gemm_tc.cu for the mathematics) for up to 384 token rows
+// per stream: one short sequence, a prompt, a decode batch. The work there is reading W once, and
+// the tile kernel of lora_gemm_tc.cu leaves most of the chip idle: 97 rows of two streams by 4096
+// columns are 32 tiles of 128 x 256, each with the whole of K, on 152 SMs.
+//
+// A CTA pair (tcgen05 cta_group::2) computes a tile of two row segments by bn columns:
+//  * Row segments. Every stream's rows are cut into equal segments of at most 128 rows, and the
+//    segments of all streams, in order, are taken two by two: segment 2 i is the first CTA's 128
+//    accumulator rows, 2 i + 1 the second's. Up to 128 rows, a pair holds the off and the on
+//    stream of the same rows, so one pass over a W tile serves both; three segments per stream
+//    make three pairs, not four.
+//  * Columns and K. bn (a multiple of 32 up to 256) and the split of K over ks pairs of a cluster
+//    (1 or 2) are chosen so that the pairs fill the SMs. ks depends on M, K and N alone, so that
+//    every output element is one sum in one order whatever the streams, the epilogue and the tile
+//    width: shared, stacked and three-stream calls agree bit for bit. (Four slices measured
+//    slower: only 15 clusters of eight CTAs fit on the chip, 36 of four.)
+//  * Ring items are two k-blocks of 64, and x and W have a TMA warp each. What a warp executes
+//    per item is the limit at these sizes: one warp and 64-wide items took 570 clocks each, more
+//    than the products of a tile (97 x 4096 x 12288: 44.8 us, now 26.5).
+//  * LoRA. The k-blocks of u B^T go to the last K slice and accumulate in TMEM columns of their
+//    own; y_on's partial sum there is main + lora. No drain waits for them, and a pair with an
+//    off segment never mixes B into the off rows (their part of that accumulator is not read).
+//  * Reduction and epilogue. Each of two K slices finishes half of the tile's columns: it takes
+//    the other slice's fp32 sums of those columns, pushed into its drained ring through
+//    distributed shared memory. Two warps per TMEM lane quarter drain alternate 32-column chunks
+//    through small swizzled buffers into whole-line stores (the residual add as one fp32
+//    reduction per element in L2).
+//  * Dependent launch. W is frozen: the first ring of W boxes loads before the wait on the
+//    preceding kernel. Where that kernel is this call's own lora_down (which waits for its
+//    predecessors before it lets this kernel start), x is final already and the whole main loop
+//    overlaps it; only u is waited for.
+//
+// What bounds it: HBM for W, and an SM's fill from L2 (64 B per clock: a k-block of 64 costs
+// 2 (seg + bn / 2) clocks of fill for 2 bn clocks of products), which is why the x boxes are as
+// high as the segment and not 128 rows. 97 rows x 4096 x 12288 (two streams): the main loop runs
+// at 6.6 TB/s of W; about 6 us of the 26.5 are set-up, first loads, drain and stores.
+#include <float.h>
+
+#include <mutex>
+#include <vector>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace hydra {
+namespace smallm {
+
+constexpr int BK = 128;  // a ring item: two k-blocks of 64 (128-byte swizzle each)
+// warp 0: TMA of W; 1: TMEM and MMA; 2: TMA of x; 3: barriers, L2 prefetch; 4-11: drain (two warps
+// per quarter of the TMEM lanes, alternate column chunks each)
+constexpr int NUM_THREADS = 384;
+constexpr int kMaxStages = 12;
+constexpr int kSmemMax = 232448;  // dynamic shared memory of one CTA (227 KiB)
+constexpr int kBarBytes = (2 * kMaxStages + 1) * 8 + 16;
+
+enum { EPI_STORE = 0, EPI_SWIGLU = 1, EPI_RESIDUAL = 2, EPI_ROPE = 3, EPI_LOGSOFTMAX = 4 };
+
+struct Maps {
+  CUtensorMap x[3];
+  CUtensorMap w;
+  CUtensorMap u[2];
+  CUtensorMap b[2];
+};
+
+struct Params {
+  int M, N;
+  int streams, nseg, seg, row_tiles;  // nseg segments of seg rows per stream
+  int kb_main, kb_lora, r;
+  int bn, ks, stages;
+  int shared_x, both;   // both: shared input with LoRA and both outputs wanted
+  int has_on, has_crit;
+  int epi, out_f32;
+  int paired;    // SwiGLU / rotary: tile columns [0, bn/2) and [bn/2, bn) are partner columns
+  int b_box;     // rows of a W / B box
+  int x_settled; // x is final before the preceding kernel of the stream ends
+  int lcol;      // TMEM column of the LoRA accumulator
+  uint32_t tmem_cols;
+  int stg_off;   // byte offset of the drain warps' staging buffers (over the drained ring)
+  int bar_off;
+  void* y[3];
+  int rope_P, rope_cols;
+  const float2* rope_table;
+  float* lsm_target;
+  const int32_t* lsm_ids;
+  int lsm_L, lsm_ids_ld, lsm_ids_off, lsm_tiles;
+  int* err;
+};
+
+__device__ __forceinline__ void commit_pair_mask(uint32_t bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(bar),
+      "h"(mask)
+      : "memory");
+}
+__device__ __forceinline__ void st_cluster_f4(uint32_t cluster_addr, const uint32_t* v) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+// bring the box at (x, y) of a tensor map into L2
+__device__ __forceinline__ void prefetch_box(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y)
+               : "memory");
+}
+__device__ __forceinline__ float bf16_round(float v) {
+  return __bfloat162float(__float2bfloat16_rn(v));
+}
+
+// W row of the tile's B row j of CTA half `half`, whose first row is `first` (a pair index for
+// the paired layouts): SwiGLU gate / up blocks of 128 rows, rotary halves of 64 rows of a head
+__device__ __forceinline__ int b_row(const Params& p, int n0, int half, int j) {
+  if (!p.paired) return n0 + half * (p.bn / 2) + j;
+  const int q = n0 / 2 + j;
+  return p.epi == EPI_SWIGLU ? (q >> 7) * 256 + half * 128 + (q & 127)
+                             : (q >> 6) * 128 + half * 64 + (q & 63);
+}
+
+__device__ __forceinline__ uint4 pack8(const float* v) {
+  return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
+                    pack_bf16x2(v[6], v[7]));
+}
+
+// An epilogue thread's accumulator row: its sums, 32 tile columns at a time.
+struct RowSums {
+  uint32_t taddr;  // TMEM address of the thread's lane, column 0 of the main accumulator
+  int lcol;        // columns from there to the LoRA accumulator
+  bool own_lora;   // this CTA holds the LoRA sums
+  const float4* recv;  // the other K slice's sums of this CTA's columns (ks == 2), else NULL
+  int lplane;      // float4 from there to the LoRA sums sent along (shared input, slice 0), or 0
+  int row;         // row of the tile (TMEM lane)
+
+  // v = the sums of columns [c, c + 32), the LoRA term included or not; pos: index of the chunk
+  // among those this CTA finishes. LoRA joins the last slice's sum before the slices are added.
+  __device__ __forceinline__ void get(int c, int pos, bool lora, float (&v)[32]) const {
+    uint32_t a[32];
+    tc_ld_32x32b_x32(taddr + c, a);
+    if (lora && own_lora) {
+      uint32_t l[32];
+      tc_ld_32x32b_x32(taddr + lcol + c, l);
+      tc_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(l[i]);
+    } else {
+      tc_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(a[i]);
+    }
+    if (recv == nullptr) return;
+    const float4* s = recv + pos * 8 * 128 + row;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float4 t = s[j * 128];
+      if (lora && lplane != 0) {
+        const float4 l = s[lplane + j * 128];
+        t.x += l.x; t.y += l.y; t.z += l.z; t.w += l.w;
+      }
+      v[4 * j] += t.x; v[4 * j + 1] += t.y; v[4 * j + 2] += t.z; v[4 * j + 3] += t.w;
+    }
+  }
+};
+
+// A drain warp's staging buffer: 32 rows of up to eight 16-byte pieces (piece index XOR row, so
+// neither side conflicts). A thread writes the pieces of its own accumulator row; flush() stores
+// them so that neighbouring lanes cover one row's line (a thread storing its own row touches 32
+// lines per instruction, which cost 2 us of a 20 us launch).
+struct Staging {
+  uint4* buf;
+  int lane, rows;  // rows: valid rows of the warp
+
+  __device__ __forceinline__ void put(int piece, uint4 v) const { buf[lane * 8 + (piece ^ (lane & 7))] = v; }
+  // kPieces pieces per row to base + row * ld (bytes); `keep` of them lie inside the output
+  template <int kPieces, bool kAdd>
+  __device__ __forceinline__ void flush(uint8_t* base, size_t ld, int keep) const {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kPieces; ++i) {
+      const int e = i * 32 + lane, r = e / kPieces, c = e % kPieces;
+      if (r < rows && c < keep) {
+        const uint4 v = buf[r * 8 + (c ^ (r & 7))];
+        uint8_t* d = base + r * ld + c * 16;
+        if (kAdd)  // one addend per element and call: the sum does not depend on any order
+          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(d), "f"(__uint_as_float(v.x)),
+                       "f"(__uint_as_float(v.y)), "f"(__uint_as_float(v.z)), "f"(__uint_as_float(v.w))
+                       : "memory");
+        else
+          *reinterpret_cast<uint4*>(d) = v;
+      }
+    }
+    __syncwarp();
+  }
+};
+
+// Store 32 sums of the thread's row at output columns [n, n + 32) (N % 8 == 0). `y` is the row of
+// the warp's lane 0.
+__device__ __forceinline__ void store32(const Params& p, const Staging& st, void* y, int n,
+                                        const float (&v)[32]) {
+  const int left = p.N - n;
+  if (p.epi == EPI_RESIDUAL || p.out_f32) {
+    const bool add = p.epi == EPI_RESIDUAL;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float* w = v + 4 * j;
+      st.put(j, add ? make_uint4(__float_as_uint(bf16_round(w[0])), __float_as_uint(bf16_round(w[1])),
+                                 __float_as_uint(bf16_round(w[2])), __float_as_uint(bf16_round(w[3])))
+                    : make_uint4(__float_as_uint(w[0]), __float_as_uint(w[1]), __float_as_uint(w[2]),
+                                 __float_as_uint(w[3])));
+    }
+    uint8_t* d = reinterpret_cast<uint8_t*>(static_cast<float*>(y) + n);
+    const size_t ld = static_cast<size_t>(p.N) * 4;
+    if (add) st.flush<8, true>(d, ld, left / 4);
+    else st.flush<8, false>(d, ld, left / 4);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) st.put(j, pack8(v + 8 * j));
+  st.flush<4, false>(reinterpret_cast<uint8_t*>(static_cast<__nv_bfloat16*>(y) + n),
+                     static_cast<size_t>(p.N) * 2, left / 8);
+}
+
+// 32 partner columns of a paired tile: q is the first one's pair index, v / z the sums of the
+// first and the second half; row: the thread's row, y: the output's first element
+__device__ __forceinline__ void store_pair32(const Params& p, const Staging& st, void* y, int row,
+                                             int q, float (&v)[32], float (&z)[32]) {
+  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(y);
+  const size_t row0 = static_cast<size_t>(row - st.lane);
+  if (p.epi == EPI_SWIGLU) {
+    if (q >= p.N / 2) return;  // N % 256 == 0: 32 pairs are all in or all out
+    // the bf16 gates and ups through the staging buffer, and a short loop from there: unrolled
+    // over 32 registers, the quotients are 30 KB of code that every launch fetches anew (6 us
+    // of a 53 us launch)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      st.put(j, pack8(v + 8 * j));
+      st.put(4 + j, pack8(z + 8 * j));
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {
+      const int e = i * 32 + st.lane, r = e >> 2, c = e & 3;
+      if (r < st.rows) {
+        const uint4 g4 = st.buf[r * 8 + (c ^ (r & 7))], u4 = st.buf[r * 8 + ((4 + c) ^ (r & 7))];
+        uint4 o;
+        const uint32_t *gp = &g4.x, *up = &u4.x;
+        uint32_t* op = &o.x;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 g = unpack_bf16x2(gp[k]), u = unpack_bf16x2(up[k]);
+          op[k] = pack_bf16x2(g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y);
+        }
+        *reinterpret_cast<uint4*>(out + (row0 + r) * (p.N / 2) + q + 8 * c) = o;
+      }
+    }
+    __syncwarp();
+    return;
+  }
+  // rotary: the roundings of hydra_rope on the bf16-rounded sums
+  const int i0 = q & 63, na = (q >> 6) * 128 + i0;
+  if (na < p.rope_cols) {  // whole heads: rope_cols % 128 == 0
+    const float4* cs = reinterpret_cast<const float4*>(p.rope_table + (row % p.rope_P) * 64 + i0);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float4 t = __ldg(cs + i);
+      const float a0 = bf16_round(v[2 * i]), a1 = bf16_round(v[2 * i + 1]);
+      const float b0 = bf16_round(z[2 * i]), b1 = bf16_round(z[2 * i + 1]);
+      v[2 * i] = __fsub_rn(__fmul_rn(a0, t.x), __fmul_rn(b0, t.y));
+      v[2 * i + 1] = __fsub_rn(__fmul_rn(a1, t.z), __fmul_rn(b1, t.w));
+      z[2 * i] = __fadd_rn(__fmul_rn(a0, t.y), __fmul_rn(b0, t.x));
+      z[2 * i + 1] = __fadd_rn(__fmul_rn(a1, t.w), __fmul_rn(b1, t.z));
+    }
+  }
+  uint8_t* o = reinterpret_cast<uint8_t*>(out + row0 * p.N + na);
+  const size_t ld = static_cast<size_t>(p.N) * 2;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) st.put(j, pack8(v + 8 * j));
+  st.flush<4, false>(o, ld, (p.N - na) / 8);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) st.put(j, pack8(z + 8 * j));
+  st.flush<4, false>(o + 128, ld, (p.N - na - 64) / 8);
+}
+
+// Log-softmax partials of the thread's row over a tile of 256 columns: the online (max, sum of
+// exp) pair of alternate chunks in each of the row's two warps, merged through `half` (32 pairs of
+// this quarter), and, where it lies, the sampled token's logit (an arithmetic select keeps the
+// row in registers).
+__device__ __forceinline__ void emit_lsm(const Params& p, const RowSums& r, int row, bool live, int n0,
+                                         float2* part, float* target, bool lora, int par, int q,
+                                         float2* half) {
+  int id = -1;
+  if (live) {
+    const int sq = row / p.lsm_L;
+    id = p.lsm_ids[static_cast<int64_t>(sq) * p.lsm_ids_ld + p.lsm_ids_off + row - sq * p.lsm_L];
+  }
+  float m = -FLT_MAX, sum = 0.f;
+  for (int c = 32 * par; c < 256; c += 64) {
+    const int nv = p.N - (n0 + c);
+    if (nv <= 0) break;  // uniform over the warp
+    float v[32];
+    r.get(c, 0, lora, v);
+    float mx = -FLT_MAX;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j < nv) mx = fmaxf(mx, v[j]);
+    if (mx > m) {
+      sum *= __expf(m - mx);
+      m = mx;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j < nv) sum += __expf(v[j] - m);
+    const int k = id - (n0 + c);
+    if (k >= 0 && k < min(nv, 32)) {
+      float z = 0.f;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) z += (k == j) ? v[j] : 0.f;
+      target[row] = z;
+    }
+  }
+  const int lane = threadIdx.x & 31;
+  if (par == 1) half[lane] = make_float2(m, sum);
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
+  if (par == 0 && live) {
+    const float2 o = half[lane];
+    const float t = fmaxf(m, o.x);
+    part[static_cast<int64_t>(row) * p.lsm_tiles + n0 / 256] =
+        make_float2(t, sum * __expf(m - t) + o.y * __expf(o.x - t));
+  }
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");  // the buffer serves the next output
+}
+
+__global__ void __launch_bounds__(NUM_THREADS)
+    lora_gemm_small_kernel(const __grid_constant__ Maps mp, const __grid_constant__ Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.bar_off);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const uint32_t smem_base = smem_u32(smem);
+  auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+  auto empty_bar = [&](int s) { return smem_u32(&bars[kMaxStages + s]); };
+  const uint32_t acc_full = smem_u32(&bars[2 * kMaxStages]);
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(p.tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  } else if (warp == 3) {
+    if (lane < p.stages) {
+      mbar_init(full_bar(lane), 1);
+      mbar_init(empty_bar(lane), 1);
+    }
+    if (lane == 0) {
+      mbar_init(acc_full, 1);
+      *abort_flag = 0;
+    }
+    __syncwarp();
+    fence_mbar_init();
+  }
+  tc_fence_before();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+
+  // (grid: x = the cluster's CTAs, y = row tile, z = column tile)
+  const int rank = static_cast<int>(cluster_rank());
+  const int half = rank & 1;        // which CTA of the pair
+  const int slice = rank >> 1;      // which K slice
+  const bool leader = half == 0;
+  const uint32_t lead_rank = static_cast<uint32_t>(rank & ~1);
+  const uint16_t pair_mask = static_cast<uint16_t>(3u << lead_rank);
+  const int n0 = static_cast<int>(blockIdx.z) * p.bn;
+
+  // the pair's two segments: stream and index within it (no divisions: at most three streams)
+  auto stream_of = [&](int g) { return (g >= p.nseg ? 1 : 0) + (g >= 2 * p.nseg ? 1 : 0); };
+  auto rows_of = [&](int g) {  // valid rows of segment g
+    if (g >= p.streams * p.nseg) return 0;
+    return max(0, min(p.seg, p.M - (g - stream_of(g) * p.nseg) * p.seg));
+  };
+  const int g0 = 2 * static_cast<int>(blockIdx.y), g1 = g0 + 1, gm = g0 + half;
+  const int nrow = rows_of(gm);
+  const int stream = nrow > 0 ? stream_of(gm) : 0;
+  const int m0 = nrow > 0 ? (gm - stream * p.nseg) * p.seg : 0;
+  const bool full1 = rows_of(g1) > 0;  // the second CTA has rows (the first always has)
+  auto lora_of = [&](int g) {
+    if (p.kb_lora == 0 || rows_of(g) == 0) return false;
+    if (p.shared_x) return p.has_on != 0;
+    const int s = stream_of(g);
+    return s == 1 ? p.has_on != 0 : (s == 2 ? p.has_crit != 0 : false);
+  };
+  const bool lora0 = lora_of(g0), lora1 = lora_of(g1), lora_me = half ? lora1 : lora0;
+  const int lset = !p.shared_x && stream_of(lora1 ? g1 : g0) == 2 ? 1 : 0;
+
+  const int kb0 = slice * p.kb_main / p.ks;
+  const int kb1 = (slice + 1) * p.kb_main / p.ks;
+  const int n_main = kb1 - kb0;
+  const int items = n_main + (slice == p.ks - 1 && (lora0 || lora1) ? p.kb_lora : 0);
+  const uint32_t a_bytes = static_cast<uint32_t>(p.seg) * 128;  // one k-block of this CTA's rows
+  const uint32_t b_bytes = static_cast<uint32_t>(p.bn) * 64;    // and of its half of the columns
+  const uint32_t stage_bytes = 2 * (a_bytes + b_bytes);         // [x, x, W, W]
+  // bytes of an item with `kbs` k-blocks landing on the pair's barrier
+  auto tx_bytes = [&](bool lora, uint32_t kbs) {
+    const uint32_t ctas = lora ? (lora0 ? 1u : 0u) + (lora1 ? 1u : 0u) : (full1 ? 2u : 1u);
+    return kbs * (ctas * a_bytes + 2 * b_bytes);
+  };
+  // k-blocks of 64 of LoRA item i (the second may be absent)
+  auto lora_kbs = [&](int i) { return p.r - i * BK > 64 ? 2 : 1; };
+
+  // before the barrier ends: descriptors, and this CTA's first W boxes into L2 (W is frozen)
+  const int nbox = p.bn / 2 / p.b_box;  // at most 4
+  int brow[4];                          // W rows of the boxes
+#pragma unroll
+  for (int j = 0; j < 4; ++j) brow[j] = b_row(p, n0, half, j * p.b_box);
+  if (warp == 0 && elect_one()) {
+    tma_prefetch_desc(&mp.w);
+    if (lora0 || lora1) tma_prefetch_desc(&mp.b[lset]);
+  }
+  if (warp == 2 && elect_one()) {
+    tma_prefetch_desc(&mp.x[stream]);
+    if (lora0 || lora1) tma_prefetch_desc(&mp.u[lset]);
+  }
+  if (warp == 3 && elect_one()) {
+    for (int i = 0; i < min(n_main, p.stages); ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < nbox) {
+          prefetch_box(&mp.w, (kb0 + i) * BK, brow[j]);
+          prefetch_box(&mp.w, (kb0 + i) * BK + 64, brow[j]);
+        }
+  }
+  __syncwarp();
+  // every CTA of the cluster has started, its barriers initialised
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  tc_fence_after();
+  const uint32_t tmem_acc = *tmem_slot;
+
+  bool epi_ok = false;
+  if (warp == 0 || warp == 2) {
+    // ------------------------------------------------------------------ TMA producers: warp 0
+    // moves W (and B), warp 2 x (and u). Everything an item needs is a running value, an item is
+    // two k-blocks and the two operands have a warp each: one warp with 64-wide items took about
+    // 570 clocks per item (a wait alone is 140), more than the pair's products.
+    const uint32_t lead_full0 = map_to_rank(full_bar(0), lead_rank);
+    const CUtensorMap* tm_main = warp == 0 ? &mp.w : &mp.x[stream];
+    const CUtensorMap* tm_lora = warp == 0 ? &mp.b[lset] : &mp.u[lset];
+    const uint32_t box_bytes = static_cast<uint32_t>(p.b_box) * 128;
+    auto load_b = [&](uint32_t stage, uint32_t fbar, uint32_t bar, bool lora, int i, int kbs) {
+      if (leader) mbar_arrive_expect_tx(fbar, tx_bytes(lora, kbs));
+      const CUtensorMap* m = lora ? tm_lora : tm_main;
+      const int k = i * BK;
+      uint32_t dst = stage + 2 * a_bytes;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < nbox) tma_load_2d_pair(dst + j * box_bytes, m, k, brow[j], bar);
+      if (kbs == 2) {
+        dst += b_bytes;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j < nbox) tma_load_2d_pair(dst + j * box_bytes, m, k + 64, brow[j], bar);
+      }
+    };
+    const int pre = min(items, p.stages);
+    int it = 0, s = 0;
+    uint32_t ph = 0;  // parity of the next wait on stage s: its previous use is done
+    if (warp == 0) {
+      // W and B are frozen: nothing of them is waited for
+      for (; it < items; ++it) {
+        if (it >= pre && !warp_wait_bounded(empty_bar(s), ph, abort_flag, p.err, kDevTimeoutProducer))
+          break;
+        if (elect_one()) {
+          const bool lora = it >= n_main;
+          load_b(smem_base + s * stage_bytes, full_bar(s), lead_full0 + s * 8, lora,
+                 lora ? it - n_main : kb0 + it, lora ? lora_kbs(it - n_main) : 2);
+        }
+        __syncwarp();
+        if (++s == p.stages) {
+          s = 0;
+          if (it >= pre) ph ^= 1;  // the first ring waits for nothing
+        }
+      }
+    } else {
+      if (!p.x_settled) pdl_wait();  // x is written by the preceding kernel
+      for (; it < items; ++it) {
+        const bool lora = it >= n_main;
+        if (it == n_main && p.x_settled) pdl_wait();  // u is written by the preceding kernel
+        if (it >= pre && !warp_wait_bounded(empty_bar(s), ph, abort_flag, p.err, kDevTimeoutProducer))
+          break;
+        if ((lora ? lora_me : nrow > 0) && elect_one()) {
+          const uint32_t dst = smem_base + s * stage_bytes, bar = lead_full0 + s * 8;
+          const CUtensorMap* m = lora ? tm_lora : tm_main;
+          const int k = (lora ? it - n_main : kb0 + it) * BK;
+          tma_load_2d_pair(dst, m, k, m0, bar);
+          if (!lora || lora_kbs(it - n_main) == 2) tma_load_2d_pair(dst + a_bytes, m, k + 64, m0, bar);
+        }
+        __syncwarp();
+        if (++s == p.stages) {
+          s = 0;
+          if (it >= pre) ph ^= 1;
+        }
+      }
+    }
+    // copies in flight land before shared memory is reused: a stage's empty barrier is
+    // committed after the products that read it
+    for (int k = (it > p.stages ? it - p.stages : 0); k < it; ++k) {
+      volatile int no_abort = 0;
+      warp_wait_bounded(empty_bar(k % p.stages), (k / p.stages) & 1, &no_abort, p.err, kDevTimeoutDrain);
+    }
+  } else if (warp == 1) {
+    if (leader) {
+      // ---------------------------------------------------------------- MMA issuer
+      const uint32_t idesc = idesc_bf16_f32(256, p.bn);
+      int s = 0;
+      uint32_t ph = 0;
+      for (int it = 0; it < items; ++it) {
+        if (!warp_wait_bounded(full_bar(s), ph, abort_flag, p.err, kDevTimeoutMma)) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t st = smem_base + s * stage_bytes;
+          const uint64_t a0 = smem_desc_sw128(st), a1 = smem_desc_sw128(st + a_bytes);
+          const uint64_t b0 = smem_desc_sw128(st + 2 * a_bytes);
+          const uint64_t b1 = smem_desc_sw128(st + 2 * a_bytes + b_bytes);
+          if (it < n_main) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)  // + 32 bytes per k-step: 2 in the address field
+              tc_mma2_bf16(tmem_acc, a0 + 2 * k, b0 + 2 * k, idesc, (it > 0 || k > 0) ? 1u : 0u);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tc_mma2_bf16(tmem_acc, a1 + 2 * k, b1 + 2 * k, idesc, 1u);
+          } else {
+            const int nsub = min(BK / 16, (p.r - (it - n_main) * BK + 15) / 16);
+            for (int k = 0; k < nsub; ++k)
+              tc_mma2_bf16(tmem_acc + p.lcol, (k < 4 ? a0 : a1) + 2 * (k & 3),
+                           (k < 4 ? b0 : b1) + 2 * (k & 3), idesc, (it > n_main || k > 0) ? 1u : 0u);
+          }
+          commit_pair_mask(empty_bar(s), pair_mask);
+        }
+        __syncwarp();
+        if (++s == p.stages) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      // arrives in both CTAs once every product issued above is done (after an abort too)
+      if (elect_one()) commit_pair_mask(acc_full, pair_mask);
+      __syncwarp();
+    }
+    volatile int no_abort = 0;
+    warp_wait_bounded(acc_full, 0, &no_abort, p.err, kDevTimeoutDrain);
+  } else if (warp >= 4) {
+    // -------------------------------------------------------------------- drain
+    epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
+    epi_ok = __all_sync(0xffffffffu, epi_ok) && *abort_flag == 0;
+    tc_fence_after();
+  }
+  pdl_launch_dependents();
+
+  const int q = warp & 3;             // TMEM lanes 32 q .. of a drain warp
+  const int trow = q * 32 + lane;     // row of the segment
+  const int par = (warp >> 2) & 1;    // which of the two warps of its lanes
+  const bool drain = warp >= 4 && epi_ok && q * 32 < nrow;
+  const bool last = slice == p.ks - 1;
+  const int nch = p.bn / 32;          // column chunks of the tile
+  // the slice that finishes chunk i (two slices: halves of the columns, or of the pairs), and
+  // the chunk's index among those it finishes
+  auto owner = [&](int i) {
+    return p.ks == 1 ? 0 : (p.paired ? (i % (nch / 2)) / (nch / 4) : i / (nch / 2));
+  };
+  auto pos_of = [&](int i) {
+    return p.ks == 1 ? 0 : (p.paired ? i % (nch / 4) + (i / (nch / 2)) * (nch / 4) : i % (nch / 2));
+  };
+  RowSums rs;
+  rs.taddr = tmem_acc + (static_cast<uint32_t>(q * 32) << 16);
+  rs.lcol = p.lcol;
+  rs.own_lora = last && lora_me;
+  rs.row = trow;
+  rs.recv = nullptr;
+  rs.lplane = 0;
+  if (p.ks == 2) {
+    const int plane = nch / 2 * 8 * 128;  // float4 of one slice's sums
+    float4* xch = reinterpret_cast<float4*>(smem);
+    cluster_sync_all();  // both slices' products are done: the rings are free
+    if (drain) {
+      const uint32_t dst0 = map_to_rank(smem_u32(xch + trow), static_cast<uint32_t>(2 * (1 - slice) + half));
+      for (int i = 0; i < nch; ++i) {
+        if (owner(i) == slice || (i & 1) != par) continue;
+        uint32_t v[32], l[32];
+        tc_ld_32x32b_x32(rs.taddr + 32 * i, v);
+        if (rs.own_lora) tc_ld_32x32b_x32(rs.taddr + p.lcol + 32 * i, l);
+        tc_wait_ld();
+        if (rs.own_lora && !p.both) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(l[j]));
+        }
+        const uint32_t dst = dst0 + pos_of(i) * (8 * 128 * 16);
+        if (trow < nrow) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) st_cluster_f4(dst + j * 2048, v + 4 * j);
+          if (rs.own_lora && p.both) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) st_cluster_f4(dst + plane * 16 + j * 2048, l + 4 * j);
+          }
+        }
+      }
+    }
+    rs.recv = xch;
+    rs.lplane = p.both && slice == 0 ? plane : 0;
+    tc_fence_before();
+    cluster_sync_all();  // the other slice's sums have landed
+    tc_fence_after();
+  }
+  if (drain) {
+    pdl_wait();  // outputs are written only after the preceding kernel
+    const bool live = trow < nrow;
+    const int row = m0 + trow;
+    const Staging st{reinterpret_cast<uint4*>(smem + p.stg_off) + (warp - 4) * 256, lane, nrow - q * 32};
+    const size_t warp_row = static_cast<size_t>(m0 + q * 32);
+    const size_t elem = p.out_f32 || p.epi == EPI_RESIDUAL ? 4 : 2;
+    for (int o = 0; o < 2; ++o) {
+      void* y;
+      bool lora;
+      if (p.shared_x) {
+        y = p.y[o];
+        lora = o == 1;
+      } else {
+        y = o == 0 ? p.y[stream] : nullptr;
+        lora = true;
+      }
+      if (y == nullptr) continue;
+      if (p.epi == EPI_LOGSOFTMAX) {
+        emit_lsm(p, rs, row, live, n0, static_cast<float2*>(y),
+                 p.lsm_target + ((p.shared_x ? o : stream) == 0 ? 0 : p.M), lora, par, q,
+                 reinterpret_cast<float2*>(smem + p.stg_off) + q * 32);
+      } else if (!p.paired) {
+        for (int i = 0; i < nch; ++i) {
+          if (owner(i) != slice || (i & 1) != par || n0 + 32 * i >= p.N) continue;
+          float v[32];
+          rs.get(32 * i, pos_of(i), lora, v);
+          store32(p, st, static_cast<uint8_t*>(y) + warp_row * p.N * elem, n0 + 32 * i, v);
+        }
+      } else {
+        for (int i = 0; i < nch / 2; ++i) {
+          if (owner(i) != slice || (i & 1) != par) continue;
+          float v[32], z[32];
+          rs.get(32 * i, pos_of(i), lora, v);
+          rs.get(32 * (i + nch / 2), pos_of(i + nch / 2), lora, z);
+          store_pair32(p, st, y, row, n0 / 2 + 32 * i, v, z);
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  // no CTA leaves while a peer may touch its barriers or shared memory. Relaxed: nothing is
+  // published here, and a releasing arrive would wait for the outputs to reach memory (2 us)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  __syncwarp();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc),
+                 "r"(p.tmem_cols)
+                 : "memory");
+  }
+}
+
+}  // namespace smallm
+// ------------------------------------------------------------------ host side
+
+namespace {
+
+using smallm::kBarBytes;
+using smallm::kMaxStages;
+using smallm::kSmemMax;
+
+int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
+int pow2_at_least(int v) {
+  int p = 32;
+  while (p < v) p *= 2;
+  return p;
+}
+
+struct Shape {  // what the launch needs besides the arguments
+  int streams, nseg, seg, row_tiles, ks;
+  bool lora, both, paired;
+};
+
+struct Config {
+  int bn, stages;
+  int stg_off, bar_off, smem;
+};
+
+// Shared-memory layout for a tile width; false if it does not fit with 3 stages.
+bool lay_out(const Shape& s, int bn, Config* c) {
+  const int stage = 2 * (s.seg * 128 + bn * 64);
+  const int xch = s.ks == 2 ? bn / 2 * 128 * 4 * (s.both ? 2 : 1) : 0;
+  int st = (kSmemMax - 1024 - kBarBytes) / stage;
+  if (st > kMaxStages) st = kMaxStages;
+  if (st < 3) return false;
+  // the products read 128 rows of an x box, whatever its height: the last one stays inside
+  int ring = st * stage;
+  const int last = (st - 1) * stage + s.seg * 128 + 16384;
+  if (last > ring) ring = last;
+  const int over = xch + 8 * 4096;  // exchange buffer and the drain warps' staging, over the ring
+  const int end = ((ring > over ? ring : over) + 15) / 16 * 16;
+  if (end + 1024 + kBarBytes > kSmemMax) return false;
+  c->bn = bn;
+  c->stages = st;
+  c->stg_off = xch;
+  c->bar_off = end;
+  c->smem = end + 1024 + kBarBytes;
+  return true;
+}
+
+// Clusters of 2 ks CTAs with this shared memory that the device holds at once.
+int resident_clusters(int dev, int ks, int smem) {
+  static std::mutex mu;
+  static std::vector<std::pair<long long, int>> cache;
+  const long long key = static_cast<long long>(dev) << 40 | static_cast<long long>(ks) << 32 | smem;
+  std::lock_guard<std::mutex> lock(mu);
+  for (auto& e : cache)
+    if (e.first == key) return e.second;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * ks * 128));
+  cfg.blockDim = dim3(smallm::NUM_THREADS);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(2 * ks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  if (cache.size() < 256) cache.emplace_back(key, n);
+  return n;
+}
+
+}  // namespace
+
+// Sizes alone decide, not streams or epilogue: the sums of one (M, K, N) have one order. Above
+// 128 rows the tile kernel of lora_gemm_tc.cu takes over where its 256-column tiles fill the chip
+// (measured on GB300, us, this kernel / that one; rows x K x N, two streams): 97 x 4096 x 4096
+// 13.0 / 30.4, x 12288 26.5 / 35.3, x 22016 51.1 / 80.3; 97 x 11008 x 4096 23.7 / 69.3;
+// 200 x 4096 x 11008 36.8 / 39.0, x 12288 46.9 / 44.9, x 16384 47.0 / 44.0; 300 x 4096 x 4096
+// 19.5 / 23.5 (shared input 16.0 / 24.0), x 12288 58.0 / 61.9, x 22016 110 / 103;
+// 384 x 4096 x 11008 49.2 / 57.1; 448 x 4096 x 4096 23.9 / 24.7, x 12288 81.8 / 63.0.
+bool small_gemm_wanted(int64_t M, int64_t K, int64_t N) {
+  if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
+  return M <= 128 || (M <= 256 && N <= 11264) || (M <= 384 && N <= 12288) || (M <= 448 && N <= 4096);
+}
+
+int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
+  using namespace smallm;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
+  static bool attr_set[64] = {false};
+  if (!attr_set[dev]) {
+    if (cudaFuncSetAttribute(lora_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmemMax) != cudaSuccess)
+      return -1;
+    attr_set[dev] = true;
+  }
+  const bool tri = a.x_crit != nullptr && !a.shared_x;
+  const int M = static_cast<int>(a.M), N = static_cast<int>(a.N);
+  const int kb = static_cast<int>((a.K + BK - 1) / BK);
+  const bool lora_on = a.r > 0 && a.u != nullptr && a.B != nullptr && a.y_on != nullptr;
+  const bool lora_crit = tri && a.r > 0 && a.u_crit != nullptr && a.B_crit != nullptr && a.y_crit != nullptr;
+  Shape s;
+  s.streams = a.shared_x ? 1 : (tri ? 3 : 2);
+  s.nseg = (M + 127) / 128;
+  // Split of K between the two pairs of a cluster where 256-column tiles of two streams leave
+  // half of the pairs idle: 36 clusters of four CTAs fit on the chip.
+  s.ks = a.epi != EPI_LOGSOFTMAX && s.nseg * ((N + 255) / 256) <= 36 && kb >= 8 ? 2 : 1;
+  if (s.streams == 1 && (s.nseg & 1)) ++s.nseg;
+  s.seg = ((M + s.nseg - 1) / s.nseg + 7) / 8 * 8;
+  s.row_tiles = (s.streams * s.nseg + 1) / 2;
+  s.lora = lora_on || lora_crit;
+  s.both = a.shared_x && lora_on && a.y_off != nullptr;
+  s.paired = a.epi == EPI_SWIGLU || a.epi == EPI_ROPE;
+  const int npair = a.epi == EPI_SWIGLU ? N / 2 : (N + 127) / 128 * 64;
+
+  // Tile width: the fewest clocks over the waves. A k-block of 64 costs the pair its products
+  // (2 bn) or a CTA's fill from L2 at 64 B per clock (2 (seg + bn / 2)), and a wave about 6000
+  // clocks of set-up, first loads and drain.
+  Config best{};
+  double best_t = 1e30;
+  auto tiles_of = [&](int bn) {
+    return s.row_tiles * (s.paired ? (npair + bn / 2 - 1) / (bn / 2) : (N + bn - 1) / bn);
+  };
+  for (int bn : {256, 224, 192, 160, 128, 96, 64}) {
+    if ((s.paired && bn % (64 * s.ks) != 0) || (s.ks == 2 && bn % 64 != 0)) continue;
+    if (a.epi == EPI_LOGSOFTMAX && bn != 256) continue;
+    Config c{};
+    if (!lay_out(s, bn, &c)) continue;
+    const int fit = resident_clusters(dev, s.ks, c.smem);
+    if (fit < 1) continue;
+    const int fill = 2 * (s.seg + bn / 2), mma = 2 * bn;
+    const double item = 2.0 * (fill > mma ? fill : mma);
+    const int waves = (tiles_of(bn) + fit - 1) / fit;
+    const double t = waves * (static_cast<double>((kb + s.ks - 1) / s.ks) * item + 6000.0);
+    if (t < best_t) {
+      best_t = t;
+      best = c;
+    }
+  }
+  if (best.bn == 0) return -4;
+  const int bn = best.bn;
+
+  Params p{};
+  p.b_box = s.paired ? gcd(bn / 2, a.epi == EPI_SWIGLU ? 128 : 64) : bn / 2;
+  Maps mp;
+  const void* xs[3] = {a.x_off, a.shared_x ? a.x_off : a.x_on, a.x_crit};
+  for (int i = 0; i < 3; ++i) {
+    if (i >= s.streams) mp.x[i] = mp.x[0];
+    else if (!make_tma_map(&mp.x[i], xs[i], a.M, a.K, a.K, s.seg, false)) return -2;
+  }
+  if (!make_tma_map(&mp.w, a.W, a.N, a.K, a.K, p.b_box, false)) return -2;
+  for (int i = 0; i < 2; ++i) {
+    if (i == 0 ? lora_on : lora_crit) {
+      if (!make_tma_map(&mp.u[i], i == 0 ? a.u : a.u_crit, a.M, a.r, a.r, s.seg, false)) return -2;
+      if (!make_tma_map(&mp.b[i], i == 0 ? a.B : a.B_crit, a.N, a.r, a.r, p.b_box, false)) return -2;
+    } else {  // never read
+      mp.u[i] = mp.x[0];
+      mp.b[i] = mp.w;
+    }
+  }
+  p.M = M;
+  p.N = N;
+  p.streams = s.streams;
+  p.nseg = s.nseg;
+  p.seg = s.seg;
+  p.row_tiles = s.row_tiles;
+  p.kb_main = kb;
+  p.kb_lora = s.lora ? static_cast<int>((a.r + BK - 1) / BK) : 0;
+  p.r = static_cast<int>(a.r);
+  p.bn = bn;
+  p.ks = s.ks;
+  p.stages = best.stages;
+  p.shared_x = a.shared_x ? 1 : 0;
+  p.both = s.both ? 1 : 0;
+  p.has_on = lora_on ? 1 : 0;
+  p.has_crit = lora_crit ? 1 : 0;
+  p.epi = a.epi;
+  p.out_f32 = a.out_f32;
+  p.paired = s.paired ? 1 : 0;
+  p.x_settled = a.x_settled ? 1 : 0;
+  p.lcol = pow2_at_least(bn);
+  p.tmem_cols = static_cast<uint32_t>(s.lora ? 2 * p.lcol : p.lcol);
+  p.stg_off = best.stg_off;
+  p.bar_off = best.bar_off;
+  p.y[0] = a.y_off;
+  p.y[1] = a.y_on;
+  p.y[2] = tri ? a.y_crit : nullptr;
+  p.rope_P = static_cast<int>(a.rope_P < 1 ? 1 : a.rope_P);
+  p.rope_cols = static_cast<int>(a.rope_cols);
+  p.rope_table = static_cast<const float2*>(a.rope_table);
+  p.lsm_target = a.lsm_target;
+  p.lsm_ids = a.lsm_ids;
+  p.lsm_L = static_cast<int>(a.lsm_L < 1 ? 1 : a.lsm_L);
+  p.lsm_ids_ld = static_cast<int>(a.lsm_ids_ld);
+  p.lsm_ids_off = static_cast<int>(a.lsm_ids_off);
+  p.lsm_tiles = (N + 255) / 256;
+  p.err = a.err;
+  const int tiles = tiles_of(bn);
+
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * s.ks), static_cast<unsigned>(s.row_tiles),
+                     static_cast<unsigned>(tiles / s.row_tiles));
+  cfg.blockDim = dim3(NUM_THREADS);
+  cfg.dynamicSmemBytes = static_cast<size_t>(best.smem);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(2 * s.ks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, lora_gemm_small_kernel, mp, p) == cudaSuccess ? 0 : -3;
+}
+
+}  // namespace hydra

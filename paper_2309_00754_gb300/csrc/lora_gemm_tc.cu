@@ -1000,6 +1000,13 @@ static int pick_tile_width(const GemmArgs& a, int nclusters) {
 
 int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   using namespace tcgemm;
+  // Few rows per stream take their own kernel. The log-softmax epilogue, whose tiles are 256
+  // columns wide, does where a pair then holds both streams (32000 columns, 100 rows: 69.9 us
+  // against 70.2, with LoRA 70.6 against 75.2); one shared input fills this file's single-CTA
+  // tiles just as well (57.4 us against 73.8).
+  const bool lsm_ok = a.epi != EPI_LOGSOFTMAX || (!a.shared_x && a.M <= BM);
+  if (!a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N))
+    return launch_dual_lora_gemm_small(a, stream);
   static bool attr_set = false;
   if (!attr_set) {
     if (cudaFuncSetAttribute(dual_lora_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -51,8 +51,8 @@ __global__ void __launch_bounds__(32 * kDownWarps)
                      __nv_bfloat16* __restrict__ u, int ck) {
   __shared__ float red[kDownWarps][16][NT * 8 + 1];
   __shared__ float tile[16][NT * 8];  // this CTA's sum over its warps
-  pdl_launch_dependents();
   pdl_wait();  // x is written by the preceding kernel
+  pdl_launch_dependents();  // after the wait: a dependent may take x as final
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, c = lane & 3;
@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(kThreads)
   // first half of a cluster barrier: its wait, before the first store to another CTA's shared
   // memory, ensures every CTA of the cluster has started
   if (ck > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  pdl_launch_dependents();
   pdl_wait();  // x is written by the preceding kernel, which may also still read u
+  pdl_launch_dependents();  // after the wait: a dependent may take x as final
 
   float d[4][NT][4];
 #pragma unroll

@@ -147,6 +147,7 @@ int stacked_linear_impl(int prof_class, const void* x, int64_t T, int64_t K, int
   g.out_f32 = f32 ? 1 : 0;
   g.err = err;
   g.epi = epi;
+  g.x_settled = r > 0;
   if (rope != nullptr) {
     g.rope_P = rope->P;
     g.rope_cols = rope->cols;
@@ -393,6 +394,7 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
       g.y_on = static_cast<uint8_t*>(qkv) + static_cast<size_t>(T) * 3 * d * 2;
       g.out_f32 = 0;
       g.err = err;
+      g.x_settled = true;
       g.epi = hydra::kStackEpiRope;
       g.rope_P = P;
       g.rope_cols = 2 * d;

@@ -1,0 +1,116 @@
+"""The linear of few token rows per stream (lora_gemm_small.cu) at the edges of its segments,
+tiles, K items and K slices, against the oracle; and its one order of summation: the shared,
+stacked and three-stream forms, the fused epilogues and the separate ones agree bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from tests.helpers import TOL_LINEAR, O, assert_rel, dev_bf16, dev_f32, f64, host_f64, synth
+from paper_2309_00754_gb300 import hydra as H
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(M, K, N, r, seed):
+    g = lambda i, shape, std: synth.normal_bf16(1000 * seed + i, shape, std)  # noqa: E731
+    x = [g(i, (M, K), 1.0) for i in range(3)]
+    ab = [(g(10 + i, (r, K), 0.02), g(20 + i, (N, r), 0.02)) for i in range(2)] if r else [(None, None)] * 2
+    return x, g(3, (N, K), 0.02), ab
+
+
+def _dev(t):
+    return None if t is None else dev_bf16(t)
+
+
+@pytest.mark.parametrize("M,K,N,r,f32", [
+    (1, 8, 8, 0, False),          # one row, one column chunk, one partial k-block
+    (5, 136, 264, 8, True),       # an empty second segment; N and K tails
+    (64, 1024, 520, 16, False),   # two K slices of four items each
+    (65, 1160, 1032, 136, True),  # two LoRA items, the second of one k-block
+    (128, 2048, 4104, 72, False),  # the largest single segment, a tail tile of one chunk
+    (129, 1032, 4104, 72, True),  # two segments per stream, two slices (34 256-column tiles)
+    (257, 520, 1288, 8, False),   # three segments per stream: a pair of the off and the on stream
+    (384, 264, 12288, 16, False),  # the largest, more tiles than the chip holds at once
+    (448, 200, 520, 8, True),
+])
+def test_few_rows_against_oracle_and_one_order_of_sums(M, K, N, r, f32):
+    x, W, ab = _problem(M, K, N, r, seed=M + K)
+    dt = torch.float32 if f32 else torch.bfloat16
+    d, dW = [dev_bf16(t) for t in x], dev_bf16(W)
+    dab = [(_dev(a), _dev(b)) for a, b in ab]
+    new = lambda: torch.full((M, N), float("nan"), dtype=dt, device="cuda")  # noqa: E731
+    ws = torch.empty(max(1, H.lora_linear_tri_workspace_size(M, r)), dtype=torch.uint8, device="cuda")
+
+    def two(xa, xb, a, b, want=(True, True)):
+        y = [new() if w else None for w in want]
+        H.hydra_lora_linear(xa, xb, dW, a, b, 2.0, y[0], y[1], ws, algo=1)
+        return y
+
+    tri = [new() for _ in range(3)]
+    H.hydra_lora_linear_tri(d[0], d[1], d[2], dW, *dab[0], *dab[1], 2.0, *tri, ws)
+    st = two(d[0], d[1], *dab[0])
+    sh = two(d[1], None, *dab[0])
+    crit = two(d[2], None, *dab[1], want=(False, True))
+    off = two(d[0], None, *dab[0], want=(True, False))
+    assert torch.equal(tri[0], st[0]) and torch.equal(tri[1], st[1])
+    assert torch.equal(st[1], sh[1]) and torch.equal(tri[2], crit[1]) and torch.equal(off[0], st[0])
+    # against fp64, fp32 sums of bf16 products in another order: 1e-4 as for the tile kernel's fp32
+    # outputs. u is the library's own (hydra_lora_down, tested by itself): where it rounds to bf16
+    # the other way than the oracle's, y moves by ulp(u) |B|, up to 2^-6 * 0.1 = 1.6e-3
+    tol = 1e-4 if f32 else TOL_LINEAR
+    for y, i, (a, b) in ((tri[0], 0, (None, None)), (tri[1], 1, dab[0]), (tri[2], 2, dab[1])):
+        ref = f64(x[i]) @ f64(W).T
+        if a is not None:
+            u = torch.empty(M, r, dtype=torch.bfloat16, device="cuda")
+            H.hydra_lora_down(d[i], a, 2.0, u)
+            ref += host_f64(u) @ host_f64(b).T
+        assert_rel(host_f64(y), ref if f32 else O.round_bf16(ref), tol, f"stream {i}")
+
+
+@pytest.mark.parametrize("M,N,shared", [(33, 512, False), (97, 512, True), (128, 768, False), (200, 392, False),
+                                        (300, 392, True)])
+def test_few_rows_fused_epilogues(M, N, shared):
+    """SwiGLU, rotary (N past the rotated columns, a partial last head) and residual epilogues
+    equal the plain linear followed by the separate kernel, bit for bit (two K slices)."""
+    K, r, P = 1032, 16, 50
+    x, W, ab = _problem(M, K, N, r, seed=7 * M + N)
+    d, dW, dB = [dev_bf16(t) for t in x], dev_bf16(W), dev_bf16(ab[0][1])
+    xo = None if shared else d[1]
+    u = dev_bf16(synth.normal_bf16(99, (M, r), 2.0))
+    lin = [torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    H.hydra_dual_linear(d[0], xo, dW, u, dB, lin[0], lin[1], algo=1)
+    h0 = synth.normal_f32(98, (2, M, N), 3.0)
+    h, want = dev_f32(h0), dev_f32(h0)
+    H.hydra_dual_linear_ex(d[0], xo, dW, u, dB, h[0], h[1], H.EPI_RESIDUAL)
+    for i in range(2):
+        H.hydra_residual_add(want[i].view(-1), lin[i].view(-1))
+    assert torch.equal(h, want)
+    d_rot = 128
+    got = [torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    table = torch.empty(P, 64, 2, device="cuda")
+    H.hydra_rope_table(P, 128, 10000.0, table)
+    H.hydra_dual_linear_rope(d[0], xo, dW, u, dB, got[0], got[1], P, 2 * d_rot, 128, table)
+    if N % 256 == 0:  # W rows as interleaved gate / up blocks of 128
+        m = [torch.empty(M, N // 2, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        H.hydra_dual_linear_ex(d[0], xo, dW, u, dB, m[0], m[1], H.EPI_SWIGLU)
+        for i in range(2):
+            gu = lin[i].view(M, N // 256, 2, 128).transpose(1, 2).reshape(M, N).contiguous()
+            ref = torch.empty_like(m[i])
+            H.hydra_swiglu(gu, ref)
+            assert torch.equal(m[i], ref)
+    for i in range(2):
+        H.hydra_rope(lin[i], d_rot, 128, P, 10000.0)
+        assert torch.equal(got[i], lin[i])
+    assert H.device_error(clear=True) == 0
+
+
+def test_off_rows_ignore_a_non_finite_lora_factor():
+    """A pair of an off and an on segment: infinities in B reach the LoRA-on rows alone."""
+    M, K, N, r = 40, 256, 264, 16
+    x, W, ab = _problem(M, K, N, r, seed=5)
+    d, dW = [dev_bf16(t) for t in x], dev_bf16(W)
+    A, B = dev_bf16(ab[0][0]), torch.full((N, r), float("inf"), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(H.lora_linear_workspace_size(M, r), dtype=torch.uint8, device="cuda")
+    y = [torch.empty(M, N, device="cuda") for _ in range(2)]
+    H.hydra_lora_linear(d[0], d[1], dW, A, B, 2.0, y[0], y[1], ws)
+    assert np.all(np.isfinite(host_f64(y[0]))) and not bool(torch.isfinite(y[1]).any())
