@@ -7,17 +7,24 @@
 //   loss_clip  = -(1/n) sum s_t,   d/d logp_new_t = -r_t A_t / n where r_t A_t <= clip term
 //   loss_value =  (1/n) sum (V_t - R_t)^2,   d/d V_t = 2 (V_t - R_t) / n
 //
-// Up to four launches, chained with programmatic dependent launch:
+// Batches of up to kSmallTokens tokens run in one launch: a thread-block cluster that takes the
+// moments, meets over distributed shared memory, runs the loss pass, meets again and writes the
+// statistics. (Four chained launches cost 10 us of device time for 2048 tokens and their
+// enqueueing more; the one launch 4-5 us.)
+//
+// Larger ones take two launches, the second a programmatic dependent launch:
 //   moments:  per block, the valid count n and (with whitening) the sums of a - c and
 //             (a - c)^2 over the valid advantages, c = adv[0] a common shift;
-//   coef:     one block merges those partials (or takes the caller's moments) into
-//             (mean, 1 / std, 1 / n);
-//   loss:     streams float4 chunks of the flattened [S, L] batch, several chunks' loads
-//             in flight per thread; chunks past a row's length are written as zero
-//             gradients without reading the inputs; per-block sums go to the workspace;
-//   finalize: one block merges the per-block sums, in a fixed order, and writes the
-//             statistics.
+//   loss:     every block merges those partials (or takes the caller's moments) into
+//             (mean, 1 / std, 1 / n), all in the same order, while its first loads are in
+//             flight; streams float4 chunks of the flattened [S, L] batch; chunks without a
+//             valid token are written as zero gradients without reading the inputs; per-block
+//             sums go to the workspace, and the block that finishes last merges them, in a
+//             fixed order, into the statistics. (A launch of its own for either merge cost
+//             2.2 and 3.1 us of the 34 us that 16384 x 400 tokens took.)
 // Every grid is one wave (SMs x resident blocks), so no block waits for a second wave.
+// A chunk is four consecutive tokens of the flattened batch and may straddle two rows, so row
+// lengths that are not multiples of four take the same 16-byte loads.
 // Per-thread sums are compensated (Kahan) fp32, block and cross-block trees fp32: GB300
 // executes fp64 at a small fraction of its fp32 rate, so fp64 appears only in a few scalar
 // operations of the output.
@@ -118,10 +125,9 @@ __device__ __forceinline__ int row_length(const int32_t* lengths, int s, int L, 
   return clamp_length(lengths ? __ldg(lengths + s) : L, L, err);
 }
 
-// A thread's position in the flattened batch: row s, chunk column t (chunk q = s C + t),
-// and row s's length, fetched one batch ahead so that its latency overlaps the previous
-// batch's data loads. Advancing by a fixed number of chunks steps rows and columns without
-// a division.
+// A thread's position in the flattened batch: token e = s L + t of row s, and that row's length,
+// fetched one chunk ahead so that its latency overlaps the previous chunk's data loads. Advancing
+// by a fixed number of tokens steps rows and columns without a division.
 struct Cursor {
   int s, t, len;
 };
@@ -130,21 +136,37 @@ __device__ __forceinline__ int fetch_length(const int32_t* lengths, int s, int S
   return s < S ? (lengths ? __ldg(lengths + s) : L) : 0;
 }
 
-__device__ __forceinline__ Cursor cursor_at(unsigned q, int C, const int32_t* lengths, int S,
-                                            int L) {
-  const int s = static_cast<int>(q / static_cast<unsigned>(C));
-  return Cursor{s, static_cast<int>(q - static_cast<unsigned>(s) * C), fetch_length(lengths, s, S, L)};
+__device__ __forceinline__ Cursor cursor_at(unsigned e, int L, const int32_t* lengths, int S) {
+  const int s = static_cast<int>(e / static_cast<unsigned>(L));
+  return Cursor{s, static_cast<int>(e - static_cast<unsigned>(s) * L), fetch_length(lengths, s, S, L)};
 }
 
-__device__ __forceinline__ void cursor_advance(Cursor& c, int ds, int dt, int C,
-                                               const int32_t* lengths, int S, int L) {
+// ds, dt: rows and columns of the step
+__device__ __forceinline__ void cursor_advance(Cursor& c, int ds, int dt, const int32_t* lengths, int S,
+                                               int L) {
   c.t += dt;
   c.s += ds;
-  if (c.t >= C) {
-    c.t -= C;
+  if (c.t >= L) {
+    c.t -= L;
     ++c.s;
   }
   c.len = fetch_length(lengths, c.s, S, L);
+}
+
+// Valid tokens of the VEC-token chunk at the cursor, one bit each (VEC <= L: at most two rows).
+// ODD: rows are not whole chunks, so a chunk may straddle two rows or the end of the batch
+// (16384 x 400 tokens: the loss pass 26.3 us without that code, 27.1 with it).
+template <int VEC, bool ODD>
+__device__ __forceinline__ int chunk_mask(const Cursor& c, const int32_t* lengths, int S, int L, int* err) {
+  const int len = clamp_length(c.len, L, err);
+  const int k = min(max(len - c.t, 0), VEC);
+  int m = (1 << k) - 1;
+  const int in_row = L - c.t;  // tokens of the chunk in this row
+  if (ODD && in_row < VEC && c.s + 1 < S) {
+    const int len2 = row_length(lengths, c.s + 1, L, err);
+    m |= ((1 << min(len2, VEC - in_row)) - 1) << in_row;
+  }
+  return m;
 }
 
 template <int VEC>
@@ -165,6 +187,27 @@ struct Vec<1> {
   static __device__ __forceinline__ void put(float* p, const float* v) { __stcs(p, v[0]); }
 };
 
+// Chunk at element offset `off`; `n` < VEC elements at the end of the batch are moved one by one.
+template <int VEC, bool ODD>
+__device__ __forceinline__ void chunk_get(const float* p, unsigned off, int n, float* v) {
+  if (!ODD || n >= VEC) {
+    Vec<VEC>::get(p + off, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) v[j] = j < n ? __ldcs(p + off + j) : 0.f;
+  }
+}
+template <int VEC, bool ODD>
+__device__ __forceinline__ void chunk_put(float* p, unsigned off, int n, const float* v) {
+  if (!ODD || n >= VEC) {
+    Vec<VEC>::put(p + off, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < VEC; ++j)
+      if (j < n) __stcs(p + off + j, v[j]);
+  }
+}
+
 // Loads that keep their lines in L2 (normal eviction priority): the moments pass reads the
 // advantages this way, so that the loss pass, which reads them again with the rest of its
 // inputs streaming (evict-first), finds them there when the batch fits in L2.
@@ -178,92 +221,72 @@ __device__ __forceinline__ void get_keep(const float* p, float* v) {
   }
 }
 
-// Pass 1: valid count and shifted advantage sums per block. Chunk q of the flattened batch
-// covers tokens [VEC (q mod C), +VEC) of row q / C, C = L / VEC. Each thread holds two
-// batches of kMomBatch chunks: the next batch's loads are issued before the current one is
-// added, so that two batches per thread are in flight.
+// Shifted advantage sums and valid count of the chunks e = VEC (first + i step), i = 0, 1, ..., in
+// batches of kMomBatch chunks whose loads are issued together.
 constexpr int kMomBatch = 4;
 
-template <int VEC>
-struct MomBatch {
-  float v[kMomBatch][VEC];
-  int k[kMomBatch];  // valid tokens of each chunk
-};
-
-template <int VEC>
-__device__ __forceinline__ void mom_load(MomBatch<VEC>& x, Cursor (&cur)[kMomBatch],
-                                         const float* adv, int S, int L, int C, int ds, int dt,
-                                         const int32_t* lengths, int* err) {
+template <int VEC, bool ODD>
+__device__ __forceinline__ void moments_walk(const float* __restrict__ adv, const int32_t* lengths, int S,
+                                             int L, unsigned first, unsigned nthr, float c, int& n,
+                                             Kahan& s1, Kahan& s2, int* err) {
+  const unsigned E = static_cast<unsigned>(S) * static_cast<unsigned>(L);
+  const unsigned step = kMomBatch * nthr * VEC;  // tokens per batch over the grid
+  const int ds = static_cast<int>(step / L), dt = static_cast<int>(step % L);
+  Cursor cur[kMomBatch];
 #pragma unroll
-  for (int b = 0; b < kMomBatch; ++b) {
-    x.k[b] = 0;
-    if (cur[b].s < S) {
-      const int t0 = cur[b].t * VEC;
-      const int len = clamp_length(cur[b].len, L, t0 == 0 ? err : nullptr);
-      x.k[b] = min(max(len - t0, 0), VEC);
-      if (x.k[b] > 0) get_keep<VEC>(adv + static_cast<size_t>(cur[b].s) * L + t0, x.v[b]);
+  for (int b = 0; b < kMomBatch; ++b) cur[b] = cursor_at((first + b * nthr) * VEC, L, lengths, S);
+  while (cur[0].s < S) {
+    float v[kMomBatch][VEC];
+    int m[kMomBatch];
+#pragma unroll
+    for (int b = 0; b < kMomBatch; ++b) {
+      m[b] = 0;
+      if (cur[b].s < S) {
+        m[b] = chunk_mask<VEC, ODD>(cur[b], lengths, S, L, err);
+        const unsigned off = static_cast<unsigned>(cur[b].s) * static_cast<unsigned>(L) + cur[b].t;
+        if (m[b] != 0) {
+          if (!ODD || E - off >= VEC) get_keep<VEC>(adv + off, v[b]);
+          else chunk_get<VEC, ODD>(adv, off, static_cast<int>(E - off), v[b]);
+        }
+      }
     }
+#pragma unroll
+    for (int b = 0; b < kMomBatch; ++b) cursor_advance(cur[b], ds, dt, lengths, S, L);
+    float b1 = 0.f, b2 = 0.f;  // this batch's sums, then one compensated add each
+#pragma unroll
+    for (int b = 0; b < kMomBatch; ++b)
+#pragma unroll
+      for (int j = 0; j < VEC; ++j) {
+        const float d = (m[b] >> j) & 1 ? v[b][j] - c : 0.f;
+        b1 += d;
+        b2 += d * d;
+      }
+#pragma unroll
+    for (int b = 0; b < kMomBatch; ++b) n += __popc(m[b]);
+    s1.add(b1);
+    s2.add(b2);
   }
-#pragma unroll
-  for (int b = 0; b < kMomBatch; ++b) cursor_advance(cur[b], ds, dt, C, lengths, S, L);
 }
 
-template <int VEC>
-__device__ __forceinline__ void mom_add(const MomBatch<VEC>& x, float c, int& n, Kahan& s1,
-                                        Kahan& s2) {
-  float b1 = 0.f, b2 = 0.f;  // this batch's sums, then one compensated add each
-#pragma unroll
-  for (int b = 0; b < kMomBatch; ++b)
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) {
-      const float d = j < x.k[b] ? x.v[b][j] - c : 0.f;
-      b1 += d;
-      b2 += d * d;
-    }
-#pragma unroll
-  for (int b = 0; b < kMomBatch; ++b) n += x.k[b];
-  s1.add(b1);
-  s2.add(b2);
-}
-
-template <int VEC>
+// Pass 1: valid count and shifted advantage sums per block. `ticket` (the loss pass's block
+// counter) is cleared for the launch that follows.
+template <int VEC, bool ODD>
 __global__ void __launch_bounds__(kPpoThreads, 3)
     ppo_moments_kernel(const float* __restrict__ adv, const int32_t* __restrict__ lengths, int S,
-                       int L, int with_adv, MomPart* __restrict__ part, int* err) {
+                       int L, int with_adv, MomPart* __restrict__ part, unsigned* ticket, int* err) {
   __shared__ float sh[2][kPpoWarps];
   __shared__ int shk[kPpoWarps];
   pdl_wait();
   const unsigned tid = blockIdx.x * kPpoThreads + threadIdx.x;
   const unsigned nthr = gridDim.x * kPpoThreads;
+  if (tid == 0 && ticket != nullptr) *ticket = 0;
   int n = 0;
   Kahan s1, s2;
   if (!with_adv) {
     for (unsigned s = tid; s < static_cast<unsigned>(S); s += nthr)
       n += row_length(lengths, static_cast<int>(s), L, err);
-  } else if (L >= VEC) {  // C = L / VEC >= 1: the cursors divide by C
-    const float c = S > 0 ? __ldg(adv) : 0.f;
-    const int C = L / VEC;
-    const unsigned step = kMomBatch * nthr;  // chunks per batch over the grid
-    const int ds = static_cast<int>(step / C), dt = static_cast<int>(step % C);
-    Cursor cur[kMomBatch];
-#pragma unroll
-    for (int b = 0; b < kMomBatch; ++b) cur[b] = cursor_at(tid + b * nthr, C, lengths, S, L);
-    MomBatch<VEC> x, y;
-    mom_load(x, cur, adv, S, L, C, ds, dt, lengths, err);
-    while (true) {
-      if (cur[0].s >= S) {
-        mom_add(x, c, n, s1, s2);
-        break;
-      }
-      mom_load(y, cur, adv, S, L, C, ds, dt, lengths, err);
-      mom_add(x, c, n, s1, s2);
-      if (cur[0].s >= S) {
-        mom_add(y, c, n, s1, s2);
-        break;
-      }
-      mom_load(x, cur, adv, S, L, C, ds, dt, lengths, err);
-      mom_add(y, c, n, s1, s2);
-    }
+  } else if (L >= VEC) {
+    moments_walk<VEC, ODD>(adv, lengths, S, L, tid, nthr, S > 0 ? __ldg(adv) : 0.f, n, s1, s2, err);
   }
   float v[2] = {s1.s, s2.s};
   block_sums<2>(v, n, sh, shk);
@@ -277,10 +300,11 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
 // length are never read.
 __global__ void __launch_bounds__(kPpoThreads)
     ppo_moments_rows_kernel(const float* __restrict__ adv, const int32_t* __restrict__ lengths,
-                            int S, int L, MomPart* __restrict__ part, int* err) {
+                            int S, int L, MomPart* __restrict__ part, unsigned* ticket, int* err) {
   __shared__ float sh[2][kPpoWarps];
   __shared__ int shk[kPpoWarps];
   pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && ticket != nullptr) *ticket = 0;
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kPpoWarps + (threadIdx.x >> 5);
   const int nw = gridDim.x * kPpoWarps;
@@ -331,62 +355,80 @@ __global__ void __launch_bounds__(kPpoThreads)
   pdl_launch_dependents();
 }
 
-// Merge the moments partials (or take the caller's fp64 [n, mean, M2]) into the fp64
-// moments and the fp32 coefficients (mean, 1 / sqrt(var + 1e-8), 1 / n) of the loss pass.
-// Every thread loads its few partials at once (compensated fp32), then a fixed block tree.
+// (n, mean, M2) and the coefficients of the loss pass
+struct Moments {
+  double n, mean, m2;
+  float c_mean, inv_std, inv_n;
+};
+
+__device__ __forceinline__ Moments moments_from_ext(const double* ext) {
+  Moments m;
+  m.n = __ldcg(ext);
+  m.mean = __ldcg(ext + 1);
+  m.m2 = __ldcg(ext + 2);
+  const double var = m.n > 0.0 ? m.m2 / m.n : 0.0;
+  m.c_mean = static_cast<float>(m.mean);
+  m.inv_std = static_cast<float>(1.0 / sqrt(var + 1e-8));
+  m.inv_n = m.n > 0.0 ? static_cast<float>(1.0 / m.n) : 0.f;
+  return m;
+}
+
+// from the sums of a - c and (a - c)^2 over n tokens
+__device__ __forceinline__ Moments moments_from_sums(int n, float s1, float s2, float c) {
+  Moments m;
+  float mean = 0.f, m2 = 0.f;
+  if (n > 0) {
+    const float d1 = s1 / static_cast<float>(n);
+    mean = c + d1;
+    m2 = fmaxf(s2 - d1 * s1, 0.f);
+  }
+  const float var = n > 0 ? m2 / static_cast<float>(n) : 0.f;
+  m.n = static_cast<double>(n);
+  m.mean = static_cast<double>(mean);
+  m.m2 = static_cast<double>(m2);
+  m.c_mean = mean;
+  m.inv_std = rsqrtf(var + 1e-8f);
+  m.inv_n = n > 0 ? 1.f / static_cast<float>(n) : 0.f;
+  return m;
+}
+
+// Merge the G moments partials: every thread loads its few at once (compensated fp32), then a
+// fixed block tree. The result is valid in every thread.
 constexpr int kMaxPartsPerThread = (kPpoMaxLossBlocks + kPpoThreads - 1) / kPpoThreads;
 
+__device__ __forceinline__ Moments merge_moments(const MomPart* part, int G, float c,
+                                                 float (*sh)[kPpoWarps], int* shk) {
+  MomPart p[kMaxPartsPerThread];
+#pragma unroll
+  for (int i = 0; i < kMaxPartsPerThread; ++i) {
+    const int j = threadIdx.x + i * kPpoThreads;
+    p[i] = j < G ? load_part(part + j) : MomPart{0, 0.f, 0.f, 0.f};
+  }
+  int n = 0;
+  Kahan k1, k2;
+#pragma unroll
+  for (int i = 0; i < kMaxPartsPerThread; ++i) {
+    n += p[i].n;
+    k1.add(p[i].s1);
+    k2.add(p[i].s2);
+  }
+  float v[2] = {k1.s, k2.s};
+  block_sums<2>(v, n, sh, shk);
+  return moments_from_sums(n, v[0], v[1], c);
+}
+
+// The moments alone (hydra_ppo_adv_moments): one block.
 __global__ void __launch_bounds__(kPpoThreads)
-    ppo_coef_kernel(const float* __restrict__ adv, int S, int L, int shifted,
-                    const MomPart* __restrict__ part, int G, const double* __restrict__ ext,
-                    double* __restrict__ moments, float* __restrict__ coef) {
+    ppo_merge_kernel(const float* __restrict__ adv, int S, int L, const MomPart* __restrict__ part, int G,
+                     double* __restrict__ moments) {
   __shared__ float sh[2][kPpoWarps];
   __shared__ int shk[kPpoWarps];
   pdl_wait();
-  if (ext != nullptr) {
-    if (threadIdx.x == 0) {
-      const double n = __ldcg(ext), mean = __ldcg(ext + 1), m2 = __ldcg(ext + 2);
-      moments[0] = n;
-      moments[1] = mean;
-      moments[2] = m2;
-      const double var = n > 0.0 ? m2 / n : 0.0;
-      coef[0] = static_cast<float>(mean);
-      coef[1] = static_cast<float>(1.0 / sqrt(var + 1e-8));
-      coef[2] = n > 0.0 ? static_cast<float>(1.0 / n) : 0.f;
-    }
-  } else {
-    MomPart p[kMaxPartsPerThread];
-#pragma unroll
-    for (int i = 0; i < kMaxPartsPerThread; ++i) {
-      const int j = threadIdx.x + i * kPpoThreads;
-      p[i] = j < G ? load_part(part + j) : MomPart{0, 0.f, 0.f, 0.f};
-    }
-    int n = 0;
-    Kahan k1, k2;
-#pragma unroll
-    for (int i = 0; i < kMaxPartsPerThread; ++i) {
-      n += p[i].n;
-      k1.add(p[i].s1);
-      k2.add(p[i].s2);
-    }
-    float v[2] = {k1.s, k2.s};
-    block_sums<2>(v, n, sh, shk);
-    if (threadIdx.x == 0) {
-      float mean = 0.f, m2 = 0.f;
-      if (n > 0) {
-        const float c = shifted && S > 0 && L > 0 ? __ldg(adv) : 0.f;
-        const float d1 = v[0] / static_cast<float>(n);
-        mean = c + d1;
-        m2 = fmaxf(v[1] - d1 * v[0], 0.f);
-      }
-      const float var = n > 0 ? m2 / static_cast<float>(n) : 0.f;
-      moments[0] = static_cast<double>(n);
-      moments[1] = static_cast<double>(mean);
-      moments[2] = static_cast<double>(m2);
-      coef[0] = mean;
-      coef[1] = rsqrtf(var + 1e-8f);
-      coef[2] = n > 0 ? 1.f / static_cast<float>(n) : 0.f;
-    }
+  const Moments m = merge_moments(part, G, G > 0 && S > 0 && L > 0 ? __ldg(adv) : 0.f, sh, shk);
+  if (threadIdx.x == 0) {
+    moments[0] = m.n;
+    moments[1] = m.mean;
+    moments[2] = m.m2;
   }
   pdl_launch_dependents();
 }
@@ -396,7 +438,8 @@ __global__ void __launch_bounds__(kPpoThreads)
 template <int VEC>
 struct LossChunk {
   float ln[VEC], lo[VEC], a[VEC], R[VEC], V[VEC];
-  int k;         // valid tokens; -1: past the end of the batch
+  int mask;      // valid tokens
+  int left;      // tokens of the batch from the chunk's first on, at most VEC; 0: past its end
   unsigned off;  // element offset (S * L < 2^31)
 };
 
@@ -405,42 +448,43 @@ struct LossAcc {
   int nclip = 0;
 };
 
-template <int VEC>
+template <int VEC, bool ODD>
 __device__ __forceinline__ void loss_load(LossChunk<VEC>& x, Cursor& cur, const float* logp_new,
                                           const float* logp_old, const float* adv,
                                           const float* ret, const float* val, int S, int L,
-                                          int C, int ds, int dt, const int32_t* lengths,
-                                          int* err) {
-  x.k = -1;
+                                          int ds, int dt, const int32_t* lengths, int* err) {
+  x.mask = 0;
+  x.left = 0;
   x.off = 0;
   if (cur.s < S) {
-    const int t0 = cur.t * VEC;
-    const int len = clamp_length(cur.len, L, t0 == 0 ? err : nullptr);
-    x.k = min(max(len - t0, 0), VEC);
-    x.off = static_cast<unsigned>(cur.s) * static_cast<unsigned>(L) + t0;
-    if (x.k > 0) {
-      Vec<VEC>::get(logp_new + x.off, x.ln);
-      Vec<VEC>::get(logp_old + x.off, x.lo);
-      Vec<VEC>::get(adv + x.off, x.a);
-      Vec<VEC>::get(ret + x.off, x.R);
-      Vec<VEC>::get(val + x.off, x.V);
+    x.mask = chunk_mask<VEC, ODD>(cur, lengths, S, L, err);
+    x.off = static_cast<unsigned>(cur.s) * static_cast<unsigned>(L) + cur.t;
+    x.left = VEC;
+    if (ODD) x.left = static_cast<int>(min(static_cast<unsigned>(S) * static_cast<unsigned>(L) - x.off,
+                                           static_cast<unsigned>(VEC)));
+    if (x.mask != 0) {
+      chunk_get<VEC, ODD>(logp_new, x.off, x.left, x.ln);
+      chunk_get<VEC, ODD>(logp_old, x.off, x.left, x.lo);
+      chunk_get<VEC, ODD>(adv, x.off, x.left, x.a);
+      chunk_get<VEC, ODD>(ret, x.off, x.left, x.R);
+      chunk_get<VEC, ODD>(val, x.off, x.left, x.V);
     }
   }
-  cursor_advance(cur, ds, dt, C, lengths, S, L);
+  cursor_advance(cur, ds, dt, lengths, S, L);
 }
 
-template <int VEC, bool WHITEN>
+template <int VEC, bool ODD, bool WHITEN>
 __device__ __forceinline__ void loss_compute(const LossChunk<VEC>& x, float mean, float inv_std,
                                              float inv_n, float eps, LossAcc& acc,
                                              float* grad_logp, float* grad_val) {
-  if (x.k < 0) return;
+  if (x.left == 0) return;
   const float lo_clip = 1.f - eps, hi_clip = 1.f + eps;
   float gl[VEC], gv[VEC];
   float bs = 0.f, bv = 0.f, bkl = 0.f, ba = 0.f, baa = 0.f;  // this chunk's sums
 #pragma unroll
   for (int j = 0; j < VEC; ++j) {
     gl[j] = gv[j] = 0.f;
-    if (j < x.k) {
+    if ((x.mask >> j) & 1) {
       const float d = x.ln[j] - x.lo[j];
       const float r = expf(d);
       const float A = WHITEN ? (x.a[j] - mean) * inv_std : x.a[j];
@@ -457,9 +501,9 @@ __device__ __forceinline__ void loss_compute(const LossChunk<VEC>& x, float mean
       gv[j] = 2.f * dv * inv_n;
     }
   }
-  Vec<VEC>::put(grad_logp + x.off, gl);
-  Vec<VEC>::put(grad_val + x.off, gv);
-  if (x.k > 0) {
+  chunk_put<VEC, ODD>(grad_logp, x.off, x.left, gl);
+  chunk_put<VEC, ODD>(grad_val, x.off, x.left, gv);
+  if (x.mask != 0) {
     acc.s.add(bs);
     acc.v.add(bv);
     acc.kl.add(bkl);
@@ -468,40 +512,64 @@ __device__ __forceinline__ void loss_compute(const LossChunk<VEC>& x, float mean
   }
 }
 
-template <int VEC, bool WHITEN>
+// The statistics of a batch from its loss sums.
+__device__ __forceinline__ void write_stats(double* stats, const float (&v)[kLossSums], int nclip,
+                                            const Moments& m, bool report_moments) {
+  const double n = m.n, inv = n > 0.0 ? 1.0 / n : 0.0;
+  stats[0] = -static_cast<double>(v[0]) * inv;
+  stats[1] = static_cast<double>(v[1]) * inv;
+  stats[2] = static_cast<double>(nclip) * inv;
+  stats[3] = static_cast<double>(v[2]) * inv;
+  if (report_moments) {
+    stats[4] = m.mean;
+    stats[5] = n > 0.0 ? sqrt(m.m2 * inv) : 0.0;
+  } else {
+    const double a = static_cast<double>(v[3]) * inv;
+    stats[4] = a;
+    stats[5] = n > 0.0 ? sqrt(fmax(static_cast<double>(v[4]) * inv - a * a, 0.0)) : 0.0;
+  }
+  stats[6] = n;
+}
+
+// Pass 2 over the grid, and the statistics by the block that finishes last.
+template <int VEC, bool ODD, bool WHITEN>
 __global__ void __launch_bounds__(kPpoThreads, 3)
     ppo_loss_kernel(const float* __restrict__ logp_new, const float* __restrict__ logp_old,
                     const float* __restrict__ adv, const float* __restrict__ ret,
                     const float* __restrict__ val, const int32_t* __restrict__ lengths, int S,
-                    int L, float eps, const float* __restrict__ coef,
-                    LossPart* __restrict__ lpart, float* __restrict__ grad_logp,
-                    float* __restrict__ grad_val, int* err) {
+                    int L, float eps, const MomPart* __restrict__ mpart, int Gm,
+                    const double* __restrict__ ext, int report_moments, LossPart* __restrict__ lpart,
+                    unsigned* ticket, float* __restrict__ grad_logp, float* __restrict__ grad_val,
+                    double* __restrict__ stats, int* err) {
   __shared__ float sh[kLossSums][kPpoWarps];
   __shared__ int shk[kPpoWarps];
+  __shared__ bool last;
   pdl_wait();
-  const float mean = __ldcg(coef), inv_std = __ldcg(coef + 1), inv_n = __ldcg(coef + 2);
   const unsigned tid = blockIdx.x * kPpoThreads + threadIdx.x;
   const unsigned nthr = gridDim.x * kPpoThreads;
-  // C >= 1 here: the host launches this pass only for S * L > 0 with L % VEC == 0
-  const int C = L / VEC;
-  const int ds = static_cast<int>(nthr / C), dt = static_cast<int>(nthr % C);
-  Cursor cur = cursor_at(tid, C, lengths, S, L);
+  // L >= VEC here: the host launches this pass only for S * L > 0
+  const unsigned step = nthr * VEC;
+  const int ds = static_cast<int>(step / L), dt = static_cast<int>(step % L);
+  Cursor cur = cursor_at(tid * VEC, L, lengths, S);
   LossAcc acc;
   LossChunk<VEC> x, y;
-  loss_load(x, cur, logp_new, logp_old, adv, ret, val, S, L, C, ds, dt, lengths, err);
+  loss_load<VEC, ODD>(x, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
+  const Moments mom = ext != nullptr ? moments_from_ext(ext)
+                                     : merge_moments(mpart, Gm, WHITEN ? __ldg(adv) : 0.f, sh, shk);
+  const float mean = mom.c_mean, inv_std = mom.inv_std, inv_n = mom.inv_n;
   while (true) {
     if (cur.s >= S) {
-      loss_compute<VEC, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
+      loss_compute<VEC, ODD, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
       break;
     }
-    loss_load(y, cur, logp_new, logp_old, adv, ret, val, S, L, C, ds, dt, lengths, err);
-    loss_compute<VEC, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
+    loss_load<VEC, ODD>(y, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
+    loss_compute<VEC, ODD, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
     if (cur.s >= S) {
-      loss_compute<VEC, WHITEN>(y, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
+      loss_compute<VEC, ODD, WHITEN>(y, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
       break;
     }
-    loss_load(x, cur, logp_new, logp_old, adv, ret, val, S, L, C, ds, dt, lengths, err);
-    loss_compute<VEC, WHITEN>(y, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
+    loss_load<VEC, ODD>(x, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
+    loss_compute<VEC, ODD, WHITEN>(y, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
   }
   float v[kLossSums] = {acc.s.s, acc.v.s, acc.kl.s, acc.a.s, acc.aa.s};
   int nclip = acc.nclip;
@@ -513,56 +581,140 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
     for (int i = 0; i < kLossSums; ++i) p.s[i] = v[i];
     p.pad[0] = p.pad[1] = 0.f;
     lpart[blockIdx.x] = p;
+    __threadfence();  // the partial is visible before the ticket
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    const int G = static_cast<int>(gridDim.x);
+    Kahan k[kLossSums];
+    nclip = 0;
+#pragma unroll
+    for (int i = 0; i < kMaxPartsPerThread; ++i) {
+      const int j = threadIdx.x + i * kPpoThreads;
+      if (j < G) {
+        const LossPart p = load_part(lpart + j);
+        nclip += p.nclip;
+#pragma unroll
+        for (int q = 0; q < kLossSums; ++q) k[q].add(p.s[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kLossSums; ++q) v[q] = k[q].s;
+    block_sums<kLossSums>(v, nclip, sh, shk);
+    if (threadIdx.x == 0) write_stats(stats, v, nclip, mom, report_moments != 0);
   }
   pdl_launch_dependents();
 }
 
-// Pass 3: merge the G loss partials (every thread loads its few at once, compensated fp32,
-// then a fixed block tree) and write the statistics.
+// The statistics of an empty batch (the caller's moments, or none).
+__global__ void ppo_empty_kernel(const double* __restrict__ ext, int report_moments, double* __restrict__ stats) {
+  pdl_wait();
+  const float v[kLossSums] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  write_stats(stats, v, 0, ext != nullptr ? moments_from_ext(ext) : moments_from_sums(0, 0.f, 0.f, 0.f),
+              report_moments != 0);
+}
+
+// ---------------------------------------------------------------- one launch for small batches
+
+// A cluster of up to kMaxCluster CTAs covers the batch; each CTA's sums go to the CTAs that need
+// them with stores to distributed shared memory and are added in rank order.
+constexpr int kMaxCluster = 8;
+constexpr long long kSmallTokens = 16384;
+
+__device__ __forceinline__ void st_cluster_u32(const void* local, uint32_t rank, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_rank(smem_u32(local), rank)), "r"(v) : "memory");
+}
+
+template <int VEC, bool ODD, bool WHITEN>
 __global__ void __launch_bounds__(kPpoThreads)
-    ppo_finalize_kernel(const LossPart* __restrict__ lpart, int G, const double* __restrict__ mom,
-                        int report_moments, double* __restrict__ stats) {
+    ppo_small_kernel(const float* __restrict__ logp_new, const float* __restrict__ logp_old,
+                     const float* __restrict__ adv, const float* __restrict__ ret,
+                     const float* __restrict__ val, const int32_t* __restrict__ lengths, int S,
+                     int L, float eps, const double* __restrict__ ext, int report_moments,
+                     float* __restrict__ grad_logp, float* __restrict__ grad_val,
+                     double* __restrict__ stats, int* err) {
   __shared__ float sh[kLossSums][kPpoWarps];
   __shared__ int shk[kPpoWarps];
+  __shared__ uint32_t mrecv[kMaxCluster][3], lrecv[kMaxCluster][kLossSums + 1];
+  const int c = static_cast<int>(gridDim.x);
+  const uint32_t rank = blockIdx.x;  // one cluster
+  // first half of a cluster barrier: every CTA has started before the first push
+  if (c > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   pdl_wait();
-  LossPart p[kMaxPartsPerThread];
-#pragma unroll
-  for (int i = 0; i < kMaxPartsPerThread; ++i) {
-    const int j = threadIdx.x + i * kPpoThreads;
-    if (j < G) {
-      p[i] = load_part(lpart + j);
+  pdl_launch_dependents();
+  const unsigned tid = rank * kPpoThreads + threadIdx.x;
+  const unsigned nthr = c * kPpoThreads;
+  const unsigned step = nthr * VEC;
+  const int ds = static_cast<int>(step / L), dt = static_cast<int>(step % L);
+  Cursor cur = cursor_at(tid * VEC, L, lengths, S);
+  LossChunk<VEC> x, y;
+  loss_load<VEC, ODD>(x, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
+  Moments mom;
+  if (ext != nullptr) {
+    mom = moments_from_ext(ext);
+    if (c > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  } else {
+    int n = 0;
+    Kahan s1, s2;
+    const float shift = WHITEN ? __ldg(adv) : 0.f;
+    if (WHITEN) {
+      moments_walk<VEC, ODD>(adv, lengths, S, L, tid, nthr, shift, n, s1, s2, err);
     } else {
-      p[i] = LossPart{0, {0.f, 0.f, 0.f, 0.f, 0.f}, {0.f, 0.f}};
+      for (unsigned s = tid; s < static_cast<unsigned>(S); s += nthr)
+        n += row_length(lengths, static_cast<int>(s), L, err);
     }
+    float v[2] = {s1.s, s2.s};
+    block_sums<2>(v, n, sh, shk);
+    if (c > 1) {
+      asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+      if (threadIdx.x < static_cast<unsigned>(c)) {
+        st_cluster_u32(&mrecv[rank][0], threadIdx.x, static_cast<uint32_t>(n));
+        st_cluster_u32(&mrecv[rank][1], threadIdx.x, __float_as_uint(v[0]));
+        st_cluster_u32(&mrecv[rank][2], threadIdx.x, __float_as_uint(v[1]));
+      }
+      cluster_sync_all();
+      n = 0;
+      v[0] = v[1] = 0.f;
+      for (int q = 0; q < c; ++q) {
+        n += static_cast<int>(mrecv[q][0]);
+        v[0] += __uint_as_float(mrecv[q][1]);
+        v[1] += __uint_as_float(mrecv[q][2]);
+      }
+    }
+    mom = moments_from_sums(n, v[0], v[1], shift);
   }
-  int nclip = 0;
-  Kahan acc[kLossSums];
-#pragma unroll
-  for (int i = 0; i < kMaxPartsPerThread; ++i) {
-    nclip += p[i].nclip;
-#pragma unroll
-    for (int k = 0; k < kLossSums; ++k) acc[k].add(p[i].s[k]);
+  LossAcc acc;
+  while (true) {
+    const bool more = cur.s < S;
+    if (more) loss_load<VEC, ODD>(y, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
+    loss_compute<VEC, ODD, WHITEN>(x, mom.c_mean, mom.inv_std, mom.inv_n, eps, acc, grad_logp, grad_val);
+    if (!more) break;
+    x = y;
   }
-  float v[kLossSums];
-#pragma unroll
-  for (int k = 0; k < kLossSums; ++k) v[k] = acc[k].s;
+  float v[kLossSums] = {acc.s.s, acc.v.s, acc.kl.s, acc.a.s, acc.aa.s};
+  int nclip = acc.nclip;
   block_sums<kLossSums>(v, nclip, sh, shk);
-  if (threadIdx.x == 0) {
-    const double n = __ldcg(mom), inv = n > 0.0 ? 1.0 / n : 0.0;
-    stats[0] = -static_cast<double>(v[0]) * inv;
-    stats[1] = static_cast<double>(v[1]) * inv;
-    stats[2] = static_cast<double>(nclip) * inv;
-    stats[3] = static_cast<double>(v[2]) * inv;
-    if (report_moments) {
-      stats[4] = __ldcg(mom + 1);
-      stats[5] = n > 0.0 ? sqrt(__ldcg(mom + 2) * inv) : 0.0;
-    } else {
-      const double m = static_cast<double>(v[3]) * inv;
-      stats[4] = m;
-      stats[5] = n > 0.0 ? sqrt(fmax(static_cast<double>(v[4]) * inv - m * m, 0.0)) : 0.0;
+  if (c > 1) {
+    if (threadIdx.x == 0) {
+      st_cluster_u32(&lrecv[rank][kLossSums], 0, static_cast<uint32_t>(nclip));
+#pragma unroll
+      for (int q = 0; q < kLossSums; ++q) st_cluster_u32(&lrecv[rank][q], 0, __float_as_uint(v[q]));
     }
-    stats[6] = n;
+    cluster_sync_all();
+    if (rank == 0 && threadIdx.x == 0) {
+      nclip = 0;
+#pragma unroll
+      for (int q = 0; q < kLossSums; ++q) v[q] = 0.f;
+      for (int r = 0; r < c; ++r) {
+        nclip += static_cast<int>(lrecv[r][kLossSums]);
+#pragma unroll
+        for (int q = 0; q < kLossSums; ++q) v[q] += __uint_as_float(lrecv[r][q]);
+      }
+    }
   }
+  if (rank == 0 && threadIdx.x == 0) write_stats(stats, v, nclip, mom, report_moments != 0);
 }
 
 int num_sms() {
@@ -594,8 +746,7 @@ int one_wave(K kernel, long long work_items, int cap) {
 struct WsLayout {
   MomPart* mom;
   LossPart* loss;
-  double* moments;
-  float* coef;
+  unsigned* ticket;
 };
 
 WsLayout layout(void* ws) {
@@ -605,49 +756,41 @@ WsLayout layout(void* ws) {
   p += sizeof(MomPart) * kPpoMaxMomentBlocks;
   w.loss = reinterpret_cast<LossPart*>(p);
   p += sizeof(LossPart) * kPpoMaxLossBlocks;
-  w.moments = reinterpret_cast<double*>(p);
-  w.coef = reinterpret_cast<float*>(p + 4 * sizeof(double));
+  w.ticket = reinterpret_cast<unsigned*>(p);
   return w;
 }
 
+// 16-byte chunks of four tokens: rows of at least four tokens, aligned arrays
 bool vec4_ok(int64_t L, std::initializer_list<const void*> ptrs) {
-  if (L % 4 != 0) return false;
+  if (L < 4) return false;
   for (const void* p : ptrs)
     if (reinterpret_cast<uintptr_t>(p) % 16 != 0) return false;
   return true;
 }
 
-// Pass 1 and the coefficient merge. moments_out: where the fp64 moments go.
-int launch_moments_coef(const float* adv, const int32_t* lengths, int S, int L, bool with_adv,
-                        const double* ext, const WsLayout& w, double* moments_out, int* err,
-                        cudaStream_t st) {
+// Pass 1 into w.mom; returns its number of blocks, or a negative code. Clears the ticket.
+int launch_moments(const float* adv, const int32_t* lengths, int S, int L, bool with_adv,
+                   const WsLayout& w, int* err, cudaStream_t st) {
+  const bool v4 = vec4_ok(L, {adv});
+  const long long tokens = static_cast<long long>(S) * L;
   int G = 0;
-  if (ext == nullptr) {
-    const bool v4 = vec4_ok(L, {adv});
-    cudaError_t e;
-    if (v4 && with_adv) {
-      // a warp per row pair: S / 2 warps of work
-      G = one_wave(ppo_moments_rows_kernel, (static_cast<long long>(S) + 1) / 2 * 32,
-                   kPpoMaxMomentBlocks);
-      e = launch_pdl(ppo_moments_rows_kernel, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
-                     L, w.mom, err);
-    } else if (v4) {
-      G = one_wave(ppo_moments_kernel<4>, S, kPpoMaxMomentBlocks);
-      e = launch_pdl(ppo_moments_kernel<4>, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
-                     L, 0, w.mom, err);
-    } else {
-      G = one_wave(ppo_moments_kernel<1>, with_adv ? static_cast<long long>(S) * L : S,
-                   kPpoMaxMomentBlocks);
-      e = launch_pdl(ppo_moments_kernel<1>, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
-                     L, with_adv ? 1 : 0, w.mom, err);
-    }
-    if (e != cudaSuccess) return -3;
+  cudaError_t e;
+  if (v4 && with_adv && L % 4 == 0) {
+    // a warp per row pair: S / 2 warps of work
+    G = one_wave(ppo_moments_rows_kernel, (static_cast<long long>(S) + 1) / 2 * 32,
+                 kPpoMaxMomentBlocks);
+    e = launch_pdl(ppo_moments_rows_kernel, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
+                   L, w.mom, w.ticket, err);
+  } else if (v4) {
+    G = one_wave(ppo_moments_kernel<4, true>, with_adv ? (tokens + 3) / 4 : S, kPpoMaxMomentBlocks);
+    e = launch_pdl(ppo_moments_kernel<4, true>, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
+                   L, with_adv ? 1 : 0, w.mom, w.ticket, err);
+  } else {
+    G = one_wave(ppo_moments_kernel<1, false>, with_adv ? tokens : S, kPpoMaxMomentBlocks);
+    e = launch_pdl(ppo_moments_kernel<1, false>, dim3(G), dim3(kPpoThreads), 0, st, adv, lengths, S,
+                   L, with_adv ? 1 : 0, w.mom, w.ticket, err);
   }
-  return launch_pdl(ppo_coef_kernel, dim3(1), dim3(kPpoThreads), 0, st, adv, S, L, with_adv ? 1 : 0,
-                    static_cast<const MomPart*>(w.mom), G, ext, moments_out, w.coef) ==
-                 cudaSuccess
-             ? 0
-             : -3;
+  return e == cudaSuccess ? G : -3;
 }
 
 }  // namespace
@@ -659,17 +802,17 @@ size_t ppo_loss_workspace_bytes() {
 
 int launch_ppo_adv_moments(const float* adv, const int32_t* lengths, int64_t S, int64_t L,
                            double* out, void* ws, int* err, cudaStream_t st) {
-  if (S * L == 0) {
-    const WsLayout w = layout(ws);
-    return launch_pdl(ppo_coef_kernel, dim3(1), dim3(kPpoThreads), 0, st, adv,
-                      static_cast<int>(S), static_cast<int>(L), 0,
-                      static_cast<const MomPart*>(w.mom), 0, static_cast<const double*>(nullptr),
-                      out, w.coef) == cudaSuccess
-               ? 0
-               : -3;
+  const int Si = static_cast<int>(S), Li = static_cast<int>(L);
+  const WsLayout w = layout(ws);
+  int G = 0;
+  if (S * L > 0) {
+    G = launch_moments(adv, lengths, Si, Li, true, w, err, st);
+    if (G < 0) return G;
   }
-  return launch_moments_coef(adv, lengths, static_cast<int>(S), static_cast<int>(L), true,
-                             nullptr, layout(ws), out, err, st);
+  return launch_pdl(ppo_merge_kernel, dim3(1), dim3(kPpoThreads), 0, st, adv, Si, Li,
+                    static_cast<const MomPart*>(w.mom), G, out) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 int launch_ppo_loss(const float* logp_new, const float* logp_old, const float* adv,
@@ -678,43 +821,54 @@ int launch_ppo_loss(const float* logp_new, const float* logp_old, const float* a
                     float* grad_logp, float* grad_val, double* stats, void* ws, int* err,
                     cudaStream_t st) {
   const int Si = static_cast<int>(S), Li = static_cast<int>(L);
-  const WsLayout w = layout(ws);
   const int report = (whiten || ext_moments != nullptr) ? 1 : 0;
-  if (S * L == 0) {
-    // empty batch: moments (the caller's, or none) and statistics only
-    if (launch_pdl(ppo_coef_kernel, dim3(1), dim3(kPpoThreads), 0, st, adv, Si, Li, 0,
-                   static_cast<const MomPart*>(w.mom), 0, ext_moments, w.moments, w.coef) !=
-        cudaSuccess)
-      return -3;
-    return launch_pdl(ppo_finalize_kernel, dim3(1), dim3(kPpoThreads), 0, st,
-                      static_cast<const LossPart*>(w.loss), 0,
-                      static_cast<const double*>(w.moments), report, stats) == cudaSuccess
-               ? 0
-               : -3;
-  }
-  if (launch_moments_coef(adv, lengths, Si, Li, whiten, ext_moments, w, w.moments, err, st) != 0)
-    return -3;
-  const bool v4 = vec4_ok(L, {logp_new, logp_old, adv, ret, val, grad_logp, grad_val});
-  const long long items = S * (v4 ? L / 4 : L);
-  int G = 0;
   cudaError_t e;
-#define HY_PPO_LAUNCH(V, W)                                                                      \
-  G = one_wave(ppo_loss_kernel<V, W>, items, kPpoMaxLossBlocks);                                \
-  e = launch_pdl(ppo_loss_kernel<V, W>, dim3(G), dim3(kPpoThreads), 0, st, logp_new, logp_old, \
-                 adv, ret, val, lengths, Si, Li, eps, static_cast<const float*>(w.coef), w.loss, \
-                 grad_logp, grad_val, err)
-  if (v4) {
-    if (whiten) { HY_PPO_LAUNCH(4, true); } else { HY_PPO_LAUNCH(4, false); }
-  } else {
-    if (whiten) { HY_PPO_LAUNCH(1, true); } else { HY_PPO_LAUNCH(1, false); }
+  if (S * L == 0) {
+    e = launch_pdl(ppo_empty_kernel, dim3(1), dim3(1), 0, st, ext_moments, report, stats);
+    return e == cudaSuccess ? 0 : -3;
   }
-#undef HY_PPO_LAUNCH
-  if (e != cudaSuccess) return -3;
-  return launch_pdl(ppo_finalize_kernel, dim3(1), dim3(kPpoThreads), 0, st,
-                    static_cast<const LossPart*>(w.loss), G,
-                    static_cast<const double*>(w.moments), report, stats) == cudaSuccess
-             ? 0
-             : -3;
+  const bool v4 = vec4_ok(L, {logp_new, logp_old, adv, ret, val, grad_logp, grad_val});
+  const long long items = v4 ? (S * L + 3) / 4 : S * L;
+  if (S * L <= kSmallTokens) {
+    // CTAs until every thread has one chunk, at most a cluster
+    const long long want = (items + kPpoThreads - 1) / kPpoThreads;
+    const int c = want >= kMaxCluster ? kMaxCluster : (want > 4 ? kMaxCluster : (want > 2 ? 4 : static_cast<int>(want)));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(c));
+    cfg.blockDim = dim3(kPpoThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = static_cast<unsigned>(c);
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = c > 1 ? 2 : 1;
+    auto go = [&](auto kernel) {
+      return cudaLaunchKernelEx(&cfg, kernel, logp_new, logp_old, adv, ret, val, lengths, Si, Li, eps,
+                                ext_moments, report, grad_logp, grad_val, stats, err);
+    };
+    // (one form for whole and odd rows: at this size the straddling code costs nothing)
+    if (v4) e = whiten ? go(ppo_small_kernel<4, true, true>) : go(ppo_small_kernel<4, true, false>);
+    else e = whiten ? go(ppo_small_kernel<1, false, true>) : go(ppo_small_kernel<1, false, false>);
+    return e == cudaSuccess ? 0 : -3;
+  }
+  // the caller's moments need no pass over the batch: an empty one clears the ticket
+  const WsLayout w = layout(ws);
+  const int Gm = launch_moments(adv, lengths, ext_moments != nullptr ? 0 : Si, Li, whiten, w, err, st);
+  if (Gm < 0) return Gm;
+  auto go = [&](auto kernel) {
+    const int G = one_wave(kernel, items, kPpoMaxLossBlocks);
+    return launch_pdl(kernel, dim3(G), dim3(kPpoThreads), 0, st, logp_new, logp_old, adv, ret, val,
+                      lengths, Si, Li, eps, static_cast<const MomPart*>(w.mom), Gm, ext_moments,
+                      report, w.loss, w.ticket, grad_logp, grad_val, stats, err);
+  };
+  if (v4 && L % 4 == 0) e = whiten ? go(ppo_loss_kernel<4, false, true>) : go(ppo_loss_kernel<4, false, false>);
+  else if (v4) e = whiten ? go(ppo_loss_kernel<4, true, true>) : go(ppo_loss_kernel<4, true, false>);
+  else e = whiten ? go(ppo_loss_kernel<1, false, true>) : go(ppo_loss_kernel<1, false, false>);
+  return e == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace hydra
