@@ -213,31 +213,44 @@ __device__ __forceinline__ void tc_mma_ts_bf16(uint32_t d_tmem, uint32_t a_tmem,
 
 
 // This CTA's work: units t = blockIdx.x + i * gridDim.x (i = 0, 1, ...). Unit (p, head, seq)
-// holds the two query tiles qa = 2p and qb = 2p + 1 (qb only when it exists): tile a runs key
-// blocks 0..qa, tile b 0..qb, and every key block the two share is loaded once for both. Two
-// orders of the units t:
+// holds two adjacent query tiles q0 (a) and q0 + 1 (b): tile a runs key blocks 0..q0, tile b
+// 0..q0 + 1, and every key block the two share is loaded once for both. An odd number of tiles
+// leaves one alone. With several units per CTA that is the first tile, which has a single key
+// block (kLoneFirst: tiles 0 | 1, 2 | 3, 4 | ...); with one unit per CTA the last, which then runs
+// the longest unit by itself (3 x 640 x 16 heads: 13.5 us against 15.9).
+// Three orders of the units t:
 //  * longest first: t -> (p, head, seq) with the largest p (most key blocks) first;
 //  * grouped: the units of one (head, sequence) consecutive, longest first within it, so
 //    that they run at the same time on neighbouring CTAs and read the key / value blocks
 //    they share from DRAM once (the longest-first order runs them waves apart, when the
-//    blocks have left L2).
-// The launcher takes the grouped order unless it raises the busiest CTA's load (in key
-// blocks) of the static round-robin assignment by more than 5 % over the longest-first order.
+//    blocks have left L2);
+//  * rotated: grouped, with the lengths within a group rotated by the wave it falls in. Where the
+//    number of units per group divides the grid (four units, 152 CTAs), the grouped order
+//    gives a CTA units of one length only.
+// 8 x 800 x 32 heads: 83.5 us with the last tile alone, longest first; 69.6 with the first alone,
+// rotated, and the rowless warps of the last tile skipped. 8 x 1000: 94.1 -> 83.6.
+// The launcher takes the grouped order that loads the busiest CTA of the static round-robin
+// assignment less, unless that is more than 5 % above the longest-first order.
+constexpr int kLongest = 0, kGrouped = 1, kRotated = 2, kLoneFirst = 4;
+
 struct UnitCursor {
   int t;               // unit
-  int p, head, seq;    // decoded unit
+  int q0, head, seq;   // decoded unit: its first query tile
   int na, nb, nblk;    // key blocks of tile a, of tile b (0: no tile b), of the unit
   // the loop-invariant sizes are recomputed from the kernel arguments (constant bank) rather
   // than kept in registers: the producer and MMA warps run with few registers
   __host__ __device__ static int units(int P, int heads, int nseq) {
     return (((P + kBQ - 1) / kBQ + 1) / 2) * heads * nseq;
   }
-  __host__ __device__ void decode(int P, int heads, int nseq, int grouped) {
+  __host__ __device__ void decode(int P, int heads, int nseq, int mode, int grid) {
     const int nqb = (P + kBQ - 1) / kBQ;
     const int npairs = (nqb + 1) / 2;
-    if (grouped) {
+    int p;
+    if ((mode & 3) != kLongest) {
       const int g = t / npairs;
-      p = npairs - 1 - t % npairs;
+      int i = t - g * npairs;
+      if ((mode & 3) == kRotated) i = (i + g * npairs / grid) % npairs;
+      p = npairs - 1 - i;
       head = g % heads;
       seq = g / heads;
     } else {
@@ -247,16 +260,22 @@ struct UnitCursor {
       head = r % heads;
       seq = r / heads;
     }
-    na = 2 * p + 1;
-    nb = (2 * p + 1 < nqb) ? 2 * p + 2 : 0;
+    const int odd = (mode & kLoneFirst) != 0 ? nqb & 1 : 0;
+    q0 = p > 0 ? 2 * p - odd : 0;
+    na = q0 + 1;
+    nb = (odd && p == 0) || q0 + 1 >= nqb ? 0 : q0 + 2;
     nblk = nb > 0 ? nb : na;
   }
 };
 
+// kMode: unit order and kLoneFirst; kRagged: the last tile has warps without a valid row. Compile-time,
+// so that a shape pays for its own form alone (as run-time values they cost 8 x 768 x 32 heads
+// 2 % and 12 x 768 3 %).
+template <int kMode, bool kRagged>
 __global__ void __launch_bounds__(kThreads, 1)
     causal_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv,
                                const __grid_constant__ CUtensorMap tm_out, int P, int d,
-                               int n_heads, int nseq, int grouped, float scale_log2, int* err) {
+                               int n_heads, int nseq, float scale_log2, int* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -323,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                              kDevTimeoutProducer))
           return false;
         if (elect_one()) {
-          const int y = c.seq * P + (2 * c.p + x) * kBQ;
+          const int y = c.seq * P + (c.q0 + x) * kBQ;
           mbar_arrive_expect_tx(q_full(x), kMat);
           tma_load_2d(sQ(x), &tm_qkv, c.head * kDh, y, q_full(x));
           tma_load_2d(sQ(x) + kTile, &tm_qkv, c.head * kDh + 64, y, q_full(x));
@@ -356,21 +375,21 @@ __global__ void __launch_bounds__(kThreads, 1)
         UnitCursor nx;
         nx.t = c.t + gridDim.x;
         if (nx.t >= nunits || !elect_one()) return;
-        nx.decode(P, n_heads, nseq, grouped);
+        nx.decode(P, n_heads, nseq, kMode, gridDim.x);
         const int y0 = nx.seq * P;
         for (int x = 0; x < (nx.nb > 0 ? 2 : 1); ++x)
           for (int h = 0; h < 2; ++h)
-            tma_prefetch_l2_2d(&tm_qkv, nx.head * kDh + 64 * h, y0 + (2 * nx.p + x) * kBQ);
+            tma_prefetch_l2_2d(&tm_qkv, nx.head * kDh + 64 * h, y0 + (nx.q0 + x) * kBQ);
         for (int j = 0; j < (nx.nblk < 2 ? nx.nblk : 2); ++j)
           for (int kv = 1; kv <= 2; ++kv)
             for (int h = 0; h < 2; ++h)
               tma_prefetch_l2_2d(&tm_qkv, kv * d + nx.head * kDh + 64 * h, y0 + j * kBK);
       };
       for (c.t = blockIdx.x; ok && c.t < nunits; c.t += gridDim.x) {
-        c.decode(P, n_heads, nseq, grouped);
+        c.decode(P, n_heads, nseq, kMode, gridDim.x);
         // prefetch after this block's loads (longest-first order only: with the grouped
         // order the next unit's blocks are mostly in L2 already, and the prefetch measured slower)
-        const int jpf = grouped ? -1 : (c.nblk > 3 ? c.nblk - 3 : 0);
+        const int jpf = (kMode & 3) != kLongest ? -1 : (c.nblk > 3 ? c.nblk - 3 : 0);
         ok = load_q(0) && load_kv(1, 0);
         if (ok && c.nb > 0) ok = load_q(1);
         if (ok) ok = load_kv(2, 0);
@@ -463,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     float l = 0.f;                            // row sum of the probabilities
     UnitCursor c;
     for (c.t = blockIdx.x; ok && c.t < nunits; c.t += gridDim.x) {
-      c.decode(P, n_heads, nseq, grouped);
+      c.decode(P, n_heads, nseq, kMode, gridDim.x);
       const int n = x == 0 ? c.na : c.nb;     // this tile's key blocks (0: no tile b)
       const int on = x == 0 ? c.nb : c.na;    // the other tile's
       const int J = c.nblk;
@@ -472,6 +491,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         s0_issued = false;
         continue;
       }
+      // a warp whose 32 rows lie past the sequence's end has nothing to compute: it only meets its
+      // group's barriers (its rows of P and O hold whatever they held and are never stored)
+      const bool dead = kRagged && (c.q0 + x) * kBQ + q4 * 32 >= P;
       // ring positions: K_j at 2 (kbase + j), V_j right after it
       if (!s0_issued && issuer) ok = issue_s(true, 2 * kbase, on > 0 ? 1 : 2, n == 1);
       for (int j = 0; ok && j < n; ++j) {
@@ -481,71 +503,73 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         ++gs;
         tc_fence_after();
-        float sv[kBK];
-        tc_ld_x64(t_s, *reinterpret_cast<float(*)[64]>(sv));
-        tc_ld_x64(t_s + 64, *reinterpret_cast<float(*)[64]>(sv + 64));
-        tc_wait_ld();
-        // the diagonal block (the tile's last): key c is visible to row `row` iff c <= row
-        const bool diag = (j == n - 1);
-        if (diag) {
+        if (!dead) {
+          float sv[kBK];
+          tc_ld_x64(t_s, *reinterpret_cast<float(*)[64]>(sv));
+          tc_ld_x64(t_s + 64, *reinterpret_cast<float(*)[64]>(sv + 64));
+          tc_wait_ld();
+          // the diagonal block (the tile's last): key c is visible to row `row` iff c <= row
+          const bool diag = (j == n - 1);
+          if (diag) {
 #pragma unroll
-          for (int k = 1; k < kBK; ++k)
-            if (k > row) sv[k] = -INFINITY;
-        }
-        float pm[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) pm[i] = -FLT_MAX;
-#pragma unroll
-        for (int i = 0; i < kBK / 2; ++i) pm[i & 7] = max3(pm[i & 7], sv[2 * i], sv[2 * i + 1]);
-        const float mx = max3(max3(pm[0], pm[1], pm[2]), max3(pm[3], pm[4], pm[5]),
-                              fmaxf(pm[6], pm[7])) *
-                         scale_log2;
-        bool rescale = false;
-        float corr = 1.f;
-        if (j == 0) {
-          m_ref = mx;
-          l = 0.f;
-        } else if (mx > m_ref + 8.f) {
-          corr = ex2(m_ref - mx);
-          m_ref = mx;
-          rescale = true;
-        }
-        // P = 2^(scale s - m_ref) as bf16 pairs over the first 64 columns of S_x; the argument
-        // and the row sum in packed pairs
-        const uint64_t sc2 = f2_pack(scale_log2, scale_log2), nm2 = f2_pack(-m_ref, -m_ref);
-        uint64_t acc[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = f2_pack(0.f, 0.f);
-        uint32_t w[kBK / 2];
-#pragma unroll
-        for (int i = 0; i < kBK / 2; ++i) {
-          float a0, a1;
-          f2_unpack(f2_fma(f2_pack(sv[2 * i], sv[2 * i + 1]), sc2, nm2), a0, a1);
-          const float p0 = ex2(a0), p1 = ex2(a1);
-          acc[i & 3] = f2_add(acc[i & 3], f2_pack(p0, p1));
-          w[i] = pack_bf16x2(p0, p1);
-        }
-        float ps[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) f2_unpack(acc[i], ps[2 * i], ps[2 * i + 1]);
-        l = l * corr + (((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7])));
-        // O_x holds the sum through the previous block (that P V finished before this S was
-        // issued): rescale the row when the reference moved
-        if (__any_sync(0xffffffffu, rescale)) {
-#pragma unroll 1
-          for (int h = 0; h < 4; ++h) {
-            uint32_t o[32];
-            tc_ld_32x32b_x32(t_o + 32 * h, o);
-            tc_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
-            tc_st_x32(t_o + 32 * h, o);
-            tc_wait_st();
+            for (int k = 1; k < kBK; ++k)
+              if (k > row) sv[k] = -INFINITY;
           }
+          float pm[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pm[i] = -FLT_MAX;
+#pragma unroll
+          for (int i = 0; i < kBK / 2; ++i) pm[i & 7] = max3(pm[i & 7], sv[2 * i], sv[2 * i + 1]);
+          const float mx = max3(max3(pm[0], pm[1], pm[2]), max3(pm[3], pm[4], pm[5]),
+                                fmaxf(pm[6], pm[7])) *
+                           scale_log2;
+          bool rescale = false;
+          float corr = 1.f;
+          if (j == 0) {
+            m_ref = mx;
+            l = 0.f;
+          } else if (mx > m_ref + 8.f) {
+            corr = ex2(m_ref - mx);
+            m_ref = mx;
+            rescale = true;
+          }
+          // P = 2^(scale s - m_ref) as bf16 pairs over the first 64 columns of S_x; the argument
+          // and the row sum in packed pairs
+          const uint64_t sc2 = f2_pack(scale_log2, scale_log2), nm2 = f2_pack(-m_ref, -m_ref);
+          uint64_t acc[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[i] = f2_pack(0.f, 0.f);
+          uint32_t w[kBK / 2];
+#pragma unroll
+          for (int i = 0; i < kBK / 2; ++i) {
+            float a0, a1;
+            f2_unpack(f2_fma(f2_pack(sv[2 * i], sv[2 * i + 1]), sc2, nm2), a0, a1);
+            const float p0 = ex2(a0), p1 = ex2(a1);
+            acc[i & 3] = f2_add(acc[i & 3], f2_pack(p0, p1));
+            w[i] = pack_bf16x2(p0, p1);
+          }
+          float ps[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) f2_unpack(acc[i], ps[2 * i], ps[2 * i + 1]);
+          l = l * corr + (((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7])));
+          // O_x holds the sum through the previous block (that P V finished before this S was
+          // issued): rescale the row when the reference moved
+          if (__any_sync(0xffffffffu, rescale)) {
+#pragma unroll 1
+            for (int h = 0; h < 4; ++h) {
+              uint32_t o[32];
+              tc_ld_32x32b_x32(t_o + 32 * h, o);
+              tc_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
+              tc_st_x32(t_o + 32 * h, o);
+              tc_wait_st();
+            }
+          }
+          tc_st_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(w));
+          tc_st_x32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(w + 32));
+          tc_wait_st();
         }
-        tc_st_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(w));
-        tc_st_x32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(w + 32));
-        tc_wait_st();
         tc_fence_before();
         wg_sync(x);  // P_x of the whole tile is in TMEM
         if (issuer) {
@@ -558,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             nx.t = c.t + gridDim.x;
             s0_issued = false;
             if (nx.t < nunits) {
-              nx.decode(P, n_heads, nseq, grouped);
+              nx.decode(P, n_heads, nseq, kMode, gridDim.x);
               const int nn = x == 0 ? nx.na : nx.nb, non = x == 0 ? nx.nb : nx.na;
               if (nn > 0) {
                 ok = issue_s(true, 2 * (kbase + J), non > 0 ? 1 : 2, nn == 1);
@@ -583,7 +607,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       tc_fence_after();
-      {
+      if (dead) {
+        wg_sync(x);  // the previous unit's stores have read the staging buffer
+      } else {
         uint32_t o[4][32];
 #pragma unroll
         for (int q = 0; q < 4; ++q) tc_ld_32x32b_x32(t_o + 32 * q, o[q]);
@@ -607,7 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (issuer) {
         if (elect_one()) {
           for (int h = 0; h < 2; ++h)
-            tma_store_3d(&tm_out, s_stage + h * kTile, c.head * kDh + 64 * h, (2 * c.p + x) * kBQ,
+            tma_store_3d(&tm_out, s_stage + h * kTile, c.head * kDh + 64 * h, (c.q0 + x) * kBQ,
                          c.seq);
           bulk_commit();
         }
@@ -627,6 +653,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+struct Launch {
+  CUtensorMap map, map_out;
+  int P, d, n_heads, nseq;
+  float scale_log2;
+  int* err;
+  unsigned grid;
+  int dev;
+  cudaStream_t st;
+};
+
+template <int kMode, bool kRagged>
+int launch_form(const Launch& l) {
+  static bool attr_set[64] = {false};  // the shared-memory limit is a per-device attribute
+  if (l.dev < 0 || l.dev >= 64) return -1;
+  if (!attr_set[l.dev]) {
+    if (cudaFuncSetAttribute(causal_attention_tc_kernel<kMode, kRagged>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+      return -1;
+    attr_set[l.dev] = true;
+  }
+  causal_attention_tc_kernel<kMode, kRagged><<<l.grid, kThreads, kSmem, l.st>>>(
+      l.map, l.map_out, l.P, l.d, l.n_heads, l.nseq, l.scale_log2, l.err);
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+}
+
 }  // namespace attn_tc
 
 int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld, int64_t n_heads,
@@ -634,13 +685,6 @@ int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld
   using namespace attn_tc;
   if (nseq == 0 || P == 0) return 0;
   if (head_dim != kDh) return -4;
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(causal_attention_tc_kernel,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
-      return -1;
-    attr_set = true;
-  }
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
@@ -654,35 +698,51 @@ int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld
   if (!make_tma_map_3d(&map_out, out, d, P, nseq, ld_out, P * ld_out, kBQ)) return -2;
   const int64_t nunits = ((P + 2 * kBQ - 1) / (2 * kBQ)) * n_heads * nseq;
   const unsigned grid = static_cast<unsigned>(nunits < nsm ? nunits : nsm);
-  // unit order: grouped unless it loads the busiest CTA of the static round-robin assignment
-  // with more than 5 % more key blocks than the longest-first order does (its shared reads
-  // measured worth that much: 8 x 768 x 32 heads, equal loads, 64 -> 58 us; 16 x 768 x 32
-  // heads, 46 against 44 blocks, 119 -> 102 us; 16 x 300 x 12 heads, 9 against 8, slower).
-  // The choice for the last shape is kept.
+  // unit order (see UnitCursor): a grouped one unless it loads the busiest CTA of the static
+  // round-robin assignment with more than 5 % more key blocks than the longest-first order does
+  // (its shared reads measured worth that much: 8 x 768 x 32 heads, equal loads, 64 -> 58 us;
+  // 16 x 768 x 32 heads, 46 against 44 blocks, 119 -> 102 us; 16 x 300 x 12 heads, 9 against 8,
+  // slower). The choice for the last shape is kept.
   struct OrderChoice {
     int64_t nseq, P, heads;
     unsigned grid;
-    int grouped;
+    int mode;
   };
   static thread_local OrderChoice last = {-1, -1, -1, 0, 0};
   if (last.nseq != nseq || last.P != P || last.heads != n_heads || last.grid != grid) {
-    auto busiest = [&](int grouped) {
+    const int lone = nunits > static_cast<int64_t>(grid) ? kLoneFirst : 0;
+    auto busiest = [&](int order) {
       std::vector<int64_t> load(grid, 0);
       UnitCursor c;
       for (int64_t t = 0; t < nunits; ++t) {
         c.t = static_cast<int>(t);
-        c.decode(static_cast<int>(P), static_cast<int>(n_heads), static_cast<int>(nseq), grouped);
+        c.decode(static_cast<int>(P), static_cast<int>(n_heads), static_cast<int>(nseq), order | lone,
+                 static_cast<int>(grid));
         load[t % grid] += c.nblk;
       }
       return *std::max_element(load.begin(), load.end());
     };
-    last = {nseq, P, n_heads, grid, busiest(1) * 20 <= busiest(0) * 21 ? 1 : 0};
+    const int64_t lf = busiest(kLongest), gr = busiest(kGrouped), ro = busiest(kRotated);
+    const int order = std::min(gr, ro) * 20 <= lf * 21 ? (ro < gr ? kRotated : kGrouped) : kLongest;
+    last = {nseq, P, n_heads, grid, order | lone};
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(head_dim));
-  causal_attention_tc_kernel<<<grid, kThreads, kSmem, st>>>(
-      map, map_out, static_cast<int>(P), static_cast<int>(d), static_cast<int>(n_heads),
-      static_cast<int>(nseq), last.grouped, scale_log2, err);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+  const bool ragged = (P - 1) % kBQ < kBQ - 32;
+  const Launch l{map, map_out, static_cast<int>(P), static_cast<int>(d), static_cast<int>(n_heads),
+                 static_cast<int>(nseq), scale_log2, err, grid, dev, st};
+#define HY_ATT(mode) \
+  case mode:         \
+    return ragged ? launch_form<mode, true>(l) : launch_form<mode, false>(l)
+  switch (last.mode) {
+    HY_ATT(kLongest);
+    HY_ATT(kGrouped);
+    HY_ATT(kRotated);
+    HY_ATT(kLongest | kLoneFirst);
+    HY_ATT(kGrouped | kLoneFirst);
+    HY_ATT(kRotated | kLoneFirst);
+  }
+#undef HY_ATT
+  return -4;
 }
 
 }  // namespace hydra
