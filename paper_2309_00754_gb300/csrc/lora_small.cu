@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(32 * kGvWarps)
                           const __nv_bfloat16* __restrict__ x_on, int M, int K, int N,
                           const __nv_bfloat16* __restrict__ W, const __nv_bfloat16* __restrict__ u,
                           const __nv_bfloat16* __restrict__ B, int r, void* y_off, void* y_on,
-                          int out_f32, int shared_x) {
+                          int out_f32, int shared_x, int x_settled) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int kGvStages = Gv<NT, kGvWarps>::kStages;
   constexpr int kGvStageBytes = Gv<NT, kGvWarps>::kStageBytes;
@@ -458,12 +458,15 @@ __global__ void __launch_bounds__(32 * kGvWarps)
   // W is frozen: the first chunks of this warp's [16 x K-range] slice stream into L2 while
   // the preceding kernel finishes (programmatic dependent launch); x, u and y are touched
   // only after pdl_wait(). Prefetching the whole slice instead evicts, on the large
-  // shapes, lines the running kernel has yet to read.
+  // shapes, lines the running kernel has yet to read. Where the preceding kernel is this call's
+  // own lora_down (x_settled), x was final before this kernel could start: the stream of W runs
+  // beside it and only u waits (one row of two streams, 4096 x 4096: 10.8 us for the two launches
+  // in turn, 8.5 so; 8 rows x 11008 columns 29.1, 24.5).
   pdl_launch_dependents();
   if (c0 < c1 && lane < 16 && n0 + lane < N)
     prefetch_l2_bulk(W + static_cast<size_t>(n0 + lane) * K + c0 * 64,
                      static_cast<uint32_t>(min(K, min(c1, c0 + kGvStages) * 64) - c0 * 64) * 2u);
-  pdl_wait();
+  if (!x_settled) pdl_wait();
 
   // token row copied by this lane's slice of the x stage (rows lane >> 3 and 4 + lane >> 3...)
   auto xrow = [&](int tk) {
@@ -538,6 +541,7 @@ __global__ void __launch_bounds__(32 * kGvWarps)
     __syncwarp();
   }
   gv_wait<0>();
+  if (x_settled) pdl_wait();    // u is complete; y may be written
   if (kAlias) __syncthreads();  // the ring is free before it holds the partial tiles
 
   // partial [16 rows x 8 NT tokens] of this warp -> shared memory
@@ -573,7 +577,7 @@ __global__ void __launch_bounds__(32 * kGvWarps)
         const uint4* up = reinterpret_cast<const uint4*>(u + static_cast<size_t>(m) * r);
         const uint4* bp = reinterpret_cast<const uint4*>(B + static_cast<size_t>(n) * r);
         for (int j = 0; j < r / 8; ++j) {
-          const uint4 a4 = __ldg(up + j), b4 = __ldg(bp + j);
+          const uint4 a4 = __ldcg(up + j), b4 = __ldg(bp + j);  // u may be younger than this launch
           const uint32_t* ap = &a4.x;
           const uint32_t* bq = &b4.x;
 #pragma unroll
@@ -623,7 +627,7 @@ void launch_gemv_t(const GemmArgs& a, int nsm, cudaStream_t stream) {
       static_cast<const __nv_bfloat16*>(a.shared_x ? a.x_off : a.x_on), static_cast<int>(a.M),
       static_cast<int>(a.K), static_cast<int>(a.N), static_cast<const __nv_bfloat16*>(a.W),
       static_cast<const __nv_bfloat16*>(a.u), static_cast<const __nv_bfloat16*>(a.B),
-      static_cast<int>(a.r), a.y_off, a.y_on, a.out_f32, a.shared_x ? 1 : 0);
+      static_cast<int>(a.r), a.y_off, a.y_on, a.out_f32, a.shared_x ? 1 : 0, a.x_settled ? 1 : 0);
 }
 
 // Streaming lora_down: clusters of ck CTAs (a power of two up to 8) along K, ck as large as

@@ -114,3 +114,29 @@ def test_off_rows_ignore_a_non_finite_lora_factor():
     y = [torch.empty(M, N, device="cuda") for _ in range(2)]
     H.hydra_lora_linear(d[0], d[1], dW, A, B, 2.0, y[0], y[1], ws)
     assert np.all(np.isfinite(host_f64(y[0]))) and not bool(torch.isfinite(y[1]).any())
+
+
+@pytest.mark.parametrize("M,K,N,r,shared", [(1, 4096, 4096, 16, False), (8, 520, 1048, 64, False), (16, 1032, 264, 8, True)])
+def test_gemv_beside_its_lora_down_matches_the_two_calls_in_turn(M, K, N, r, shared):
+    """hydra_lora_linear's GEMV starts before its lora_down has ended; hydra_lora_down followed by
+    hydra_dual_linear runs the same arithmetic in turn: the same bits, also with new inputs in the
+    same buffers, call after call."""
+    x, W, ab = _problem(M, K, N, r, seed=17 + M)
+    dW, A, B = dev_bf16(W), dev_bf16(ab[0][0]), dev_bf16(ab[0][1])
+    buf = [torch.empty(M, K, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    ws = torch.empty(H.lora_linear_workspace_size(M, r), dtype=torch.uint8, device="cuda")
+    got = [[torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(2)] for _ in range(40)]
+    for i, y in enumerate(got):
+        for j in range(2):
+            buf[j].copy_(dev_bf16(x[(i + j) % 3]))
+        H.hydra_lora_linear(buf[0], None if shared else buf[1], dW, A, B, 2.0, y[0], y[1], ws)
+    for i in range(3):
+        xs = [dev_bf16(x[(i + j) % 3]) for j in range(2)]
+        xo = xs[0] if shared else xs[1]
+        u = torch.empty(M, r, dtype=torch.bfloat16, device="cuda")
+        H.hydra_lora_down(xo, A, 2.0, u)
+        torch.cuda.synchronize()
+        y = [torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        H.hydra_dual_linear(xs[0], None if shared else xo, dW, u, B, y[0], y[1])
+        for k in range(i, 40, 3):
+            assert torch.equal(got[k][0], y[0]) and torch.equal(got[k][1], y[1])
