@@ -175,9 +175,17 @@ def _p(t):
     return None if t is None else t.data_ptr()
 
 
+# The current stream's handle without a Stream object around it (3.0 us of a 13 us call, 0.2 so).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def _out_dtype(t, name="output"):
@@ -190,7 +198,7 @@ def _out_dtype(t, name="output"):
 
 
 def _req(t, dtype, name):
-    if t is None:
+    if t is None or (t.dtype is dtype and t.is_cuda and t.is_contiguous()):
         return
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
