@@ -322,6 +322,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // a dependent launch: the set-up above overlaps the end of the preceding kernel, which wrote qkv
+  // and may still read out
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
@@ -673,9 +677,10 @@ int launch_form(const Launch& l) {
       return -1;
     attr_set[l.dev] = true;
   }
-  causal_attention_tc_kernel<kMode, kRagged><<<l.grid, kThreads, kSmem, l.st>>>(
-      l.map, l.map_out, l.P, l.d, l.n_heads, l.nseq, l.scale_log2, l.err);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+  return launch_pdl(causal_attention_tc_kernel<kMode, kRagged>, dim3(l.grid), dim3(kThreads), kSmem, l.st,
+                    l.map, l.map_out, l.P, l.d, l.n_heads, l.nseq, l.scale_log2, l.err) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 }  // namespace attn_tc

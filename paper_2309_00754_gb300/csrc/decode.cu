@@ -32,6 +32,8 @@ constexpr int kDh = 128;  // head_dim of every decoder in this library
 __global__ void kv_store_prefill_kernel(const __nv_bfloat16* __restrict__ qkv, int P0, int ld,
                                         int d, int H, int Pmax, __nv_bfloat16* __restrict__ ck,
                                         __nv_bfloat16* __restrict__ cv) {
+  pdl_wait();
+  pdl_launch_dependents();
   // block = one prompt row (i, p); 8 bf16 per thread step over the k and v blocks
   const long long row = blockIdx.x;
   const int i = static_cast<int>(row / P0), p = static_cast<int>(row % P0);
@@ -932,11 +934,12 @@ __global__ void __launch_bounds__(kSampleThreads)
 int launch_kv_store_prefill(const void* qkv, int64_t R, int64_t P0, int64_t ld, int64_t d,
                             int64_t H, int64_t Pmax, void* ck, void* cv, cudaStream_t st) {
   if (R * P0 == 0) return 0;
-  kv_store_prefill_kernel<<<static_cast<unsigned>(R * P0), 256, 0, st>>>(
-      static_cast<const __nv_bfloat16*>(qkv), static_cast<int>(P0), static_cast<int>(ld),
-      static_cast<int>(d), static_cast<int>(H), static_cast<int>(Pmax),
-      static_cast<__nv_bfloat16*>(ck), static_cast<__nv_bfloat16*>(cv));
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+  return launch_pdl(kv_store_prefill_kernel, dim3(static_cast<unsigned>(R * P0)), dim3(256), 0, st,
+                    static_cast<const __nv_bfloat16*>(qkv), static_cast<int>(P0), static_cast<int>(ld),
+                    static_cast<int>(d), static_cast<int>(H), static_cast<int>(Pmax),
+                    static_cast<__nv_bfloat16*>(ck), static_cast<__nv_bfloat16*>(cv)) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 size_t decode_attention_smem(int64_t Pmax) {

@@ -200,7 +200,7 @@ int launch_head_dot(const void* x, int64_t d, const void* w, const RowMap& map, 
                     const int32_t* lengths, int64_t L, float* out, cudaStream_t st);
 int launch_seq_score(const float* h, const void* norm, const void* w, int64_t d, float eps,
                      const int32_t* lengths, int64_t S, int64_t L, int64_t P, int64_t p0,
-                     float* score, cudaStream_t st);
+                     float* score, float* score2, cudaStream_t st);
 int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld, int64_t n_heads,
                             int64_t head_dim, void* out, int64_t ld_out, cudaStream_t st);
 // dst row i = src row map(i) for i < rows, rows of row_bytes bytes (a multiple of 16)

@@ -195,6 +195,8 @@ __global__ void __launch_bounds__(256)
                        const float* __restrict__ score, float beta, float* __restrict__ la,
                        float* __restrict__ lr, float* __restrict__ rew, float* __restrict__ lse_a,
                        float* __restrict__ lse_r, int* err) {
+  pdl_wait();
+  pdl_launch_dependents();
   const long long row = blockIdx.x * 8LL + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -257,11 +259,13 @@ int launch_lse_combine(const void* part_ref, const void* part_act, int64_t n_til
                        float* lse_a, float* lse_r, int* err, cudaStream_t stream) {
   const int64_t rows = S * L;
   if (rows == 0) return 0;
-  lse_combine_kernel<<<static_cast<unsigned>((rows + 7) / 8), 256, 0, stream>>>(
-      static_cast<const float2*>(part_ref), static_cast<const float2*>(part_act),
-      static_cast<int>(n_tiles), tgt_ref, tgt_act, rows, static_cast<int>(L), static_cast<int>(V),
-      ids, ids_ld, lengths, score, beta, la, lr, rew, lse_a, lse_r, err);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+  return launch_pdl(lse_combine_kernel, dim3(static_cast<unsigned>((rows + 7) / 8)), dim3(256), 0, stream,
+                    static_cast<const float2*>(part_ref), static_cast<const float2*>(part_act),
+                    static_cast<int>(n_tiles), tgt_ref, tgt_act, static_cast<long long>(rows),
+                    static_cast<int>(L), static_cast<int>(V), ids, static_cast<long long>(ids_ld), lengths,
+                    score, beta, la, lr, rew, lse_a, lse_r, err) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 int launch_token_logprobs_kl(const void* za, const void* zr, int bf16_logits, int64_t S, int64_t L,

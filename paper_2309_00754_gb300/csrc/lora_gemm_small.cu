@@ -25,10 +25,10 @@
 //    distributed shared memory. Two warps per TMEM lane quarter drain alternate 32-column chunks
 //    through small swizzled buffers into whole-line stores (the residual add as one fp32
 //    reduction per element in L2).
-//  * Dependent launch. W is frozen: the first ring of W boxes loads before the wait on the
+//  * Dependent launch. W is frozen: the first ring of W boxes moves into L2 before the wait on the
 //    preceding kernel. Where that kernel is this call's own lora_down (which waits for its
-//    predecessors before it lets this kernel start), x is final already and the whole main loop
-//    overlaps it; only u is waited for.
+//    predecessors before it lets this kernel start), x and W are final already and the whole main
+//    loop overlaps it; only u is waited for.
 //
 // What bounds it: HBM for W, and an SM's fill from L2 (64 B per clock: a k-block of 64 costs
 // 2 (seg + bn / 2) clocks of fill for 2 bn clocks of products), which is why the x boxes are as
@@ -467,7 +467,9 @@ __global__ void __launch_bounds__(NUM_THREADS)
     int it = 0, s = 0;
     uint32_t ph = 0;  // parity of the next wait on stage s: its previous use is done
     if (warp == 0) {
-      // W and B are frozen: nothing of them is waited for
+      // W and B are frozen, but a caller may have written them just before this call: they are in
+      // L2 by now, and read once everything before the call is final
+      if (!p.x_settled) pdl_wait();
       for (; it < items; ++it) {
         if (it >= pre && !warp_wait_bounded(empty_bar(s), ph, abort_flag, p.err, kDevTimeoutProducer))
           break;

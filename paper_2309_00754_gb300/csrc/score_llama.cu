@@ -346,7 +346,8 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
   // score, at the last valid token). Its q/k/v projection and attention run over every
   // position (the prompt's keys and values); from the o projection on it runs on those
   // Lc = L + 1 rows of each sequence, gathered into compact buffers: per row the same
-  // arithmetic, so the same bits.
+  // arithmetic, and the same bits where both row counts take the same kernel (the few-rows
+  // linear adds a sum's two halves of K apart).
   const int64_t Lc = L + 1, Tc = S * Lc;
   const bool compact = Lc < P;
   const hydra::RowMap pick{Lc, P, c.prompt_len - 1};  // compact row -> row of the full stream
@@ -469,7 +470,7 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
   // (position P0 + len - 1: compact row len of its sequence)
   HY_PROF(HYDRA_PROF_HEADS, hydra::launch_seq_score(hf, w->final_norm, w->w_rm, d, c.rms_eps,
                                                     lengths, S, L, compact ? Lc : P,
-                                                    compact ? 1 : c.prompt_len, sc, st));
+                                                    compact ? 1 : c.prompt_len, sc, score, st));
   // values from the last stream: the on stream (J-Hydra) or the critic stream (Hydra-PPO)
   const void* fin_on = static_cast<uint8_t*>(fin) + static_cast<size_t>(ns - 1) * SL * d * 2;
   const hydra::RowMap dense{SL, SL, 0};
@@ -480,9 +481,6 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
                                     nullptr, nullptr, err, st));
   HY_PROF(HYDRA_PROF_GAE, hydra::launch_gae(reward, values, lengths, S, L, c.gamma, c.lam,
                                             advantages, returns, err, st));
-  if (cudaMemcpyAsync(score, sc, static_cast<size_t>(S) * 4, cudaMemcpyDeviceToDevice, st) !=
-      cudaSuccess)
-    return HYDRA_ERR_CUDA;
 #undef HY_TRY
 #undef HY_PROF
   return HYDRA_OK;
