@@ -1,4 +1,4 @@
-// The dual-output LoRA linear (see lora_gemm_tc.cu for the mathematics) for up to 384 token rows
+// The dual-output LoRA linear (see lora_gemm_tc.cu for the mathematics) for up to 448 token rows
 // per stream: one short sequence, a prompt, a decode batch. The work there is reading W once, and
 // the tile kernel of lora_gemm_tc.cu leaves most of the chip idle: 97 rows of two streams by 4096
 // columns are 32 tiles of 128 x 256, each with the whole of K, on 152 SMs.
@@ -16,15 +16,16 @@
 //    slower: only 15 clusters of eight CTAs fit on the chip, 36 of four.)
 //  * Ring items are two k-blocks of 64, and x and W have a TMA warp each. What a warp executes
 //    per item is the limit at these sizes: one warp and 64-wide items took 570 clocks each, more
-//    than the products of a tile (97 x 4096 x 12288: 44.8 us, now 26.5).
+//    than the products of a tile (97 x 4096 x 12288: 44.8 us, then 26.5).
 //  * LoRA. The k-blocks of u B^T go to the last K slice and accumulate in TMEM columns of their
 //    own; y_on's partial sum there is main + lora. No drain waits for them, and a pair with an
 //    off segment never mixes B into the off rows (their part of that accumulator is not read).
 //  * Reduction and epilogue. Each of two K slices finishes half of the tile's columns: it takes
 //    the other slice's fp32 sums of those columns, pushed into its drained ring through
-//    distributed shared memory. Two warps per TMEM lane quarter drain alternate 32-column chunks
-//    through small swizzled buffers into whole-line stores (the residual add as one fp32
-//    reduction per element in L2).
+//    distributed shared memory. Once the products are done all twelve warps drain, three per
+//    TMEM lane quarter, a chunk of 32 columns each (paired tiles: 16 of each half) through small
+//    swizzled buffers into whole-line stores (the residual add as one fp32 reduction per element
+//    in L2).
 //  * Dependent launch. W is frozen: the first ring of W boxes moves into L2 before the wait on the
 //    preceding kernel. Where that kernel is this call's own lora_down (which waits for its
 //    predecessors before it lets this kernel start), x and W are final already and the whole main
@@ -33,7 +34,7 @@
 // What bounds it: HBM for W, and an SM's fill from L2 (64 B per clock: a k-block of 64 costs
 // 2 (seg + bn / 2) clocks of fill for 2 bn clocks of products), which is why the x boxes are as
 // high as the segment and not 128 rows. 97 rows x 4096 x 12288 (two streams): the main loop runs
-// at 6.6 TB/s of W; about 6 us of the 26.5 are set-up, first loads, drain and stores.
+// at 6.6 TB/s of W; about 6 us of the 25.6 are set-up, first loads, drain and stores.
 #include <float.h>
 
 #include <mutex>
@@ -46,14 +47,19 @@ namespace hydra {
 namespace smallm {
 
 constexpr int BK = 128;  // a ring item: two k-blocks of 64 (128-byte swizzle each)
-// warp 0: TMA of W; 1: TMEM and MMA; 2: TMA of x; 3: barriers, L2 prefetch; 4-11: drain (two warps
-// per quarter of the TMEM lanes, alternate column chunks each)
+// warp 0: TMA of W; 1: TMEM and MMA; 2: TMA of x; 3: barriers, L2 prefetch; all of them: drain
 constexpr int NUM_THREADS = 384;
 constexpr int kMaxStages = 12;
 constexpr int kSmemMax = 232448;  // dynamic shared memory of one CTA (227 KiB)
 constexpr int kBarBytes = (2 * kMaxStages + 1) * 8 + 16;
 
-enum { EPI_STORE = 0, EPI_SWIGLU = 1, EPI_RESIDUAL = 2, EPI_ROPE = 3, EPI_LOGSOFTMAX = 4 };
+// Epilogues. The kernel is compiled for each: a launch then fetches about 40 KB of code and not its
+// parts of 82 KB (a 3-layer scoring pass of 97 rows 500 -> 495 us).
+enum { EPI_STORE = 0, EPI_SWIGLU = 1, EPI_RESIDUAL = 2, EPI_ROPE = 3, EPI_LOGSOFTMAX = 4, EPI_STORE_F32 = 5 };
+constexpr bool paired_epi(int epi) { return epi == EPI_SWIGLU || epi == EPI_ROPE; }
+// columns a drain warp takes at a time; of a paired tile, as many of each half
+constexpr int chunk_of(int epi) { return paired_epi(epi) ? 16 : 32; }
+constexpr int kMaxBoxes = 5;  // W boxes of a CTA and k-block
 
 struct Maps {
   CUtensorMap x[3];
@@ -69,8 +75,6 @@ struct Params {
   int bn, ks, stages;
   int shared_x, both;   // both: shared input with LoRA and both outputs wanted
   int has_on, has_crit;
-  int epi, out_f32;
-  int paired;    // SwiGLU / rotary: tile columns [0, bn/2) and [bn/2, bn) are partner columns
   int b_box;     // rows of a W / B box
   int x_settled; // x is final before the preceding kernel of the stream ends
   int lcol;      // TMEM column of the LoRA accumulator
@@ -109,12 +113,13 @@ __device__ __forceinline__ float bf16_round(float v) {
   return __bfloat162float(__float2bfloat16_rn(v));
 }
 
-// W row of the tile's B row j of CTA half `half`, whose first row is `first` (a pair index for
-// the paired layouts): SwiGLU gate / up blocks of 128 rows, rotary halves of 64 rows of a head
+// W row of the tile's B row j of CTA half `half`. In the paired layouts tile columns [0, bn/2) and
+// [bn/2, bn) are partners: SwiGLU gate / up blocks of 128 rows, rotary halves of 64 rows of a head.
+template <int kEpi>
 __device__ __forceinline__ int b_row(const Params& p, int n0, int half, int j) {
-  if (!p.paired) return n0 + half * (p.bn / 2) + j;
+  if (!paired_epi(kEpi)) return n0 + half * (p.bn / 2) + j;
   const int q = n0 / 2 + j;
-  return p.epi == EPI_SWIGLU ? (q >> 7) * 256 + half * 128 + (q & 127)
+  return kEpi == EPI_SWIGLU ? (q >> 7) * 256 + half * 128 + (q & 127)
                              : (q >> 6) * 128 + half * 64 + (q & 63);
 }
 
@@ -123,7 +128,10 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
                     pack_bf16x2(v[6], v[7]));
 }
 
-// An epilogue thread's accumulator row: its sums, 32 tile columns at a time.
+__device__ __forceinline__ void ld_cols(uint32_t taddr, uint32_t (&v)[32]) { tc_ld_32x32b_x32(taddr, v); }
+__device__ __forceinline__ void ld_cols(uint32_t taddr, uint32_t (&v)[16]) { tc_ld_32x32b_x16(taddr, v); }
+
+// An epilogue thread's accumulator row: its sums, a chunk of tile columns at a time.
 struct RowSums {
   uint32_t taddr;  // TMEM address of the thread's lane, column 0 of the main accumulator
   int lcol;        // columns from there to the LoRA accumulator
@@ -132,26 +140,27 @@ struct RowSums {
   int lplane;      // float4 from there to the LoRA sums sent along (shared input, slice 0), or 0
   int row;         // row of the tile (TMEM lane)
 
-  // v = the sums of columns [c, c + 32), the LoRA term included or not; pos: index of the chunk
+  // v = the sums of columns [c, c + n), the LoRA term included or not; pos: index of the chunk
   // among those this CTA finishes. LoRA joins the last slice's sum before the slices are added.
-  __device__ __forceinline__ void get(int c, int pos, bool lora, float (&v)[32]) const {
-    uint32_t a[32];
-    tc_ld_32x32b_x32(taddr + c, a);
+  template <int n>
+  __device__ __forceinline__ void get(int c, int pos, bool lora, float (&v)[n]) const {
+    uint32_t a[n];
+    ld_cols(taddr + c, a);
     if (lora && own_lora) {
-      uint32_t l[32];
-      tc_ld_32x32b_x32(taddr + lcol + c, l);
+      uint32_t l[n];
+      ld_cols(taddr + lcol + c, l);
       tc_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(l[i]);
+      for (int i = 0; i < n; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(l[i]);
     } else {
       tc_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(a[i]);
+      for (int i = 0; i < n; ++i) v[i] = __uint_as_float(a[i]);
     }
     if (recv == nullptr) return;
-    const float4* s = recv + pos * 8 * 128 + row;
+    const float4* s = recv + pos * (n / 4) * 128 + row;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < n / 4; ++j) {
       float4 t = s[j * 128];
       if (lora && lplane != 0) {
         const float4 l = s[lplane + j * 128];
@@ -195,11 +204,12 @@ struct Staging {
 
 // Store 32 sums of the thread's row at output columns [n, n + 32) (N % 8 == 0). `y` is the row of
 // the warp's lane 0.
+template <int kEpi>
 __device__ __forceinline__ void store32(const Params& p, const Staging& st, void* y, int n,
                                         const float (&v)[32]) {
   const int left = p.N - n;
-  if (p.epi == EPI_RESIDUAL || p.out_f32) {
-    const bool add = p.epi == EPI_RESIDUAL;
+  if constexpr (kEpi == EPI_RESIDUAL || kEpi == EPI_STORE_F32) {
+    constexpr bool add = kEpi == EPI_RESIDUAL;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float* w = v + 4 * j;
@@ -210,75 +220,78 @@ __device__ __forceinline__ void store32(const Params& p, const Staging& st, void
     }
     uint8_t* d = reinterpret_cast<uint8_t*>(static_cast<float*>(y) + n);
     const size_t ld = static_cast<size_t>(p.N) * 4;
-    if (add) st.flush<8, true>(d, ld, left / 4);
-    else st.flush<8, false>(d, ld, left / 4);
-    return;
-  }
+    st.flush<8, add>(d, ld, left / 4);
+  } else {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) st.put(j, pack8(v + 8 * j));
-  st.flush<4, false>(reinterpret_cast<uint8_t*>(static_cast<__nv_bfloat16*>(y) + n),
-                     static_cast<size_t>(p.N) * 2, left / 8);
+    for (int j = 0; j < 4; ++j) st.put(j, pack8(v + 8 * j));
+    st.flush<4, false>(reinterpret_cast<uint8_t*>(static_cast<__nv_bfloat16*>(y) + n),
+                       static_cast<size_t>(p.N) * 2, left / 8);
+  }
 }
 
-// 32 partner columns of a paired tile: q is the first one's pair index, v / z the sums of the
+__device__ __forceinline__ void swiglu2(uint32_t& g, uint32_t u) {
+  const float2 a = unpack_bf16x2(g), b = unpack_bf16x2(u);
+  g = pack_bf16x2(silu(a.x) * b.x, silu(a.y) * b.y);
+}
+
+// 16 partner columns of a paired tile: q is the first one's pair index, v / z the sums of the
 // first and the second half; row: the thread's row, y: the output's first element
-__device__ __forceinline__ void store_pair32(const Params& p, const Staging& st, void* y, int row,
-                                             int q, float (&v)[32], float (&z)[32]) {
+template <int kEpi>
+__device__ __forceinline__ void store_pair16(const Params& p, const Staging& st, void* y, int row,
+                                             int q, float (&v)[16], float (&z)[16]) {
   __nv_bfloat16* out = static_cast<__nv_bfloat16*>(y);
   const size_t row0 = static_cast<size_t>(row - st.lane);
-  if (p.epi == EPI_SWIGLU) {
-    if (q >= p.N / 2) return;  // N % 256 == 0: 32 pairs are all in or all out
-    // the bf16 gates and ups through the staging buffer, and a short loop from there: unrolled
-    // over 32 registers, the quotients are 30 KB of code that every launch fetches anew (6 us
-    // of a 53 us launch)
+  if constexpr (kEpi == EPI_SWIGLU) {
+    if (q >= p.N / 2) return;  // N % 256 == 0: 16 pairs are all in or all out
+    // the bf16 gates and ups through the staging buffer, and a short loop from there, eight
+    // features a lane: unrolled over the registers, the quotients are 30 KB of code that every
+    // launch fetches anew, and with the division operator they follow one another (13000 clocks
+    // of drain per tile, now 5800; 97 rows x 4096 x 22016: 53.3 -> 47.8 us by this loop and
+    // silu(), 45.3 by three drain warps per quarter in place of two, 43.9 by 160-column tiles)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < 2; ++j) {
       st.put(j, pack8(v + 8 * j));
-      st.put(4 + j, pack8(z + 8 * j));
+      st.put(2 + j, pack8(z + 8 * j));
     }
     __syncwarp();
+    const int c = st.lane & 1;
 #pragma unroll 1
-    for (int i = 0; i < 4; ++i) {
-      const int e = i * 32 + st.lane, r = e >> 2, c = e & 3;
-      if (r < st.rows) {
-        const uint4 g4 = st.buf[r * 8 + (c ^ (r & 7))], u4 = st.buf[r * 8 + ((4 + c) ^ (r & 7))];
-        uint4 o;
-        const uint32_t *gp = &g4.x, *up = &u4.x;
-        uint32_t* op = &o.x;
+    for (int r = st.lane >> 1; r < 32; r += 16) {
+      if (r >= st.rows) break;
+      uint4 g = st.buf[r * 8 + (c ^ (r & 7))];
+      const uint4 u = st.buf[r * 8 + ((2 + c) ^ (r & 7))];
+      swiglu2(g.x, u.x);
+      swiglu2(g.y, u.y);
+      swiglu2(g.z, u.z);
+      swiglu2(g.w, u.w);
+      *reinterpret_cast<uint4*>(out + (row0 + r) * (p.N / 2) + q + 8 * c) = g;
+    }
+    __syncwarp();
+  } else {
+    // rotary: the roundings of hydra_rope on the bf16-rounded sums
+    const int i0 = q & 63, na = (q >> 6) * 128 + i0;
+    if (na < p.rope_cols) {  // whole heads: rope_cols % 128 == 0
+      const float4* cs = reinterpret_cast<const float4*>(p.rope_table + (row % p.rope_P) * 64 + i0);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float2 g = unpack_bf16x2(gp[k]), u = unpack_bf16x2(up[k]);
-          op[k] = pack_bf16x2(g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y);
-        }
-        *reinterpret_cast<uint4*>(out + (row0 + r) * (p.N / 2) + q + 8 * c) = o;
+      for (int i = 0; i < 8; ++i) {
+        const float4 t = __ldg(cs + i);
+        const float a0 = bf16_round(v[2 * i]), a1 = bf16_round(v[2 * i + 1]);
+        const float b0 = bf16_round(z[2 * i]), b1 = bf16_round(z[2 * i + 1]);
+        v[2 * i] = __fsub_rn(__fmul_rn(a0, t.x), __fmul_rn(b0, t.y));
+        v[2 * i + 1] = __fsub_rn(__fmul_rn(a1, t.z), __fmul_rn(b1, t.w));
+        z[2 * i] = __fadd_rn(__fmul_rn(a0, t.y), __fmul_rn(b0, t.x));
+        z[2 * i + 1] = __fadd_rn(__fmul_rn(a1, t.w), __fmul_rn(b1, t.z));
       }
     }
-    __syncwarp();
-    return;
+    uint8_t* o = reinterpret_cast<uint8_t*>(out + row0 * p.N + na);
+    const size_t ld = static_cast<size_t>(p.N) * 2;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) st.put(j, pack8(v + 8 * j));
+    st.flush<2, false>(o, ld, (p.N - na) / 8);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) st.put(j, pack8(z + 8 * j));
+    st.flush<2, false>(o + 128, ld, (p.N - na - 64) / 8);
   }
-  // rotary: the roundings of hydra_rope on the bf16-rounded sums
-  const int i0 = q & 63, na = (q >> 6) * 128 + i0;
-  if (na < p.rope_cols) {  // whole heads: rope_cols % 128 == 0
-    const float4* cs = reinterpret_cast<const float4*>(p.rope_table + (row % p.rope_P) * 64 + i0);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float4 t = __ldg(cs + i);
-      const float a0 = bf16_round(v[2 * i]), a1 = bf16_round(v[2 * i + 1]);
-      const float b0 = bf16_round(z[2 * i]), b1 = bf16_round(z[2 * i + 1]);
-      v[2 * i] = __fsub_rn(__fmul_rn(a0, t.x), __fmul_rn(b0, t.y));
-      v[2 * i + 1] = __fsub_rn(__fmul_rn(a1, t.z), __fmul_rn(b1, t.w));
-      z[2 * i] = __fadd_rn(__fmul_rn(a0, t.y), __fmul_rn(b0, t.x));
-      z[2 * i + 1] = __fadd_rn(__fmul_rn(a1, t.w), __fmul_rn(b1, t.z));
-    }
-  }
-  uint8_t* o = reinterpret_cast<uint8_t*>(out + row0 * p.N + na);
-  const size_t ld = static_cast<size_t>(p.N) * 2;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) st.put(j, pack8(v + 8 * j));
-  st.flush<4, false>(o, ld, (p.N - na) / 8);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) st.put(j, pack8(z + 8 * j));
-  st.flush<4, false>(o + 128, ld, (p.N - na - 64) / 8);
 }
 
 // Log-softmax partials of the thread's row over a tile of 256 columns: the online (max, sum of
@@ -330,6 +343,7 @@ __device__ __forceinline__ void emit_lsm(const Params& p, const RowSums& r, int 
   asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");  // the buffer serves the next output
 }
 
+template <int kEpi>
 __global__ void __launch_bounds__(NUM_THREADS)
     lora_gemm_small_kernel(const __grid_constant__ Maps mp, const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
@@ -411,10 +425,10 @@ __global__ void __launch_bounds__(NUM_THREADS)
   auto lora_kbs = [&](int i) { return p.r - i * BK > 64 ? 2 : 1; };
 
   // before the barrier ends: descriptors, and this CTA's first W boxes into L2 (W is frozen)
-  const int nbox = p.bn / 2 / p.b_box;  // at most 4
-  int brow[4];                          // W rows of the boxes
+  const int nbox = p.bn / 2 / p.b_box;
+  int brow[kMaxBoxes];                          // W rows of the boxes
 #pragma unroll
-  for (int j = 0; j < 4; ++j) brow[j] = b_row(p, n0, half, j * p.b_box);
+  for (int j = 0; j < kMaxBoxes; ++j) brow[j] = b_row<kEpi>(p, n0, half, j * p.b_box);
   if (warp == 0 && elect_one()) {
     tma_prefetch_desc(&mp.w);
     if (lora0 || lora1) tma_prefetch_desc(&mp.b[lset]);
@@ -426,7 +440,7 @@ __global__ void __launch_bounds__(NUM_THREADS)
   if (warp == 3 && elect_one()) {
     for (int i = 0; i < min(n_main, p.stages); ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < kMaxBoxes; ++j)
         if (j < nbox) {
           prefetch_box(&mp.w, (kb0 + i) * BK, brow[j]);
           prefetch_box(&mp.w, (kb0 + i) * BK + 64, brow[j]);
@@ -438,7 +452,14 @@ __global__ void __launch_bounds__(NUM_THREADS)
   tc_fence_after();
   const uint32_t tmem_acc = *tmem_slot;
 
-  bool epi_ok = false;
+  // The dependent kernel may start once every CTA has said so. After a plain linear that is the next
+  // call's lora_down: let in at once, it waits on the SMs that this grid leaves free, and the SMs
+  // of this grid are the next linear's (let in after the products, it spread over them and held
+  // that linear up in most runs: 300 rows, shared, 22.6 us a call, now 17.9). After the fused
+  // epilogues of a pass come row kernels, whose early CTAs take what the last tiles need (a
+  // 97-row scoring pass 457 us, let in at once 465).
+  constexpr bool kEarly = kEpi == EPI_STORE || kEpi == EPI_STORE_F32;
+  if (kEarly) pdl_launch_dependents();
   if (warp == 0 || warp == 2) {
     // ------------------------------------------------------------------ TMA producers: warp 0
     // moves W (and B), warp 2 x (and u). Everything an item needs is a running value, an item is
@@ -454,12 +475,12 @@ __global__ void __launch_bounds__(NUM_THREADS)
       const int k = i * BK;
       uint32_t dst = stage + 2 * a_bytes;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < kMaxBoxes; ++j)
         if (j < nbox) tma_load_2d_pair(dst + j * box_bytes, m, k, brow[j], bar);
       if (kbs == 2) {
         dst += b_bytes;
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < kMaxBoxes; ++j)
           if (j < nbox) tma_load_2d_pair(dst + j * box_bytes, m, k + 64, brow[j], bar);
       }
     };
@@ -551,27 +572,29 @@ __global__ void __launch_bounds__(NUM_THREADS)
     }
     volatile int no_abort = 0;
     warp_wait_bounded(acc_full, 0, &no_abort, p.err, kDevTimeoutDrain);
-  } else if (warp >= 4) {
-    // -------------------------------------------------------------------- drain
-    epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
-    epi_ok = __all_sync(0xffffffffu, epi_ok) && *abort_flag == 0;
-    tc_fence_after();
   }
-  pdl_launch_dependents();
+  // ---------------------------------------------------------------------- drain: every warp,
+  // three per quarter of the TMEM lanes (log-softmax: the two that meet at its barriers)
+  constexpr int kDrainers = kEpi == EPI_LOGSOFTMAX ? 2 : 3;
+  bool epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
+  epi_ok = __all_sync(0xffffffffu, epi_ok) && *abort_flag == 0;
+  tc_fence_after();
+  if (!kEarly) pdl_launch_dependents();
 
   const int q = warp & 3;             // TMEM lanes 32 q .. of a drain warp
   const int trow = q * 32 + lane;     // row of the segment
-  const int par = (warp >> 2) & 1;    // which of the two warps of its lanes
-  const bool drain = warp >= 4 && epi_ok && q * 32 < nrow;
+  const int par = kDrainers == 3 ? warp >> 2 : (warp >> 2) - 1;  // which of the warps of its lanes
+  const bool drain = par >= 0 && epi_ok && q * 32 < nrow;
   const bool last = slice == p.ks - 1;
-  const int nch = p.bn / 32;          // column chunks of the tile
+  constexpr int kChunk = chunk_of(kEpi);
+  const int nch = p.bn / kChunk;      // column chunks of the tile
   // the slice that finishes chunk i (two slices: halves of the columns, or of the pairs), and
   // the chunk's index among those it finishes
   auto owner = [&](int i) {
-    return p.ks == 1 ? 0 : (p.paired ? (i % (nch / 2)) / (nch / 4) : i / (nch / 2));
+    return p.ks == 1 ? 0 : (paired_epi(kEpi) ? (i % (nch / 2)) / (nch / 4) : i / (nch / 2));
   };
   auto pos_of = [&](int i) {
-    return p.ks == 1 ? 0 : (p.paired ? i % (nch / 4) + (i / (nch / 2)) * (nch / 4) : i % (nch / 2));
+    return p.ks == 1 ? 0 : (paired_epi(kEpi) ? i % (nch / 4) + (i / (nch / 2)) * (nch / 4) : i % (nch / 2));
   };
   RowSums rs;
   rs.taddr = tmem_acc + (static_cast<uint32_t>(q * 32) << 16);
@@ -581,28 +604,28 @@ __global__ void __launch_bounds__(NUM_THREADS)
   rs.recv = nullptr;
   rs.lplane = 0;
   if (p.ks == 2) {
-    const int plane = nch / 2 * 8 * 128;  // float4 of one slice's sums
+    const int plane = p.bn / 2 / 4 * 128;  // float4 of one slice's sums
     float4* xch = reinterpret_cast<float4*>(smem);
     cluster_sync_all();  // both slices' products are done: the rings are free
     if (drain) {
       const uint32_t dst0 = map_to_rank(smem_u32(xch + trow), static_cast<uint32_t>(2 * (1 - slice) + half));
-      for (int i = 0; i < nch; ++i) {
-        if (owner(i) == slice || (i & 1) != par) continue;
-        uint32_t v[32], l[32];
-        tc_ld_32x32b_x32(rs.taddr + 32 * i, v);
-        if (rs.own_lora) tc_ld_32x32b_x32(rs.taddr + p.lcol + 32 * i, l);
+      for (int i = par; i < nch; i += kDrainers) {
+        if (owner(i) == slice) continue;
+        uint32_t v[kChunk], l[kChunk];
+        ld_cols(rs.taddr + kChunk * i, v);
+        if (rs.own_lora) ld_cols(rs.taddr + p.lcol + kChunk * i, l);
         tc_wait_ld();
         if (rs.own_lora && !p.both) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(l[j]));
+          for (int j = 0; j < kChunk; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(l[j]));
         }
-        const uint32_t dst = dst0 + pos_of(i) * (8 * 128 * 16);
+        const uint32_t dst = dst0 + pos_of(i) * (kChunk / 4 * 128 * 16);
         if (trow < nrow) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) st_cluster_f4(dst + j * 2048, v + 4 * j);
+          for (int j = 0; j < kChunk / 4; ++j) st_cluster_f4(dst + j * 2048, v + 4 * j);
           if (rs.own_lora && p.both) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) st_cluster_f4(dst + plane * 16 + j * 2048, l + 4 * j);
+            for (int j = 0; j < kChunk / 4; ++j) st_cluster_f4(dst + plane * 16 + j * 2048, l + 4 * j);
           }
         }
       }
@@ -617,9 +640,9 @@ __global__ void __launch_bounds__(NUM_THREADS)
     pdl_wait();  // outputs are written only after the preceding kernel
     const bool live = trow < nrow;
     const int row = m0 + trow;
-    const Staging st{reinterpret_cast<uint4*>(smem + p.stg_off) + (warp - 4) * 256, lane, nrow - q * 32};
+    const Staging st{reinterpret_cast<uint4*>(smem + p.stg_off) + warp * 256, lane, nrow - q * 32};
     const size_t warp_row = static_cast<size_t>(m0 + q * 32);
-    const size_t elem = p.out_f32 || p.epi == EPI_RESIDUAL ? 4 : 2;
+    constexpr size_t elem = kEpi == EPI_STORE_F32 || kEpi == EPI_RESIDUAL ? 4 : 2;
     for (int o = 0; o < 2; ++o) {
       void* y;
       bool lora;
@@ -631,24 +654,24 @@ __global__ void __launch_bounds__(NUM_THREADS)
         lora = true;
       }
       if (y == nullptr) continue;
-      if (p.epi == EPI_LOGSOFTMAX) {
+      if constexpr (kEpi == EPI_LOGSOFTMAX) {
         emit_lsm(p, rs, row, live, n0, static_cast<float2*>(y),
                  p.lsm_target + ((p.shared_x ? o : stream) == 0 ? 0 : p.M), lora, par, q,
                  reinterpret_cast<float2*>(smem + p.stg_off) + q * 32);
-      } else if (!p.paired) {
-        for (int i = 0; i < nch; ++i) {
-          if (owner(i) != slice || (i & 1) != par || n0 + 32 * i >= p.N) continue;
+      } else if constexpr (!paired_epi(kEpi)) {
+        for (int i = par; i < nch; i += kDrainers) {
+          if (owner(i) != slice || n0 + 32 * i >= p.N) continue;
           float v[32];
           rs.get(32 * i, pos_of(i), lora, v);
-          store32(p, st, static_cast<uint8_t*>(y) + warp_row * p.N * elem, n0 + 32 * i, v);
+          store32<kEpi>(p, st, static_cast<uint8_t*>(y) + warp_row * p.N * elem, n0 + 32 * i, v);
         }
       } else {
-        for (int i = 0; i < nch / 2; ++i) {
-          if (owner(i) != slice || (i & 1) != par) continue;
-          float v[32], z[32];
-          rs.get(32 * i, pos_of(i), lora, v);
-          rs.get(32 * (i + nch / 2), pos_of(i + nch / 2), lora, z);
-          store_pair32(p, st, y, row, n0 / 2 + 32 * i, v, z);
+        for (int i = par; i < nch / 2; i += kDrainers) {
+          if (owner(i) != slice) continue;
+          float v[kChunk], z[kChunk];
+          rs.get(kChunk * i, pos_of(i), lora, v);
+          rs.get(kChunk * (i + nch / 2), pos_of(i + nch / 2), lora, z);
+          store_pair16<kEpi>(p, st, y, row, n0 / 2 + kChunk * i, v, z);
         }
       }
     }
@@ -703,7 +726,7 @@ bool lay_out(const Shape& s, int bn, Config* c) {
   int ring = st * stage;
   const int last = (st - 1) * stage + s.seg * 128 + 16384;
   if (last > ring) ring = last;
-  const int over = xch + 8 * 4096;  // exchange buffer and the drain warps' staging, over the ring
+  const int over = xch + smallm::NUM_THREADS / 32 * 4096;  // exchange buffer and the drain warps' staging, over the ring
   const int end = ((ring > over ? ring : over) + 15) / 16 * 16;
   if (end + 1024 + kBarBytes > kSmemMax) return false;
   c->bn = bn;
@@ -714,7 +737,20 @@ bool lay_out(const Shape& s, int bn, Config* c) {
   return true;
 }
 
-// Clusters of 2 ks CTAs with this shared memory that the device holds at once.
+using Kernel = void (*)(smallm::Maps, smallm::Params);
+Kernel kernel_of(int epi) {
+  switch (epi) {
+    case smallm::EPI_SWIGLU: return smallm::lora_gemm_small_kernel<smallm::EPI_SWIGLU>;
+    case smallm::EPI_RESIDUAL: return smallm::lora_gemm_small_kernel<smallm::EPI_RESIDUAL>;
+    case smallm::EPI_ROPE: return smallm::lora_gemm_small_kernel<smallm::EPI_ROPE>;
+    case smallm::EPI_LOGSOFTMAX: return smallm::lora_gemm_small_kernel<smallm::EPI_LOGSOFTMAX>;
+    case smallm::EPI_STORE_F32: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE_F32>;
+    default: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE>;
+  }
+}
+
+// Clusters of 2 ks CTAs with this shared memory that the device holds at once (the same for every
+// epilogue: shared memory and threads decide).
 int resident_clusters(int dev, int ks, int smem) {
   static std::mutex mu;
   static std::vector<std::pair<long long, int>> cache;
@@ -734,7 +770,7 @@ int resident_clusters(int dev, int ks, int smem) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel<smallm::EPI_STORE>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -747,7 +783,7 @@ int resident_clusters(int dev, int ks, int smem) {
 // Sizes alone decide, not streams or epilogue: the sums of one (M, K, N) have one order. Above
 // 128 rows the tile kernel of lora_gemm_tc.cu takes over where its 256-column tiles fill the chip
 // (measured on GB300, us, this kernel / that one; rows x K x N, two streams): 97 x 4096 x 4096
-// 13.0 / 30.4, x 12288 26.5 / 35.3, x 22016 51.1 / 80.3; 97 x 11008 x 4096 23.7 / 69.3;
+// 12.3 / 30.4, x 12288 25.6 / 35.3, x 22016 43.9 / 80.3; 97 x 11008 x 4096 22.5 / 69.3;
 // 200 x 4096 x 11008 36.8 / 39.0, x 12288 46.9 / 44.9, x 16384 47.0 / 44.0; 300 x 4096 x 4096
 // 19.5 / 23.5 (shared input 16.0 / 24.0), x 12288 58.0 / 61.9, x 22016 110 / 103;
 // 384 x 4096 x 11008 49.2 / 57.1; 448 x 4096 x 4096 23.9 / 24.7, x 12288 81.8 / 63.0.
@@ -762,9 +798,9 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   static bool attr_set[64] = {false};
   if (!attr_set[dev]) {
-    if (cudaFuncSetAttribute(lora_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSmemMax) != cudaSuccess)
-      return -1;
+    for (int e = EPI_STORE; e <= EPI_STORE_F32; ++e)
+      if (cudaFuncSetAttribute(kernel_of(e), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
+        return -1;
     attr_set[dev] = true;
   }
   const bool tri = a.x_crit != nullptr && !a.shared_x;
@@ -786,6 +822,8 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   s.paired = a.epi == EPI_SWIGLU || a.epi == EPI_ROPE;
   const int npair = a.epi == EPI_SWIGLU ? N / 2 : (N + 127) / 128 * 64;
 
+  const int box = a.epi == EPI_SWIGLU ? 128 : 64;  // partner rows of W that are neighbours
+
   // Tile width: the fewest clocks over the waves. A k-block of 64 costs the pair its products
   // (2 bn) or a CTA's fill from L2 at 64 B per clock (2 (seg + bn / 2)), and a wave about 6000
   // clocks of set-up, first loads and drain.
@@ -795,7 +833,8 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
     return s.row_tiles * (s.paired ? (npair + bn / 2 - 1) / (bn / 2) : (N + bn - 1) / bn);
   };
   for (int bn : {256, 224, 192, 160, 128, 96, 64}) {
-    if ((s.paired && bn % (64 * s.ks) != 0) || (s.ks == 2 && bn % 64 != 0)) continue;
+    if (s.ks == 2 && bn % (s.paired ? 128 : 64) != 0) continue;  // whole chunks for each slice
+    if (s.paired && bn / 2 / gcd(bn / 2, box) > kMaxBoxes) continue;
     if (a.epi == EPI_LOGSOFTMAX && bn != 256) continue;
     Config c{};
     if (!lay_out(s, bn, &c)) continue;
@@ -814,7 +853,7 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   const int bn = best.bn;
 
   Params p{};
-  p.b_box = s.paired ? gcd(bn / 2, a.epi == EPI_SWIGLU ? 128 : 64) : bn / 2;
+  p.b_box = s.paired ? gcd(bn / 2, box) : bn / 2;
   Maps mp;
   const void* xs[3] = {a.x_off, a.shared_x ? a.x_off : a.x_on, a.x_crit};
   for (int i = 0; i < 3; ++i) {
@@ -847,9 +886,6 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   p.both = s.both ? 1 : 0;
   p.has_on = lora_on ? 1 : 0;
   p.has_crit = lora_crit ? 1 : 0;
-  p.epi = a.epi;
-  p.out_f32 = a.out_f32;
-  p.paired = s.paired ? 1 : 0;
   p.x_settled = a.x_settled ? 1 : 0;
   p.lcol = pow2_at_least(bn);
   p.tmem_cols = static_cast<uint32_t>(s.lora ? 2 * p.lcol : p.lcol);
@@ -885,7 +921,8 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, lora_gemm_small_kernel, mp, p) == cudaSuccess ? 0 : -3;
+  const int epi = a.epi == EPI_STORE && a.out_f32 ? EPI_STORE_F32 : a.epi;
+  return cudaLaunchKernelEx(&cfg, kernel_of(epi), mp, p) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace hydra

@@ -68,10 +68,11 @@ def test_few_rows_against_oracle_and_one_order_of_sums(M, K, N, r, f32):
 
 
 @pytest.mark.parametrize("M,N,shared", [(33, 512, False), (97, 512, True), (128, 768, False), (200, 392, False),
-                                        (300, 392, True)])
+                                        (300, 392, True), (97, 22016, False), (7, 22016, True)])
 def test_few_rows_fused_epilogues(M, N, shared):
     """SwiGLU, rotary (N past the rotated columns, a partial last head) and residual epilogues
-    equal the plain linear followed by the separate kernel, bit for bit (two K slices)."""
+    equal the plain linear followed by the separate kernel, bit for bit (two K slices; at 22016
+    columns one, and 160-column tiles of five boxes)."""
     K, r, P = 1032, 16, 50
     x, W, ab = _problem(M, K, N, r, seed=7 * M + N)
     d, dW, dB = [dev_bf16(t) for t in x], dev_bf16(W), dev_bf16(ab[0][1])
@@ -102,6 +103,27 @@ def test_few_rows_fused_epilogues(M, N, shared):
         H.hydra_rope(lin[i], d_rot, 128, P, 10000.0)
         assert torch.equal(got[i], lin[i])
     assert H.device_error(clear=True) == 0
+
+
+def test_fused_silu_has_the_operators_bits_for_every_bf16_gate():
+    """W's first column is every bf16 value (infinities, NaN and both zeros among them) and x picks
+    it out: the epilogue's branch-free quotient against hydra_swiglu's division operator."""
+    F, K, M = 65536, 8, 3
+    gate = torch.arange(F, device="cuda", dtype=torch.int32).to(torch.int16).view(torch.bfloat16)
+    W = torch.zeros(F // 128, 2, 128, K, dtype=torch.bfloat16, device="cuda")
+    W[:, 0, :, 0] = gate.view(-1, 128)
+    W[:, 1, :, 0] = 1.0
+    x = torch.zeros(M, K, dtype=torch.bfloat16, device="cuda")
+    x[:, 0] = 1.0
+    m = [torch.empty(M, F, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    H.hydra_dual_linear_ex(x, x, W.view(2 * F, K), None, None, m[0], m[1], H.EPI_SWIGLU)
+    # the tensor core's sum 1 * g + 0 keeps every g but -0, which it makes +0
+    g = torch.where(gate == 0, torch.zeros_like(gate), gate)
+    ref = torch.empty(1, F, dtype=torch.bfloat16, device="cuda")
+    H.hydra_swiglu(torch.cat([g, torch.ones_like(g)]).view(1, 2 * F), ref)
+    for y in m:
+        assert bool(((y == ref) | (y.isnan() & ref.isnan())).all())
+    assert int(ref.isnan().sum()) >= 254  # the NaN patterns, and -inf / inf
 
 
 def test_off_rows_ignore_a_non_finite_lora_factor():
