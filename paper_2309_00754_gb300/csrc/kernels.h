@@ -198,14 +198,16 @@ int launch_swiglu(const void* gu, int64_t R, int64_t F, void* m, cudaStream_t st
 int launch_residual_add(float* h, const void* y, int64_t n, cudaStream_t st);
 int launch_head_dot(const void* x, int64_t d, const void* w, const RowMap& map, int64_t n,
                     const int32_t* lengths, int64_t L, float* out, cudaStream_t st);
-int launch_seq_score(const float* h, const void* norm, const void* w, int64_t d, float eps,
-                     const int32_t* lengths, int64_t S, int64_t L, int64_t P, int64_t p0,
-                     float* score, float* score2, cudaStream_t st);
+// Sequence scores (score and score2) from h, and the values of the S L rows of x.
+int launch_score_heads(const float* h, const void* norm, const void* w, int64_t d, float eps,
+                       const int32_t* lengths, int64_t S, int64_t L, int64_t P, int64_t p0,
+                       float* score, float* score2, const void* x, float* values, cudaStream_t st);
 int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld, int64_t n_heads,
                             int64_t head_dim, void* out, int64_t ld_out, cudaStream_t st);
-// dst row i = src row map(i) for i < rows, rows of row_bytes bytes (a multiple of 16)
-int launch_gather_rows(const void* src, int64_t rows, int64_t row_bytes, const RowMap& map,
-                       void* dst, cudaStream_t st);
+// dst row i = src row map(i) for i < rows, rows of row_bytes bytes (a multiple of 16), and the
+// same rows of a second array
+int launch_gather_rows(const void* src, int64_t row_bytes, void* dst, const void* src2,
+                       int64_t row_bytes2, void* dst2, int64_t rows, const RowMap& map, cudaStream_t st);
 
 // Largest sequence length the shared-memory GAE scan accepts.
 constexpr int64_t kGaeMaxL = 16384;

@@ -212,15 +212,13 @@ __global__ void residual_add_kernel(float* __restrict__ h, const __nv_bfloat16* 
 
 // out[i] = sum_k x[map(i), k] w[k], one warp per output row (reward model / value head).
 // With `lengths`, rows are [S, L] (i = s L + t) and rows t >= lengths[s] are written 0.
-__global__ void head_dot_kernel(const __nv_bfloat16* __restrict__ x, int d,
-                                const __nv_bfloat16* __restrict__ w, RowMap map, long long n,
-                                const int32_t* __restrict__ lengths, int L,
-                                float* __restrict__ out) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const long long i = blockIdx.x * 8LL + (threadIdx.x >> 5);
+// Few rows are bound by the latency of their loads: eight in flight per lane and operand, summed
+// in column order (60 rows of 4096: 10.2 us a launch before).
+__device__ __forceinline__ void head_row(const __nv_bfloat16* __restrict__ x, int d,
+                                         const __nv_bfloat16* __restrict__ w, const RowMap& map,
+                                         long long i, const int32_t* __restrict__ lengths, int L,
+                                         float* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  if (i >= n) return;
   if (lengths != nullptr && (i % L) >= lengths[i / L]) {
     if (lane == 0) out[i] = 0.f;
     return;
@@ -228,8 +226,7 @@ __global__ void head_dot_kernel(const __nv_bfloat16* __restrict__ x, int d,
   const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(map_row(i, map)) * d);
   const uint4* wr = reinterpret_cast<const uint4*>(w);
   float acc = 0.f;
-  for (int c = lane; c < d / 8; c += 32) {
-    const uint4 a = __ldg(xr + c), b = __ldg(wr + c);
+  auto dot8 = [&](const uint4& a, const uint4& b) {
     const uint32_t* ap = &a.x;
     const uint32_t* bp = &b.x;
 #pragma unroll
@@ -238,9 +235,33 @@ __global__ void head_dot_kernel(const __nv_bfloat16* __restrict__ x, int d,
       acc = fmaf(fa.x, fb.x, acc);
       acc = fmaf(fa.y, fb.y, acc);
     }
+  };
+  constexpr int kAhead = 8;
+  const int n8 = d / 8;
+  int c = lane;
+  for (; c + 32 * (kAhead - 1) < n8; c += 32 * kAhead) {
+    uint4 a[kAhead], b[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      a[j] = __ldg(xr + c + 32 * j);
+      b[j] = __ldg(wr + c + 32 * j);
+    }
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) dot8(a[j], b[j]);
   }
+  for (; c < n8; c += 32) dot8(__ldg(xr + c), __ldg(wr + c));
   acc = warp_sum(acc);
   if (lane == 0) out[i] = acc;
+}
+
+__global__ void __launch_bounds__(256)
+    head_dot_kernel(const __nv_bfloat16* __restrict__ x, int d, const __nv_bfloat16* __restrict__ w,
+                    RowMap map, long long n, const int32_t* __restrict__ lengths, int L,
+                    float* __restrict__ out) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const long long i = blockIdx.x * 8LL + (threadIdx.x >> 5);
+  if (i < n) head_row(x, d, w, map, i, lengths, L, out);
 }
 
 // ---------------------------------------------------------------- sequence score
@@ -262,14 +283,12 @@ __device__ __forceinline__ float score_block_sum(float v, float* red) {
   return t;
 }
 
-__global__ void __launch_bounds__(kScoreThreads)
-    seq_score_kernel(const float* __restrict__ h, const __nv_bfloat16* __restrict__ g,
-                     const __nv_bfloat16* __restrict__ w, int d, float eps,
-                     const int32_t* __restrict__ lengths, int L, long long P, long long p0,
-                     float* __restrict__ score, float* __restrict__ score2) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int s = blockIdx.x;
+__device__ __forceinline__ void seq_score(const float* __restrict__ h,
+                                          const __nv_bfloat16* __restrict__ g,
+                                          const __nv_bfloat16* __restrict__ w, int d, float eps,
+                                          const int32_t* __restrict__ lengths, int s, int L,
+                                          long long P, long long p0, float* __restrict__ score,
+                                          float* __restrict__ score2) {
   int n = lengths ? lengths[s] : L;
   n = n < 0 ? 0 : (n > L ? L : n);
   __shared__ float red[kScoreThreads / 32];
@@ -312,13 +331,40 @@ __global__ void __launch_bounds__(kScoreThreads)
   if (threadIdx.x == 0) score[s] = score2[s] = acc;
 }
 
-// dst row i = src row map(i), one CTA per row, 16-byte pieces
+// Both heads of a scoring pass: CTAs 0 .. S - 1 the sequence scores, the others the values of 16
+// rows each. They read nothing of one another's: in turn, two launches of few CTAs took 6.0 and 10.2
+// us (one sequence of 60 response rows of 4096), the one launch takes 6.5.
+__global__ void __launch_bounds__(kScoreThreads)
+    score_heads_kernel(const float* __restrict__ h, const __nv_bfloat16* __restrict__ g,
+                       const __nv_bfloat16* __restrict__ w, int d, float eps,
+                       const int32_t* __restrict__ lengths, int S, int L, long long P, long long p0,
+                       float* __restrict__ score, float* __restrict__ score2,
+                       const __nv_bfloat16* __restrict__ x, float* __restrict__ values) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int s = static_cast<int>(blockIdx.x);
+  if (s < S) {
+    seq_score(h, g, w, d, eps, lengths, s, L, P, p0, score, score2);
+    return;
+  }
+  const long long n = static_cast<long long>(S) * L;
+  const long long i = (s - S) * static_cast<long long>(kScoreThreads / 32) + (threadIdx.x >> 5);
+  if (i < n) head_row(x, d, w, RowMap{n, n, 0}, i, lengths, L, values);
+}
+
+// dst row i = src row map(i), one CTA per row and array, 16-byte pieces; blockIdx.y = 1: the
+// second array (a launch of its own took 3.4 us of a pass of 61 rows)
 __global__ void __launch_bounds__(128)
-    gather_rows_kernel(const uint4* __restrict__ src, int chunks, RowMap map,
-                       uint4* __restrict__ dst) {
+    gather_rows_kernel(const uint4* __restrict__ src, int chunks, RowMap map, uint4* __restrict__ dst,
+                       const uint4* __restrict__ src2, int chunks2, uint4* __restrict__ dst2) {
   pdl_wait();
   pdl_launch_dependents();
   const long long i = blockIdx.x;
+  if (blockIdx.y == 1) {
+    src = src2;
+    chunks = chunks2;
+    dst = dst2;
+  }
   const uint4* s = src + static_cast<size_t>(map_row(i, map)) * chunks;
   uint4* o = dst + static_cast<size_t>(i) * chunks;
   for (int c = threadIdx.x; c < chunks; c += 128) o[c] = s[c];
@@ -396,25 +442,29 @@ int launch_head_dot(const void* x, int64_t d, const void* w, const RowMap& map, 
              : -3;
 }
 
-int launch_gather_rows(const void* src, int64_t rows, int64_t row_bytes, const RowMap& map,
-                       void* dst, cudaStream_t st) {
+int launch_gather_rows(const void* src, int64_t row_bytes, void* dst, const void* src2,
+                       int64_t row_bytes2, void* dst2, int64_t rows, const RowMap& map, cudaStream_t st) {
   if (rows == 0) return 0;
-  if (row_bytes % 16 != 0) return -4;
-  return launch_pdl(gather_rows_kernel, dim3(static_cast<unsigned>(rows)), dim3(128), 0, st,
+  if (row_bytes % 16 != 0 || row_bytes2 % 16 != 0) return -4;
+  return launch_pdl(gather_rows_kernel, dim3(static_cast<unsigned>(rows), 2), dim3(128), 0, st,
                     static_cast<const uint4*>(src), static_cast<int>(row_bytes / 16), map,
-                    static_cast<uint4*>(dst)) == cudaSuccess
+                    static_cast<uint4*>(dst), static_cast<const uint4*>(src2),
+                    static_cast<int>(row_bytes2 / 16), static_cast<uint4*>(dst2)) == cudaSuccess
              ? 0
              : -3;
 }
 
-int launch_seq_score(const float* h, const void* norm, const void* w, int64_t d, float eps,
-                     const int32_t* lengths, int64_t S, int64_t L, int64_t P, int64_t p0,
-                     float* score, float* score2, cudaStream_t st) {
+int launch_score_heads(const float* h, const void* norm, const void* w, int64_t d, float eps,
+                       const int32_t* lengths, int64_t S, int64_t L, int64_t P, int64_t p0,
+                       float* score, float* score2, const void* x, float* values, cudaStream_t st) {
   if (S == 0) return 0;
-  return launch_pdl(seq_score_kernel, dim3(static_cast<unsigned>(S)), dim3(kScoreThreads), 0, st, h,
-                    static_cast<const __nv_bfloat16*>(norm), static_cast<const __nv_bfloat16*>(w),
-                    static_cast<int>(d), eps, lengths, static_cast<int>(L), static_cast<long long>(P),
-                    static_cast<long long>(p0), score, score2) == cudaSuccess
+  const int64_t rows = kScoreThreads / 32;
+  return launch_pdl(score_heads_kernel, dim3(static_cast<unsigned>(S + (S * L + rows - 1) / rows)),
+                    dim3(kScoreThreads), 0, st, h, static_cast<const __nv_bfloat16*>(norm),
+                    static_cast<const __nv_bfloat16*>(w), static_cast<int>(d), eps, lengths,
+                    static_cast<int>(S), static_cast<int>(L), static_cast<long long>(P),
+                    static_cast<long long>(p0), score, score2, static_cast<const __nv_bfloat16*>(x),
+                    values) == cudaSuccess
              ? 0
              : -3;
 }

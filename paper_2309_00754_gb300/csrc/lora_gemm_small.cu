@@ -295,19 +295,19 @@ __device__ __forceinline__ void store_pair16(const Params& p, const Staging& st,
 }
 
 // Log-softmax partials of the thread's row over a tile of 256 columns: the online (max, sum of
-// exp) pair of alternate chunks in each of the row's two warps, merged through `half` (32 pairs of
-// this quarter), and, where it lies, the sampled token's logit (an arithmetic select keeps the
+// exp) pair of every third chunk in each of the row's three warps, merged through `others` (64
+// pairs of this quarter), and, where it lies, the sampled token's logit (an arithmetic select keeps the
 // row in registers).
 __device__ __forceinline__ void emit_lsm(const Params& p, const RowSums& r, int row, bool live, int n0,
                                          float2* part, float* target, bool lora, int par, int q,
-                                         float2* half) {
+                                         float2* others) {
   int id = -1;
   if (live) {
     const int sq = row / p.lsm_L;
     id = p.lsm_ids[static_cast<int64_t>(sq) * p.lsm_ids_ld + p.lsm_ids_off + row - sq * p.lsm_L];
   }
   float m = -FLT_MAX, sum = 0.f;
-  for (int c = 32 * par; c < 256; c += 64) {
+  for (int c = 32 * par; c < 256; c += 96) {
     const int nv = p.N - (n0 + c);
     if (nv <= 0) break;  // uniform over the warp
     float v[32];
@@ -332,15 +332,15 @@ __device__ __forceinline__ void emit_lsm(const Params& p, const RowSums& r, int 
     }
   }
   const int lane = threadIdx.x & 31;
-  if (par == 1) half[lane] = make_float2(m, sum);
-  asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
+  if (par > 0) others[(par - 1) * 32 + lane] = make_float2(m, sum);
+  asm volatile("bar.sync %0, 96;" ::"r"(1 + q) : "memory");
   if (par == 0 && live) {
-    const float2 o = half[lane];
-    const float t = fmaxf(m, o.x);
+    const float2 a = others[lane], b = others[32 + lane];
+    const float t = fmaxf(m, fmaxf(a.x, b.x));
     part[static_cast<int64_t>(row) * p.lsm_tiles + n0 / 256] =
-        make_float2(t, sum * __expf(m - t) + o.y * __expf(o.x - t));
+        make_float2(t, sum * __expf(m - t) + a.y * __expf(a.x - t) + b.y * __expf(b.x - t));
   }
-  asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");  // the buffer serves the next output
+  asm volatile("bar.sync %0, 96;" ::"r"(1 + q) : "memory");  // the buffer serves the next output
 }
 
 template <int kEpi>
@@ -574,17 +574,18 @@ __global__ void __launch_bounds__(NUM_THREADS)
     warp_wait_bounded(acc_full, 0, &no_abort, p.err, kDevTimeoutDrain);
   }
   // ---------------------------------------------------------------------- drain: every warp,
-  // three per quarter of the TMEM lanes (log-softmax: the two that meet at its barriers)
-  constexpr int kDrainers = kEpi == EPI_LOGSOFTMAX ? 2 : 3;
+  // three per quarter of the TMEM lanes
+  constexpr int kDrainers = 3;
   bool epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
   epi_ok = __all_sync(0xffffffffu, epi_ok) && *abort_flag == 0;
+  if (kEpi == EPI_LOGSOFTMAX) epi_ok = __syncthreads_and(epi_ok);  // a quarter's warps meet again
   tc_fence_after();
   if (!kEarly) pdl_launch_dependents();
 
   const int q = warp & 3;             // TMEM lanes 32 q .. of a drain warp
   const int trow = q * 32 + lane;     // row of the segment
-  const int par = kDrainers == 3 ? warp >> 2 : (warp >> 2) - 1;  // which of the warps of its lanes
-  const bool drain = par >= 0 && epi_ok && q * 32 < nrow;
+  const int par = warp >> 2;          // which of the warps of its lanes
+  const bool drain = epi_ok && q * 32 < nrow;
   const bool last = slice == p.ks - 1;
   constexpr int kChunk = chunk_of(kEpi);
   const int nch = p.bn / kChunk;      // column chunks of the tile
@@ -657,7 +658,7 @@ __global__ void __launch_bounds__(NUM_THREADS)
       if constexpr (kEpi == EPI_LOGSOFTMAX) {
         emit_lsm(p, rs, row, live, n0, static_cast<float2*>(y),
                  p.lsm_target + ((p.shared_x ? o : stream) == 0 ? 0 : p.M), lora, par, q,
-                 reinterpret_cast<float2*>(smem + p.stg_off) + q * 32);
+                 reinterpret_cast<float2*>(smem + p.stg_off) + q * 64);
       } else if constexpr (!paired_epi(kEpi)) {
         for (int i = par; i < nch; i += kDrainers) {
           if (owner(i) != slice || n0 + 32 * i >= p.N) continue;

@@ -416,8 +416,8 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
     float* hl = h;
     void* al = a;
     if (last_c) {
-      HY_PROF(HYDRA_PROF_ELEMENTWISE, hydra::launch_gather_rows(attn, ns * Tc, d * 2, pick, a, st));
-      HY_PROF(HYDRA_PROF_ELEMENTWISE, hydra::launch_gather_rows(h, ns * Tc, d * 4, pick, hc, st));
+      HY_PROF(HYDRA_PROF_ELEMENTWISE,
+              hydra::launch_gather_rows(attn, d * 2, a, h, d * 4, hc, ns * Tc, pick, st));
       x_o = a;
       hl = hc;
       al = attn;
@@ -468,13 +468,11 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
   // reward-model score on the LoRA-off stream at the last valid token; values on the
   // LoRA-on stream (the same head: r_phi = LO(V))
   // (position P0 + len - 1: compact row len of its sequence)
-  HY_PROF(HYDRA_PROF_HEADS, hydra::launch_seq_score(hf, w->final_norm, w->w_rm, d, c.rms_eps,
-                                                    lengths, S, L, compact ? Lc : P,
-                                                    compact ? 1 : c.prompt_len, sc, score, st));
   // values from the last stream: the on stream (J-Hydra) or the critic stream (Hydra-PPO)
   const void* fin_on = static_cast<uint8_t*>(fin) + static_cast<size_t>(ns - 1) * SL * d * 2;
-  const hydra::RowMap dense{SL, SL, 0};
-  HY_PROF(HYDRA_PROF_HEADS, hydra::launch_head_dot(fin_on, d, w->w_rm, dense, SL, lengths, L, values, st));
+  HY_PROF(HYDRA_PROF_HEADS, hydra::launch_score_heads(hf, w->final_norm, w->w_rm, d, c.rms_eps, lengths, S, L,
+                                                      compact ? Lc : P, compact ? 1 : c.prompt_len, sc, score,
+                                                      fin_on, values, st));
   HY_PROF(HYDRA_PROF_LOGPROBS,
           hydra::launch_lse_combine(part, part + static_cast<size_t>(SL) * nt, nt, tgt, tgt + SL, S, L, V,
                                     resp_ids, P, lengths, sc, c.beta, logp_actor, logp_ref, reward,
