@@ -68,6 +68,7 @@ struct Params {
   int shared_x;   // 1 = x_on is x_off
   int deferred;   // shared input with LoRA and both outputs: y_off drain, then LoRA
   int streams;    // 1 (shared) or 2 (stacked)
+  int packed;     // the rows of both streams in one 128-row tile, 64 accumulator rows each
   int m_tiles, n_tiles, total_tiles;
   int m_group;  // CTA-pair kernel: 0 = m fastest over all of M; else groups of m_group
                 // m-tiles, m fastest inside a group, then n, then the next group
@@ -486,6 +487,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         mbar_arrive_expect_tx(full_bar(s), STAGE_BYTES);
         const uint32_t a_dst = smem_base + s * STAGE_BYTES;
         tma_load_2d(a_dst, ma, xa, ya, full_bar(s));
+        if (p.packed) tma_load_2d(a_dst + A_TILE / 2, &mp.x[1], xa, ya, full_bar(s));
         tma_load_2d(a_dst + A_TILE, mb, xb, yb, full_bar(s));
       }
       __syncwarp();
@@ -592,7 +594,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int i = 0; i < 3; ++i) tma_prefetch_desc(&mp.y[i]);
     }
     for (int j = 0; j < n_local; ++j) {
-      const Tile tl = decode(p, blockIdx.x + j * gridDim.x);
+      Tile tl = decode(p, blockIdx.x + j * gridDim.x);
+      if (p.packed && q >= 2) {  // accumulator rows 64 .. 127 are the on stream's rows 0 .. 63
+        tl.stream = 1;
+        tl.m0 = -BM / 2;
+      }
       const int b = j & 1;
       const uint32_t acc = tmem_base + b * 256;
       if (p.deferred) {
@@ -1005,7 +1011,12 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   // against 70.2, with LoRA 70.6 against 75.2); one shared input fills this file's single-CTA
   // tiles just as well (57.4 us against 73.8).
   const bool lsm_ok = a.epi != EPI_LOGSOFTMAX || (!a.shared_x && a.M <= BM);
-  if (!a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N))
+  // Log-softmax of up to 64 rows of two streams without LoRA: both fit one 128-row tile here, and
+  // 32000 columns are 125 of these tiles on 152 SMs where the few-rows kernel has two waves of
+  // pairs (60 rows x 4096 x 32000, with the combining launch: 52.6 us, 60.2 there).
+  const bool packed = a.epi == EPI_LOGSOFTMAX && !a.shared_x && a.x_crit == nullptr && a.r == 0 && a.M <= BM / 2 &&
+                      a.y_off != nullptr && a.y_on != nullptr;
+  if (!packed && !a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N))
     return launch_dual_lora_gemm_small(a, stream);
   static bool attr_set = false;
   if (!attr_set) {
@@ -1026,8 +1037,9 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   Maps mp;
   const bool lora = a.r > 0;
   const bool f32 = a.out_f32 != 0;
-  if (!make_map(&mp.x[0], a.x_off, a.M, a.K, BM, false)) return -2;
-  if (!make_map(&mp.x[1], a.shared_x ? a.x_off : a.x_on, a.M, a.K, BM, false)) return -2;
+  const int xrows = packed ? BM / 2 : BM;
+  if (!make_map(&mp.x[0], a.x_off, a.M, a.K, xrows, false)) return -2;
+  if (!make_map(&mp.x[1], a.shared_x ? a.x_off : a.x_on, a.M, a.K, xrows, false)) return -2;
   if (!make_map(&mp.x[2], tri ? a.x_crit : a.x_off, a.M, a.K, BM, false)) return -2;
   const int brows = pair ? bn / 2 : BN;  // a CTA of a pair loads half of the tile's W rows
   if (!make_map(&mp.w, a.W, a.N, a.K, brows, false)) return -2;
@@ -1068,7 +1080,8 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   p.has_on = a.y_on != nullptr;
   p.has_crit = tri && a.y_crit != nullptr && (!lora || (a.u_crit != nullptr && a.B_crit != nullptr));
   p.deferred = (p.shared_x && lora && p.has_off && p.has_on) ? 1 : 0;
-  p.streams = a.shared_x ? 1 : (tri ? 3 : 2);
+  p.packed = packed ? 1 : 0;
+  p.streams = a.shared_x || packed ? 1 : (tri ? 3 : 2);
   p.m_tiles = static_cast<int>(pair ? (a.M + 255) / 256 : (a.M + BM - 1) / BM);
   p.n_tiles = static_cast<int>((a.N + bn - 1) / bn);
   p.total_tiles = p.m_tiles * p.n_tiles * p.streams;

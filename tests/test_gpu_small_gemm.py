@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from tests.helpers import TOL_LINEAR, O, assert_rel, dev_bf16, dev_f32, f64, host_f64, synth
+from tests.helpers import TOL_LINEAR, O, assert_rel, dev_bf16, dev_f32, dev_i32, f64, host_f64, synth
 from paper_2309_00754_gb300 import hydra as H
 
 pytestmark = pytest.mark.gpu
@@ -124,6 +124,27 @@ def test_fused_silu_has_the_operators_bits_for_every_bf16_gate():
     for y in m:
         assert bool(((y == ref) | (y.isnan() & ref.isnan())).all())
     assert int(ref.isnan().sum()) >= 254  # the NaN patterns, and -inf / inf
+
+
+@pytest.mark.parametrize("M,K,V", [(1, 8, 8), (32, 136, 1000), (33, 1032, 264), (64, 4096, 40000)])
+def test_log_softmax_of_both_streams_in_one_tile(M, K, V):
+    """Up to 64 rows of two streams without LoRA share 128-row tiles (also more tiles than SMs);
+    the same rows in a call of 200 rows take CTA pairs, one stream a tile, with the same sums in
+    the same order: equal bits."""
+    g = lambda i, shape, std: dev_bf16(synth.normal_bf16(31 * M + i, shape, std))  # noqa: E731
+    h, W = [g(i, (200, K), 1.0) for i in range(2)], g(2, (V, K), 0.05)
+    ids = dev_i32(synth.randint(77 + M, (200,), 0, V))
+
+    def run(m):
+        ws = torch.empty(H.lm_head_logprobs_workspace_size(1, m, V, 0), dtype=torch.uint8, device="cuda")
+        out = [torch.full((m,), float("nan"), device="cuda") for _ in range(5)]
+        H.hydra_lm_head_logprobs(h[0][:m], h[1][:m], W, None, None, 1.0, ids[:m], None, None, 0.1, 1, m,
+                                 out[0], out[1], out[2], ws, lse_actor=out[3], lse_ref=out[4])
+        return out
+
+    for got, want in zip(run(M), run(200)):
+        assert torch.equal(got, want[:M])
+    assert H.device_error(clear=True) == 0
 
 
 def test_off_rows_ignore_a_non_finite_lora_factor():
