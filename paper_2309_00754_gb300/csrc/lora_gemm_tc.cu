@@ -462,6 +462,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // Launched dependent: barriers and TMEM were set up beside the preceding kernel (3072 x 4096 x
+  // 4096 with its lora_down 123.4 -> 117.5 us a call, 800 x 4096 x 4096 44.7 -> 42.9). Taking x
+  // as final before the lora_down ends, as the few-rows kernel does, gave 0 to 0.5 % and cost 2 %
+  // at 3072 rows.
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp)
@@ -511,12 +516,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     if (p.deferred && n_local > 0)
       for (int kl = 0; kl < prev.n_lora && ok; ++kl)
         load(&mp.u[prev.stream == 2 ? 1 : 0], kl * BK, prev.m0, &mp.b[prev.stream == 2 ? 1 : 0], kl * BK, prev.n0);
+    pdl_launch_dependents();
     // copies still in flight must land before the CTA's shared memory is released
     for (int k = (it > STAGES ? it - STAGES : 0); k < it; ++k) {
       volatile int no_abort = 0;
       warp_wait_bounded(full_bar(k % STAGES), (k / STAGES) & 1, &no_abort, p.err, kDevTimeoutDrain);
     }
   } else if (warp == 1) {
+    pdl_launch_dependents();  // the dependents start once every warp has said so
     // ------------------------------------------------------------ MMA issuer (whole warp,
     // one elected lane issues; the same lane issues every MMA and commit, so each commit
     // covers all MMAs before it)
@@ -614,6 +621,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (!mbar_wait_bounded(acc_full(b), (j >> 1) & 1, abort_flag, p.err, kDevTimeoutEpilogue))
           break;
         tc_fence_after();
+        if (j == n_local - 1) pdl_launch_dependents();
         if (p.shared_x)
           drain(acc, q, lane, staging, chunk_ctr, p, tl.m0, tl.n0, tl.n_lora > 0 ? nullptr : y_off, y_on,
                 tl.n_lora > 0 ? nullptr : py_off, py_on);
@@ -707,6 +715,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   cluster_sync_all();  // barriers of both CTAs are initialised before any remote signal
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // as in the single-CTA kernel. No early trigger here: the next kernel's CTAs beside the last
+  // tiles cost 2 % of a power-bound loop (3072 x 11008 x 4096: 358 us a call, 365 with it).
+  pdl_wait();
 
   // tile -> (stream, 256-row block, column block); this CTA's rows are m0 + 128 rank
   auto decode2 = [&](int t) {
@@ -1122,12 +1133,10 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
     const int nclusters = nsm / 2;
     const unsigned grid =
         2u * static_cast<unsigned>(p.total_tiles < nclusters ? p.total_tiles : nclusters);
-    dual_lora_gemm_2cta_kernel<<<grid, NUM_THREADS, SMEM2_BYTES, stream>>>(mp, p);
-    return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+    return launch_pdl(dual_lora_gemm_2cta_kernel, dim3(grid), dim3(NUM_THREADS), SMEM2_BYTES, stream, mp, p) == cudaSuccess ? 0 : -3;
   }
   const unsigned grid = static_cast<unsigned>(p.total_tiles < nsm ? p.total_tiles : nsm);
-  dual_lora_gemm_kernel<<<grid, NUM_THREADS, SMEM_BYTES, stream>>>(mp, p);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -3;
+  return launch_pdl(dual_lora_gemm_kernel, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, stream, mp, p) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace hydra
