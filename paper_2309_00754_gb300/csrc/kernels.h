@@ -76,7 +76,7 @@ int* device_error_word();
 int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream);
 // The same linear for few token rows per stream (lora_gemm_small.cu), which
 // launch_dual_lora_gemm_tc takes where small_gemm_wanted.
-bool small_gemm_wanted(int64_t M, int64_t K, int64_t N);
+bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams);
 int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream);
 // TMA map over a row-major [rows, cols] bf16 (or fp32) matrix with row stride ld elements:
 // 128-byte swizzle, boxes of [box_rows x 128 bytes], zero fill out of bounds

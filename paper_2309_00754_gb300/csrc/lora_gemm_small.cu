@@ -1,4 +1,4 @@
-// The dual-output LoRA linear (see lora_gemm_tc.cu for the mathematics) for up to 448 token rows
+// The dual-output LoRA linear (see lora_gemm_tc.cu for the mathematics) for up to 512 token rows
 // per stream: one short sequence, a prompt, a decode batch. The work there is reading W once, and
 // the tile kernel of lora_gemm_tc.cu leaves most of the chip idle: 97 rows of two streams by 4096
 // columns are 32 tiles of 128 x 256, each with the whole of K, on 152 SMs.
@@ -12,7 +12,7 @@
 //  * Columns and K. bn (a multiple of 32 up to 256) and the split of K over ks pairs of a cluster
 //    (1 or 2) are chosen so that the pairs fill the SMs. ks depends on M, K and N alone, so that
 //    every output element is one sum in one order whatever the streams, the epilogue and the tile
-//    width: shared, stacked and three-stream calls agree bit for bit. (Four slices measured
+//    width: shared, stacked and three-stream calls that come here agree bit for bit. (Four slices measured
 //    slower: only 15 clusters of eight CTAs fit on the chip, 36 of four.)
 //  * Ring items are two k-blocks of 64, and x and W have a TMA warp each. What a warp executes
 //    per item is the limit at these sizes: one warp and 64-wide items took 570 clocks each, more
@@ -750,6 +750,17 @@ Kernel kernel_of(int epi) {
   }
 }
 
+// Lets every kernel have kSmemMax of shared memory (needed before the occupancy query, too).
+bool allow_smem(int dev) {
+  static bool done[64] = {false};
+  if (dev < 0 || dev >= 64) return false;
+  if (done[dev]) return true;
+  for (int e = smallm::EPI_STORE; e <= smallm::EPI_STORE_F32; ++e)
+    if (cudaFuncSetAttribute(kernel_of(e), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
+      return false;
+  return done[dev] = true;
+}
+
 // Clusters of 2 ks CTAs with this shared memory that the device holds at once (the same for every
 // epilogue: shared memory and threads decide).
 int resident_clusters(int dev, int ks, int smem) {
@@ -779,82 +790,120 @@ int resident_clusters(int dev, int ks, int smem) {
   return n;
 }
 
-}  // namespace
-
-// Sizes alone decide, not streams or epilogue: the sums of one (M, K, N) have one order. Above
-// 128 rows the tile kernel of lora_gemm_tc.cu takes over where its 256-column tiles fill the chip
-// (measured on GB300, us, this kernel / that one; rows x K x N, two streams): 97 x 4096 x 4096
-// 12.3 / 30.4, x 12288 25.6 / 35.3, x 22016 43.9 / 80.3; 97 x 11008 x 4096 22.5 / 69.3;
-// 200 x 4096 x 11008 36.8 / 39.0, x 12288 46.9 / 44.9, x 16384 47.0 / 44.0; 300 x 4096 x 4096
-// 19.5 / 23.5 (shared input 16.0 / 24.0), x 12288 58.0 / 61.9, x 22016 110 / 103;
-// 384 x 4096 x 11008 49.2 / 57.1; 448 x 4096 x 4096 23.9 / 24.7, x 12288 81.8 / 63.0.
-bool small_gemm_wanted(int64_t M, int64_t K, int64_t N) {
-  if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
-  return M <= 128 || (M <= 256 && N <= 11264) || (M <= 384 && N <= 12288) || (M <= 448 && N <= 4096);
+Shape shape_of(int64_t M, int64_t K, int64_t N, int streams, int epi) {
+  Shape s{};
+  s.streams = streams;
+  s.nseg = static_cast<int>((M + 127) / 128);
+  const int64_t kb = (K + smallm::BK - 1) / smallm::BK;
+  // Split of K between the two pairs of a cluster (36 of these fit on the chip) where 256-column
+  // tiles of two streams leave most pairs idle and half of K is worth the exchange of the sums,
+  // about 3 us. Measured, one slice against two, us, two streams: 4 to 12 tiles, 20 x 1024 x 776
+  // -4 % to 200 x 1024 x 1536 +18 %, 200 x 2048 x 1536 +4 %, 97 x 3200 x 3000 -5 %; 16 tiles,
+  // 128 x 2048 x 4096 +6 %, 97 x 4096 x 4096 -9 %; 24 tiles, 449 x 3200 x 1536 +26 %,
+  // 200 x 6000 x 3000 -1 %; 32 tiles, 200 x 4096 x 4096 +21 %, 200 x 11008 x 4096 +8 %.
+  const int64_t tiles = s.nseg * ((N + 255) / 256);
+  const int64_t kb_min = tiles <= 12 ? 16 : (tiles <= 18 ? 20 : 40);
+  s.ks = epi != smallm::EPI_LOGSOFTMAX && tiles <= 24 && kb >= kb_min ? 2 : 1;
+  if (s.streams == 1 && (s.nseg & 1)) ++s.nseg;
+  s.seg = static_cast<int>(((M + s.nseg - 1) / s.nseg + 7) / 8 * 8);
+  s.row_tiles = (s.streams * s.nseg + 1) / 2;
+  s.paired = smallm::paired_epi(epi);
+  return s;
 }
 
-int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
-  using namespace smallm;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-  static bool attr_set[64] = {false};
-  if (!attr_set[dev]) {
-    for (int e = EPI_STORE; e <= EPI_STORE_F32; ++e)
-      if (cudaFuncSetAttribute(kernel_of(e), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
-        return -1;
-    attr_set[dev] = true;
-  }
-  const bool tri = a.x_crit != nullptr && !a.shared_x;
-  const int M = static_cast<int>(a.M), N = static_cast<int>(a.N);
-  const int kb = static_cast<int>((a.K + BK - 1) / BK);
-  const bool lora_on = a.r > 0 && a.u != nullptr && a.B != nullptr && a.y_on != nullptr;
-  const bool lora_crit = tri && a.r > 0 && a.u_crit != nullptr && a.B_crit != nullptr && a.y_crit != nullptr;
-  Shape s;
-  s.streams = a.shared_x ? 1 : (tri ? 3 : 2);
-  s.nseg = (M + 127) / 128;
-  // Split of K between the two pairs of a cluster where 256-column tiles of two streams leave
-  // half of the pairs idle: 36 clusters of four CTAs fit on the chip.
-  s.ks = a.epi != EPI_LOGSOFTMAX && s.nseg * ((N + 255) / 256) <= 36 && kb >= 8 ? 2 : 1;
-  if (s.streams == 1 && (s.nseg & 1)) ++s.nseg;
-  s.seg = ((M + s.nseg - 1) / s.nseg + 7) / 8 * 8;
-  s.row_tiles = (s.streams * s.nseg + 1) / 2;
-  s.lora = lora_on || lora_crit;
-  s.both = a.shared_x && lora_on && a.y_off != nullptr;
-  s.paired = a.epi == EPI_SWIGLU || a.epi == EPI_ROPE;
-  const int npair = a.epi == EPI_SWIGLU ? N / 2 : (N + 127) / 128 * 64;
+int64_t tiles_of(const Shape& s, int64_t N, int epi, int bn) {
+  const int64_t npair = epi == smallm::EPI_SWIGLU ? N / 2 : (N + 127) / 128 * 64;
+  return s.row_tiles * (s.paired ? (npair + bn / 2 - 1) / (bn / 2) : (N + bn - 1) / bn);
+}
+// partner rows of W that are neighbours
+int box_of(int epi) { return epi == smallm::EPI_SWIGLU ? 128 : 64; }
 
-  const int box = a.epi == EPI_SWIGLU ? 128 : 64;  // partner rows of W that are neighbours
-
-  // Tile width: the fewest clocks over the waves. A k-block of 64 costs the pair its products
-  // (2 bn) or a CTA's fill from L2 at 64 B per clock (2 (seg + bn / 2)), and a wave about 6000
-  // clocks of set-up, first loads and drain.
-  Config best{};
+// Tile width: the fewest clocks over the waves (returned; `best` keeps bn = 0 if none fits). A
+// k-block of 64 costs the pair its products (2 bn) or a CTA's fill from L2 at 64 B per clock
+// (2 (seg + bn / 2)), and a wave `per_wave` clocks of set-up, first loads and drain.
+double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, double per_wave, Config* best) {
+  const int64_t kb = (K + smallm::BK - 1) / smallm::BK;
   double best_t = 1e30;
-  auto tiles_of = [&](int bn) {
-    return s.row_tiles * (s.paired ? (npair + bn / 2 - 1) / (bn / 2) : (N + bn - 1) / bn);
-  };
   for (int bn : {256, 224, 192, 160, 128, 96, 64}) {
     if (s.ks == 2 && bn % (s.paired ? 128 : 64) != 0) continue;  // whole chunks for each slice
-    if (s.paired && bn / 2 / gcd(bn / 2, box) > kMaxBoxes) continue;
-    if (a.epi == EPI_LOGSOFTMAX && bn != 256) continue;
+    if (s.paired && bn / 2 / gcd(bn / 2, box_of(epi)) > smallm::kMaxBoxes) continue;
+    if (epi == smallm::EPI_LOGSOFTMAX && bn != 256) continue;
     Config c{};
     if (!lay_out(s, bn, &c)) continue;
     const int fit = resident_clusters(dev, s.ks, c.smem);
     if (fit < 1) continue;
     const int fill = 2 * (s.seg + bn / 2), mma = 2 * bn;
     const double item = 2.0 * (fill > mma ? fill : mma);
-    const int waves = (tiles_of(bn) + fit - 1) / fit;
-    const double t = waves * (static_cast<double>((kb + s.ks - 1) / s.ks) * item + 6000.0);
+    const int64_t waves = (tiles_of(s, N, epi, bn) + fit - 1) / fit;
+    const double t = waves * (static_cast<double>((kb + s.ks - 1) / s.ks) * item + per_wave);
     if (t < best_t) {
       best_t = t;
-      best = c;
+      *best = c;
     }
   }
+  return best_t;
+}
+
+}  // namespace
+
+// Sizes alone decide, not the epilogue, nor whether one or two streams are given: the sums of one
+// (M, K, N) have one order. Above 128 rows the tile kernel of lora_gemm_tc.cu takes over where its
+// 256-column tiles fill the chip (measured on GB300, us, this kernel / that one; rows x K x N, two
+// streams):
+//  * up to 128 rows: 97 x 4096 x 4096 12.3 / 30.4, x 12288 25.6 / 35.3, x 22016 43.9 / 80.3;
+//    97 x 11008 x 4096 22.5 / 69.3;
+//  * up to 256, where a stream is one 256-row tile there: 200 x 4096 x 8192 22.9 / 24.7, x 11008
+//    35.3 / 39.5, x 14336 40.6 / 41.0, x 16384 45.4 / 44.1, x 22016 79.4 / 71.2 (above 11264
+//    columns with a long K only: 200 x 512 x 12288 15.4 / 14.9);
+//  * up to 384, where it is two and the second half empty: 300 x 4096 x 4096 18.8 / 23.8 (shared
+//    input 15.9 / 24.5), x 12288 58.9 / 63.3, x 16384 66.7 / 74.1, x 22016 105.1 / 104.0;
+//  * up to 512, while few columns leave it less than one wave or little more: 512 x 4096 x 2048
+//    18.8 / 21.7, x 4096 22.9 / 24.7, x 5120 33.1 / 38.2, x 8192 46.6 / 42.9; a long K makes up
+//    for that: 448 x 11008 x 4096 51.9 / 54.2, 512 x 11008 x 4096 57.4 / 55.0.
+// Three streams leave a row segment over in a pair, or a wave, more often (with their lora_downs:
+// 100 x 4096 x 12288 44.3 / 41.6, 300 x 512 x 12288 35.4 / 26.1, 256 x 4096 x 4096 37.7 / 32.1, but
+// 97 rows x 11008 x 4096 half of that kernel's time): the clocks of both are estimated, with shares
+// per wave and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
+// 12288), none of which is then slower.
+bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams) {
+  if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
+  const bool wanted = M <= 128 || (M <= 256 && (N <= 11264 || (N <= 14336 && K >= 2048))) ||
+                      (M <= 384 && M > 256 && N <= 16384) || (M <= 448 && N <= 5120) ||
+                      (M <= 512 && N <= 5120 && K <= 4096);
+  if (!wanted || streams < 3) return wanted;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !allow_smem(dev)) return false;
+  Config c{};
+  const double here = choose_width(shape_of(M, K, N, streams, smallm::EPI_STORE), K, N, smallm::EPI_STORE, dev,
+                                   10000.0, &c);
+  const int64_t kb = (K + 63) / 64, cols = (N + 255) / 256;
+  // that kernel: 128-row tiles, 704 clocks of fill per k-block, on 152 SMs; 256-row tiles, 512 of
+  // products, on 76 pairs
+  const int64_t tiles = streams * cols * (M <= 128 ? 1 : (M + 255) / 256);
+  const int64_t waves = M <= 128 ? (tiles + 151) / 152 : (tiles + 75) / 76;
+  const double there = static_cast<double>(waves * kb) * (M <= 128 ? 704 : 512) + 12000.0 + 1000.0 * (waves - 1);
+  return c.bn != 0 && 1.1 * here < there;
+}
+
+int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
+  using namespace smallm;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !allow_smem(dev)) return -1;
+  const bool tri = a.x_crit != nullptr && !a.shared_x;
+  const int M = static_cast<int>(a.M), N = static_cast<int>(a.N);
+  const int kb = static_cast<int>((a.K + BK - 1) / BK);
+  const bool lora_on = a.r > 0 && a.u != nullptr && a.B != nullptr && a.y_on != nullptr;
+  const bool lora_crit = tri && a.r > 0 && a.u_crit != nullptr && a.B_crit != nullptr && a.y_crit != nullptr;
+  Shape s = shape_of(a.M, a.K, a.N, a.shared_x ? 1 : (tri ? 3 : 2), a.epi);
+  s.lora = lora_on || lora_crit;
+  s.both = a.shared_x && lora_on && a.y_off != nullptr;
+  Config best{};
+  choose_width(s, a.K, a.N, a.epi, dev, 6000.0, &best);
   if (best.bn == 0) return -4;
   const int bn = best.bn;
 
   Params p{};
-  p.b_box = s.paired ? gcd(bn / 2, box) : bn / 2;
+  p.b_box = s.paired ? gcd(bn / 2, box_of(a.epi)) : bn / 2;
   Maps mp;
   const void* xs[3] = {a.x_off, a.shared_x ? a.x_off : a.x_on, a.x_crit};
   for (int i = 0; i < 3; ++i) {
@@ -905,7 +954,7 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   p.lsm_ids_off = static_cast<int>(a.lsm_ids_off);
   p.lsm_tiles = (N + 255) / 256;
   p.err = a.err;
-  const int tiles = tiles_of(bn);
+  const int64_t tiles = tiles_of(s, a.N, a.epi, bn);
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * s.ks), static_cast<unsigned>(s.row_tiles),

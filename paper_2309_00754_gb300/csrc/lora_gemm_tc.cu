@@ -1027,7 +1027,8 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   // pairs (60 rows x 4096 x 32000, with the combining launch: 52.6 us, 60.2 there).
   const bool packed = a.epi == EPI_LOGSOFTMAX && !a.shared_x && a.x_crit == nullptr && a.r == 0 && a.M <= BM / 2 &&
                       a.y_off != nullptr && a.y_on != nullptr;
-  if (!packed && !a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N))
+  const int streams = a.shared_x ? 1 : (a.x_crit != nullptr ? 3 : 2);
+  if (!packed && !a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N, streams))
     return launch_dual_lora_gemm_small(a, stream);
   static bool attr_set = false;
   if (!attr_set) {

@@ -22,18 +22,21 @@ def _dev(t):
     return None if t is None else dev_bf16(t)
 
 
-@pytest.mark.parametrize("M,K,N,r,f32", [
-    (1, 8, 8, 0, False),          # one row, one column chunk, one partial k-block
-    (5, 136, 264, 8, True),       # an empty second segment; N and K tails
-    (64, 1024, 520, 16, False),   # two K slices of four items each
-    (65, 1160, 1032, 136, True),  # two LoRA items, the second of one k-block
-    (128, 2048, 4104, 72, False),  # the largest single segment, a tail tile of one chunk
-    (129, 1032, 4104, 72, True),  # two segments per stream, two slices (34 256-column tiles)
-    (257, 520, 1288, 8, False),   # three segments per stream: a pair of the off and the on stream
-    (384, 264, 12288, 16, False),  # the largest, more tiles than the chip holds at once
-    (448, 200, 520, 8, True),
+@pytest.mark.parametrize("M,K,N,r,f32,tri_too", [
+    (1, 8, 8, 0, False, True),          # one row, one column chunk, one partial k-block
+    (5, 136, 264, 8, True, True),       # an empty second segment; N and K tails
+    (64, 1024, 520, 16, False, True),   # the longest K in one slice
+    (64, 2048, 520, 16, False, True),   # two K slices of eight items each
+    (65, 2184, 1032, 136, True, True),  # two LoRA items, the second of one k-block
+    (128, 2048, 4104, 72, False, True),  # the largest single segment, a tail tile of one chunk
+    (129, 1032, 4104, 72, True, False),  # two segments per stream, 34 256-column tiles
+    (257, 5128, 1288, 8, False, True),  # two slices again: 18 tiles
+    (257, 520, 1288, 8, False, True),   # three segments per stream: a pair of the off and the on stream
+    (384, 264, 12288, 16, False, False),  # more tiles than the chip holds at once
+    (448, 200, 520, 8, True, True),
+    (512, 136, 5120, 8, False, False),  # the most rows: full segments, four per stream
 ])
-def test_few_rows_against_oracle_and_one_order_of_sums(M, K, N, r, f32):
+def test_few_rows_against_oracle_and_one_order_of_sums(M, K, N, r, f32, tri_too):
     x, W, ab = _problem(M, K, N, r, seed=M + K)
     dt = torch.float32 if f32 else torch.bfloat16
     d, dW = [dev_bf16(t) for t in x], dev_bf16(W)
@@ -52,8 +55,9 @@ def test_few_rows_against_oracle_and_one_order_of_sums(M, K, N, r, f32):
     sh = two(d[1], None, *dab[0])
     crit = two(d[2], None, *dab[1], want=(False, True))
     off = two(d[0], None, *dab[0], want=(True, False))
-    assert torch.equal(tri[0], st[0]) and torch.equal(tri[1], st[1])
-    assert torch.equal(st[1], sh[1]) and torch.equal(tri[2], crit[1]) and torch.equal(off[0], st[0])
+    assert torch.equal(st[1], sh[1]) and torch.equal(off[0], st[0])
+    if tri_too:  # elsewhere three streams take the tile kernel, whose sums have another order
+        assert torch.equal(tri[0], st[0]) and torch.equal(tri[1], st[1]) and torch.equal(tri[2], crit[1])
     # against fp64, fp32 sums of bf16 products in another order: 1e-4 as for the tile kernel's fp32
     # outputs. u is the library's own (hydra_lora_down, tested by itself): where it rounds to bf16
     # the other way than the oracle's, y moves by ulp(u) |B|, up to 2^-6 * 0.1 = 1.6e-3
@@ -73,7 +77,7 @@ def test_few_rows_fused_epilogues(M, N, shared):
     """SwiGLU, rotary (N past the rotated columns, a partial last head) and residual epilogues
     equal the plain linear followed by the separate kernel, bit for bit (two K slices; at 22016
     columns one, and 160-column tiles of five boxes)."""
-    K, r, P = 1032, 16, 50
+    K, r, P = 2184, 16, 50
     x, W, ab = _problem(M, K, N, r, seed=7 * M + N)
     d, dW, dB = [dev_bf16(t) for t in x], dev_bf16(W), dev_bf16(ab[0][1])
     xo = None if shared else d[1]
