@@ -790,7 +790,8 @@ class HydraPPOIterationLlama7B(HydraGenerateLlama7B):
         torch.cuda.synchronize()
         n_score = sum(n for _, n in self.H.profile_collect(reset=True).values())
         self.H.profile_enable(False)
-        self.launches_per_step += n_score + 4  # + the PPO moments, coef, loss, finalize
+        # + the PPO losses: one launch up to 16384 tokens, moments and loss above
+        self.launches_per_step += n_score + (1 if self.S * self.n_steps <= 16384 else 2)
         return out
 
     def config(self):

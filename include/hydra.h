@@ -122,8 +122,9 @@ hydra_status hydra_lora_linear(const void* x_off, const void* x_on, int64_t M, i
  * hydra_lora_linear, for callers that keep u, e.g. to time the two kernels apart):
  *     y_off = x_off W^T,   y_on = x_on W^T + u B^T
  *   u : bf16 [M, r] = s (x_on A^T) as written by hydra_lora_down; B : bf16 [N, r].
- *   r == 0 (u, B ignored) means no LoRA. algo: 0 automatic, 1 tcgen05 tile kernel,
- *   2 GEMV (at most 16 token rows over both streams), 3 tcgen05 single-CTA tiles.
+ *   r == 0 (u, B ignored) means no LoRA. algo: 0 automatic, 1 a tcgen05 kernel (few rows: the
+ *   few-rows kernel, else CTA-pair tiles), 2 GEMV (at most 16 token rows over both streams),
+ *   3 tcgen05 single-CTA tiles.
  * Same layout, alignment and error rules as hydra_lora_linear; no workspace.
  */
 hydra_status hydra_dual_linear(const void* x_off, const void* x_on, int64_t M, int64_t K,
@@ -165,8 +166,8 @@ hydra_status hydra_skinny_linear(const void* x, int64_t M, int64_t K, int64_t N,
  *     y_off  = x_off  W^T
  *     y_act  = x_act  W^T + u_a B_act^T,    u_a = s (x_act  A_act^T)  stored as bf16
  *     y_crit = x_crit W^T + u_c B_crit^T,   u_c = s (x_crit A_crit^T) stored as bf16
- * on the tcgen05 kernel with the three streams' tiles of one output block adjacent, so each W
- * tile comes from HBM once and twice more from L2. Inputs may alias one another (the first
+ * on a tcgen05 kernel with the three streams' tiles of one output block adjacent, so each W
+ * tile comes from HBM once and again from L2. Inputs may alias one another (the first
  * layer of a pass); any output may be NULL (not all three), and a NULL output's LoRA set may
  * be NULL. With A_crit = A_act, B_crit = B_act and x_crit = x_act, y_crit equals y_act bit
  * for bit (J-Hydra's single LoRA set). Layouts, alignment and errors as hydra_lora_linear;
@@ -239,9 +240,10 @@ hydra_status hydra_dual_linear_rope(const void* x_off, const void* x_on, int64_t
 
 /*
  * hydra_lora_linear with the kernel family chosen by the caller:
- *   algo 0 = automatic (as hydra_lora_linear), 1 = tcgen05 tile kernel (any M; CTA pairs
- *   with 256-row tiles when M > 128), 2 = GEMV kernel (requires at most 16 token rows over
- *   both streams), 3 = tcgen05 tile kernel on single CTAs only (128-row tiles).
+ *   algo 0 = automatic (as hydra_lora_linear), 1 = a tcgen05 kernel (any M: the few-rows
+ *   kernel up to 128 rows, and up to 512 where the sizes favour it, else CTA pairs with
+ *   256-row tiles), 2 = GEMV kernel (requires at most 16 token rows over both streams),
+ *   3 = tcgen05 tile kernel on single CTAs only (128-row tiles).
  * Same arguments, results and errors otherwise; algo outside 0..3 is HYDRA_ERR_RANGE.
  */
 hydra_status hydra_lora_linear_algo(const void* x_off, const void* x_on, int64_t M, int64_t K,
