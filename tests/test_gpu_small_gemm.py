@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from tests.helpers import TOL_LINEAR, O, assert_rel, dev_bf16, dev_f32, dev_i32, f64, host_f64, synth
+from tests.helpers import TOL_LINEAR, TOL_LOGP, O, assert_abs, assert_rel, dev_bf16, dev_f32, dev_i32, f64, host_f64, synth
 from paper_2309_00754_gb300 import hydra as H
 
 pytestmark = pytest.mark.gpu
@@ -148,6 +148,24 @@ def test_log_softmax_of_both_streams_in_one_tile(M, K, V):
 
     for got, want in zip(run(M), run(200)):
         assert torch.equal(got, want[:M])
+    assert H.device_error(clear=True) == 0
+
+
+@pytest.mark.parametrize("M,K,V,r", [(1, 136, 264, 8), (60, 520, 1000, 16), (100, 1032, 520, 0), (128, 136, 4104, 136)])
+def test_log_softmax_of_a_row_segment_per_stream(M, K, V, r):
+    """Log-softmax partials of a pair that holds both streams (65 to 128 rows, or LoRA): three
+    warps per row merge their chunks; against the oracle, two streams, the last tile partial."""
+    x, W, ab = _problem(M, K, V, r, seed=3 * M + V)
+    A, B = ab[0]
+    ids = synth.randint(78 + M, (M,), 0, V)
+    ws = torch.empty(H.lm_head_logprobs_workspace_size(1, M, V, r), dtype=torch.uint8, device="cuda")
+    out = [torch.full((M,), float("nan"), device="cuda") for _ in range(5)]
+    H.hydra_lm_head_logprobs(dev_bf16(x[0]), dev_bf16(x[1]), dev_bf16(W), _dev(A), _dev(B), 2.0, dev_i32(ids), None,
+                             None, 0.1, 1, M, out[0], out[1], out[2], ws, lse_actor=out[3], lse_ref=out[4])
+    z_ref, z_act = O.dual_lora_linear(f64(x[0]), f64(x[1]), f64(W), None if A is None else f64(A),
+                                      None if B is None else f64(B), 2.0, out_bf16=False)
+    for got, z in ((out[0], z_act), (out[1], z_ref)):
+        assert_abs(host_f64(got), O.log_softmax_gather(z, ids)[0], TOL_LOGP, "logp")
     assert H.device_error(clear=True) == 0
 
 
