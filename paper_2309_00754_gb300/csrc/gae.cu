@@ -6,7 +6,7 @@
 //   R_t     = A_t + V_t;   A_t = R_t = 0 for t >= len
 //
 // Rows of whole float4 groups up to 512 tokens: the sequence lives in the warp's registers
-// (gae_scan_reg_kernel). 16384 x 400 tokens, ragged: 26.3 us through shared memory, 18.1 so.
+// (gae_scan_reg_kernel). 16384 x 400 tokens, ragged: 26.3 us through shared memory, 15.1 so.
 // Other lengths: the warp loads its sequence into shared memory with coalesced loads.
 // Lane j owns the contiguous chunk [j c, j c + c). Each lane runs the recursion over its chunk with a zero
 // carry, which gives an affine map A_start = b + m A_next (m = (gamma lambda)^count). A
@@ -124,11 +124,17 @@ __global__ void gae_scan_kernel(const float* __restrict__ rew, const float* __re
   }
 }
 
-// Register-only variant for L % 4 == 0, L <= 32 CH (CH % 4 == 0, at most 16): lane l owns
-// elements [CH l, CH l + CH), loaded and stored as float4 (rows are 16-byte aligned); the value
-// after the chunk comes from lane l + 1 by shuffle. float4 groups at or beyond the sequence length
-// are neither read nor computed, groups beyond L not written.
-template <int CH>
+// Register-only variant for L % 4 == 0, L <= 128 R (R at most 4): the row goes by rounds of 128
+// tokens, in each of which lane l owns the float4 group l, so that every load and store of the warp
+// is whole lines. The rounds' suffix scans are independent; their first lanes' maps then chain the
+// carries from the last round to the first. Groups at or beyond the sequence length are neither
+// read nor computed, groups beyond L not written.
+// Bound by HBM (8 B per valid token read, 8 B per token written). With 16 consecutive tokens per
+// lane, every access touched half of 32 sectors: 16384 x 400 ragged tokens 18.0 us, now 15.1 (5.4
+// TB/s); 65536 x 512 75.4, 63.6. The warp skips the rounds past its sequence's length (without
+// that the rounds' shuffles cost more than the lines gain: 20.7 and 84.9 us); a single round has
+// none to skip.
+template <int R>
 __global__ void __launch_bounds__(256)
     gae_scan_reg_kernel(const float* __restrict__ rew, const float* __restrict__ val,
                         const int32_t* __restrict__ lengths, int S, int L, float gamma, float lam,
@@ -143,71 +149,82 @@ __global__ void __launch_bounds__(256)
     if (lane == 0) record_error(err, kDevBadLength);
     n = n < 0 ? 0 : L;
   }
-  const int lo = lane * CH;
-  const float4* rr = reinterpret_cast<const float4*>(rew + static_cast<size_t>(s) * L + lo);
-  const float4* vv = reinterpret_cast<const float4*>(val + static_cast<size_t>(s) * L + lo);
-  float r[CH], v[CH];
+  const float4* rr = reinterpret_cast<const float4*>(rew + static_cast<size_t>(s) * L) + lane;
+  const float4* vv = reinterpret_cast<const float4*>(val + static_cast<size_t>(s) * L) + lane;
+  float r[R][4], v[R][4];  // r becomes the advantages
 #pragma unroll
-  for (int q = 0; q < CH / 4; ++q) {
+  for (int q = 0; q < R; ++q) {
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (lo + 4 * q < n) {
-      a = __ldcs(rr + q);
-      b = __ldcs(vv + q);
+    if (128 * q + 4 * lane < n) {
+      a = __ldcs(rr + 32 * q);
+      b = __ldcs(vv + 32 * q);
     }
-    r[4 * q] = a.x; r[4 * q + 1] = a.y; r[4 * q + 2] = a.z; r[4 * q + 3] = a.w;
-    v[4 * q] = b.x; v[4 * q + 1] = b.y; v[4 * q + 2] = b.z; v[4 * q + 3] = b.w;
+    r[q][0] = a.x; r[q][1] = a.y; r[q][2] = a.z; r[q][3] = a.w;
+    v[q][0] = b.x; v[q][1] = b.y; v[q][2] = b.z; v[q][3] = b.w;
   }
   const float c = gamma * lam;
-  // value following this lane's chunk: the next lane's first value while still valid
-  const float v_after = __shfl_down_sync(0xffffffffu, v[0], 1);
-  const int he = min(lo + CH, n);
-  float a = 0.f, m = 1.f;
-  float loc[CH];
+  float b[R], m[R];  // the affine map of the lane's group, then of the groups from it to the round's end
 #pragma unroll
-  for (int i = CH - 1; i >= 0; --i) {
-    const int t = lo + i;
-    loc[i] = 0.f;
-    if (t < he) {
-      const float vn = (i == CH - 1) ? ((t + 1 < n) ? v_after : 0.f) : ((t + 1 < n) ? v[i + 1] : 0.f);
-      a = (r[i] + gamma * vn - v[i]) + c * a;
-      loc[i] = a;
-      m *= c;
+  for (int q = 0; q < R; ++q) {
+    b[q] = 0.f;
+    m[q] = 1.f;
+    if (R > 1 && 128 * q >= n) continue;  // the whole warp
+    // value following the group: the next lane's first, the next round's for the last lane
+    float after = __shfl_down_sync(0xffffffffu, v[q][0], 1);
+    if (q + 1 < R) {
+      const float next = __shfl_sync(0xffffffffu, v[q + 1 < R ? q + 1 : q][0], 0);
+      if (lane == 31) after = next;
+    }
+    const int lo = 128 * q + 4 * lane;
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+      const int t = lo + i;
+      if (t < n) {
+        const float vn = t + 1 < n ? (i == 3 ? after : v[q][i < 3 ? i + 1 : 3]) : 0.f;
+        b[q] = (r[q][i] + gamma * vn - v[q][i]) + c * b[q];
+        r[q][i] = b[q];
+        m[q] *= c;
+      }
+    }
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float b2 = __shfl_down_sync(0xffffffffu, b[q], off);
+      const float m2 = __shfl_down_sync(0xffffffffu, m[q], off);
+      if (lane + off < 32) {
+        b[q] = fmaf(m[q], b2, b[q]);
+        m[q] *= m2;
+      }
     }
   }
-  float b = (he > lo) ? a : 0.f;
+  float4* ao = reinterpret_cast<float4*>(adv + static_cast<size_t>(s) * L) + lane;
+  float4* ro = reinterpret_cast<float4*>(ret + static_cast<size_t>(s) * L) + lane;
+  float from_next = 0.f;  // the advantage at the first token of the next round
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-    const float m2 = __shfl_down_sync(0xffffffffu, m, off);
-    if (lane + off < 32) {
-      b = fmaf(m, b2, b);
-      m *= m2;
+  for (int q = R - 1; q >= 0; --q) {
+    if (R > 1 && 128 * q >= n) {  // the whole warp
+      if (128 * q + 4 * lane < L) {
+        __stcs(ao + 32 * q, make_float4(0.f, 0.f, 0.f, 0.f));
+        __stcs(ro + 32 * q, make_float4(0.f, 0.f, 0.f, 0.f));
+      }
+      continue;
     }
-  }
-  float carry = __shfl_down_sync(0xffffffffu, b, 1);
-  if (lane == 31) carry = 0.f;
-  float p = c;
+    const float start = fmaf(m[q], from_next, b[q]);  // at the group's first token
+    float carry = __shfl_down_sync(0xffffffffu, start, 1);
+    if (lane == 31) carry = from_next;
+    from_next = __shfl_sync(0xffffffffu, start, 0);
+    const int lo = 128 * q + 4 * lane;
+    float e[4], f[4], p = c;
 #pragma unroll
-  for (int i = CH - 1; i >= 0; --i) {
-    if (lo + i < he) {
-      loc[i] = fmaf(p, carry, loc[i]);
-      p *= c;
+    for (int i = 3; i >= 0; --i) {
+      const bool ok = lo + i < n;
+      e[i] = ok ? fmaf(p, carry, r[q][i]) : 0.f;
+      f[i] = ok ? e[i] + v[q][i] : 0.f;
+      if (ok) p *= c;
     }
-  }
-  float4* ao = reinterpret_cast<float4*>(adv + static_cast<size_t>(s) * L + lo);
-  float4* ro = reinterpret_cast<float4*>(ret + static_cast<size_t>(s) * L + lo);
-#pragma unroll
-  for (int q = 0; q < CH / 4; ++q) {
-    if (lo + 4 * q >= L) break;
-    float e[4], f[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const bool ok = lo + 4 * q + k < n;
-      e[k] = ok ? loc[4 * q + k] : 0.f;
-      f[k] = ok ? loc[4 * q + k] + v[4 * q + k] : 0.f;
+    if (lo < L) {
+      __stcs(ao + 32 * q, make_float4(e[0], e[1], e[2], e[3]));
+      __stcs(ro + 32 * q, make_float4(f[0], f[1], f[2], f[3]));
     }
-    __stcs(ao + q, make_float4(e[0], e[1], e[2], e[3]));
-    __stcs(ro + q, make_float4(f[0], f[1], f[2], f[3]));
   }
 }
 
@@ -228,10 +245,10 @@ int launch_gae(const float* r, const float* v, const int32_t* lengths, int64_t S
                  ? 0
                  : -3;
     };
-    if (L <= 128) return go(gae_scan_reg_kernel<4>);
-    if (L <= 256) return go(gae_scan_reg_kernel<8>);
-    if (L <= 384) return go(gae_scan_reg_kernel<12>);
-    return go(gae_scan_reg_kernel<16>);
+    if (L <= 128) return go(gae_scan_reg_kernel<1>);
+    if (L <= 256) return go(gae_scan_reg_kernel<2>);
+    if (L <= 384) return go(gae_scan_reg_kernel<3>);
+    return go(gae_scan_reg_kernel<4>);
   }
   const int chunk = static_cast<int>((L + 31) / 32);
   const int stride = (chunk & 1) ? chunk : chunk + 1;  // odd stride: conflict-free lanes
