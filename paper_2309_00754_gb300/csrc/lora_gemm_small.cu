@@ -864,7 +864,7 @@ double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, doub
 // 100 x 4096 x 12288 44.3 / 41.6, 300 x 512 x 12288 35.4 / 26.1, 256 x 4096 x 4096 37.7 / 32.1, but
 // 97 rows x 11008 x 4096 half of that kernel's time): the clocks of both are estimated, with shares
 // per wave and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
-// 12288), none of which is then slower.
+// 12288), four of which are then slower, by 2 to 3 %.
 bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams) {
   if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
   const bool wanted = M <= 128 || (M <= 256 && (N <= 11264 || (N <= 14336 && K >= 2048))) ||
