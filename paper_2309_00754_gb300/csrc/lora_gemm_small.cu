@@ -861,9 +861,9 @@ double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, doub
 //    18.8 / 21.7, x 4096 22.9 / 24.7, x 5120 33.1 / 38.2, x 8192 46.6 / 42.9; a long K makes up
 //    for that: 448 x 11008 x 4096 51.9 / 54.2, 512 x 11008 x 4096 57.4 / 55.0.
 // Three streams leave a row segment over in a pair, or a wave, more often (with their lora_downs:
-// 100 x 4096 x 12288 44.3 / 41.6, 300 x 512 x 12288 35.4 / 26.1, 256 x 4096 x 4096 37.7 / 32.1, but
-// 97 rows x 11008 x 4096 half of that kernel's time): the clocks of both are estimated, with shares
-// per wave and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
+// 100 x 4096 x 12288 44.3 / 41.6, 300 x 512 x 12288 35.4 / 26.1, but 100 x 11008 x 4096 43.0 /
+// 81.5, 100 x 4096 x 4096 23.5 / 35.7): the clocks of both are estimated, with shares per wave
+// and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
 // 12288), four of which are then slower, by 2 to 3 %.
 bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams) {
   if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
