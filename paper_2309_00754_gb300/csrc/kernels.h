@@ -75,7 +75,9 @@ int* device_error_word();
 
 int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream);
 // The same linear for few token rows per stream (lora_gemm_small.cu), which
-// launch_dual_lora_gemm_tc takes where small_gemm_wanted.
+// launch_dual_lora_gemm_tc takes where small_gemm_wanted. kSmallGemmNoFit: nothing was launched, since
+// the device (a partition of it) holds no cluster of the kernel; the tile kernel serves the call.
+constexpr int kSmallGemmNoFit = 1;
 bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams);
 int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream);
 // TMA map over a row-major [rows, cols] bf16 (or fp32) matrix with row stride ld elements:

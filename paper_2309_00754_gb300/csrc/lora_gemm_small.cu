@@ -899,7 +899,7 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   s.both = a.shared_x && lora_on && a.y_off != nullptr;
   Config best{};
   choose_width(s, a.K, a.N, a.epi, dev, 6000.0, &best);
-  if (best.bn == 0) return -4;
+  if (best.bn == 0) return kSmallGemmNoFit;
   const int bn = best.bn;
 
   Params p{};

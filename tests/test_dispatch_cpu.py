@@ -1,0 +1,88 @@
+"""Which kernels a call takes, without a GPU: the library's objects linked to a fake CUDA runtime
+(fake_cudart.cpp) that records launches and answers the device queries as the test says."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2309_00754_gb300 import build as B
+from paper_2309_00754_gb300 import hydra as H
+
+P = 1 << 20  # a 16-byte aligned address; the fake runtime dereferences none
+BIG = 1 << 40
+
+
+@pytest.fixture(scope="session")
+def built(tmp_path_factory):
+    B.build()
+    objs = [os.path.join(B.BUILD, os.path.basename(s)[:-3] + ".o") for s in B.sources()]
+    if not all(os.path.exists(o) for o in objs):
+        B.build(force=True)
+    so = str(tmp_path_factory.mktemp("fake") / "libhydra_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B._nvcc()))), "include")
+    fake = os.path.join(os.path.dirname(os.path.abspath(__file__)), "fake_cudart.cpp")
+    subprocess.run(["g++", "-shared", "-fPIC", "-std=c++17", "-Wl,-Bsymbolic", "-I", cuda, fake, *objs, "-o", so],
+                   check=True)
+    return so
+
+
+class Fake:
+    def __init__(self, so):
+        self.lib = ctypes.CDLL(so)
+        for name, (res, args) in H._SIGNATURES.items():
+            f = getattr(self.lib, name)
+            f.restype, f.argtypes = res, args
+        self.lib.fake_launches.restype = ctypes.c_char_p
+
+    def device(self, device=0, sms=152, pairs=76, quads=36, error=0):
+        self.lib.fake_device(device, sms, pairs, quads, error)
+
+    def launches(self):
+        """[(kernel, grid x, y, z, cluster)] since the last call."""
+        out = [line.split() for line in self.lib.fake_launches().decode().splitlines()]
+        self.lib.fake_clear()
+        return [(v[0], *map(int, v[1:])) for v in out]
+
+    def linear(self, m, k, n, streams=2, r=0):
+        """Kernels of one LoRA linear of 1 to 3 streams, its lora_downs left out."""
+        if streams == 3:
+            rc = self.lib.hydra_lora_linear_tri(P, 2 * P, 3 * P, m, k, n, P, P, P, P, P, r, 1.0, P, P, P, 0, P, BIG, None)
+        else:
+            rc = self.lib.hydra_lora_linear_algo(P, 2 * P if streams == 2 else None, m, k, n, P, P, P, r, 1.0, P, P, 0,
+                                                 P, BIG, 1, None)
+        assert rc == 0, H.status_string(rc)
+        return [v for v in self.launches() if "lora_down" not in v[0]]
+
+    def attention(self, nseq, p, heads):
+        d = 128 * heads
+        assert self.lib.hydra_causal_attention(P, nseq, p, 3 * d, heads, 128, P, d, None) == 0
+        (v,) = self.launches()
+        return v
+
+
+@pytest.fixture()
+def fake(built, tmp_path):
+    """A library of its own for each test: nothing cached by another one."""
+    so = str(tmp_path / "lib.so")
+    f = Fake(shutil.copy(built, so))
+    f.device()
+    return f
+
+
+def _small(v):
+    return "lora_gemm_small_kernel" in v[0]
+
+
+def test_linear_falls_back_where_no_cluster_fits(fake):
+    """A partition that holds no cluster of four CTAs (or none at all): the tile kernel serves the call."""
+    assert all(_small(v) for v in fake.linear(97, 4096, 4096) + fake.linear(97, 4096, 12288))
+    fake.device(device=1, quads=0)
+    (two,), (one,) = fake.linear(97, 4096, 4096), fake.linear(97, 4096, 12288)
+    assert "dual_lora_gemm_kernel" in two[0] and _small(one)  # two K slices and one
+    fake.device(device=2, pairs=0, quads=0)
+    for streams in (1, 2, 3):
+        for m, kernel in ((1, "dual_lora_gemm_kernel"), (128, "dual_lora_gemm_kernel"), (200, "dual_lora_gemm_2cta_kernel")):
+            (v,) = fake.linear(m, 4096, 4096, streams)
+            assert kernel in v[0]
