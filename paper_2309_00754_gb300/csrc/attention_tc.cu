@@ -715,21 +715,46 @@ int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld
   };
   static thread_local OrderChoice last = {-1, -1, -1, 0, 0};
   if (last.nseq != nseq || last.P != P || last.heads != n_heads || last.grid != grid) {
-    const int lone = nunits > static_cast<int64_t>(grid) ? kLoneFirst : 0;
-    auto busiest = [&](int order) {
-      std::vector<int64_t> load(grid, 0);
-      UnitCursor c;
-      for (int64_t t = 0; t < nunits; ++t) {
-        c.t = static_cast<int>(t);
-        c.decode(static_cast<int>(P), static_cast<int>(n_heads), static_cast<int>(nseq), order | lone,
+    int mode = kGrouped;  // one unit per CTA at most: the orders load the CTAs alike
+    if (nunits > static_cast<int64_t>(grid)) {
+      const int64_t groups = n_heads * nseq, npairs = nunits / groups;
+      std::vector<int> blocks(npairs);  // key blocks of the units, longest first
+      for (int64_t i = 0; i < npairs; ++i) {
+        UnitCursor c;
+        c.t = static_cast<int>(i * groups);
+        c.decode(static_cast<int>(P), static_cast<int>(n_heads), static_cast<int>(nseq), kLongest | kLoneFirst,
                  static_cast<int>(grid));
-        load[t % grid] += c.nblk;
+        blocks[i] = c.nblk;
       }
-      return *std::max_element(load.begin(), load.end());
-    };
-    const int64_t lf = busiest(kLongest), gr = busiest(kGrouped), ro = busiest(kRotated);
-    const int order = std::min(gr, ro) * 20 <= lf * 21 ? (ro < gr ? kRotated : kGrouped) : kLongest;
-    last = {nseq, P, n_heads, grid, order | lone};
+      // key blocks of each CTA in each order, unit by unit; no divisions, as a program with a new
+      // shape each call runs this each time (8 x 1000 x 32 heads: 28 us by decoding every unit
+      // in the three orders, 4 so)
+      std::vector<int64_t> load[3];
+      for (auto& v : load) v.assign(grid, 0);
+      unsigned a = 0, b = 0;
+      for (int64_t i = 0; i < npairs; ++i)
+        for (int64_t g = 0; g < groups; ++g) {
+          load[kLongest][a] += blocks[i];
+          if (++a == grid) a = 0;
+        }
+      for (int64_t g = 0; g < groups; ++g) {
+        int64_t k = g * npairs / grid % npairs;
+        for (int64_t i = 0; i < npairs; ++i) {
+          load[kGrouped][b] += blocks[i];
+          load[kRotated][b] += blocks[k];
+          if (++b == grid) b = 0;
+          if (++k == npairs) k = 0;
+        }
+      }
+      int64_t most[3];
+      for (int o = 0; o < 3; ++o) most[o] = *std::max_element(load[o].begin(), load[o].end());
+      const int64_t together = std::min(most[kGrouped], most[kRotated]);
+      const int order = together * 20 > most[kLongest] * 21 ? kLongest
+                        : most[kRotated] < most[kGrouped]   ? kRotated
+                                                            : kGrouped;
+      mode = order | kLoneFirst;
+    }
+    last = {nseq, P, n_heads, grid, mode};
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(head_dim));
   const bool ragged = (P - 1) % kBQ < kBQ - 32;
@@ -739,9 +764,7 @@ int launch_causal_attention(const void* qkv, int64_t nseq, int64_t P, int64_t ld
   case mode:         \
     return ragged ? launch_form<mode, true>(l) : launch_form<mode, false>(l)
   switch (last.mode) {
-    HY_ATT(kLongest);
     HY_ATT(kGrouped);
-    HY_ATT(kRotated);
     HY_ATT(kLongest | kLoneFirst);
     HY_ATT(kGrouped | kLoneFirst);
     HY_ATT(kRotated | kLoneFirst);

@@ -41,6 +41,12 @@ void fake_device(int device, int sms, int pair_clusters, int quad_clusters, int 
 int fake_cluster_queries() { return g_cluster_queries; }
 const char* fake_launches() { return g_log.c_str(); }
 void fake_clear() { g_log.clear(); }
+const char* fake_kernels() {  // every kernel of the library, one per line
+  static std::string all;
+  all.clear();
+  for (auto& n : g_names) all += n.second + "\n";
+  return all.c_str();
+}
 
 // the runtime's functions that the library calls
 cudaError_t cudaGetDevice(int* d) { return *d = g_device, cudaSuccess; }

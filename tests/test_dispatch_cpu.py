@@ -34,7 +34,7 @@ class Fake:
         for name, (res, args) in H._SIGNATURES.items():
             f = getattr(self.lib, name)
             f.restype, f.argtypes = res, args
-        self.lib.fake_launches.restype = ctypes.c_char_p
+        self.lib.fake_launches.restype = self.lib.fake_kernels.restype = ctypes.c_char_p
 
     def device(self, device=0, sms=152, pairs=76, quads=36, error=0):
         self.lib.fake_device(device, sms, pairs, quads, error)
@@ -86,3 +86,10 @@ def test_linear_falls_back_where_no_cluster_fits(fake):
         for m, kernel in ((1, "dual_lora_gemm_kernel"), (128, "dual_lora_gemm_kernel"), (200, "dual_lora_gemm_2cta_kernel")):
             (v,) = fake.linear(m, 4096, 4096, streams)
             assert kernel in v[0]
+
+
+def test_every_compiled_attention_form_is_taken_by_some_shape(fake):
+    forms = {k for k in fake.lib.fake_kernels().decode().split() if "causal_attention" in k}
+    taken = {fake.attention(nseq, p, heads)[0] for nseq in (1, 2, 3, 8, 13, 16, 20, 27, 40)
+             for p in (97, 128, 300, 384, 390, 640, 700, 768, 900, 1000, 1024) for heads in (1, 5, 12, 32)}
+    assert forms == taken

@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
     (8, 900, 12),   # 8 tiles, 384 units of four lengths
     (40, 129, 5),   # 2 tiles, a last tile of one row
     (160, 97, 1),   # one tile, rows 96 .. in its last warp
+    (5, 384, 16),   # 3 tiles, 160 units in rotated order, whole tiles
+    (1, 300, 1),    # two units, the last tile alone and ragged
 ])
 def test_causal_attention_orders(nseq, P, heads):
     g = torch.Generator(device="cuda").manual_seed(nseq * P)
