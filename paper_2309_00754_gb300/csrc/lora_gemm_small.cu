@@ -37,8 +37,7 @@
 // at 6.6 TB/s of W; about 6 us of the 25.6 are set-up, first loads, drain and stores.
 #include <float.h>
 
-#include <mutex>
-#include <vector>
+#include <atomic>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -761,19 +760,17 @@ bool allow_smem(int dev) {
   return done[dev] = true;
 }
 
-// Clusters of 2 ks CTAs with this shared memory that the device holds at once (the same for every
-// epilogue: shared memory and threads decide).
-int resident_clusters(int dev, int ks, int smem) {
-  static std::mutex mu;
-  static std::vector<std::pair<long long, int>> cache;
-  const long long key = static_cast<long long>(dev) << 40 | static_cast<long long>(ks) << 32 | smem;
-  std::lock_guard<std::mutex> lock(mu);
-  for (auto& e : cache)
-    if (e.first == key) return e.second;
+// Clusters of 2 ks CTAs that the device holds at once (0: none, or it does not say, which is not kept).
+// Every layout takes more than half of an SM's shared memory (131 KB and more), so an SM holds
+// one CTA whatever the width and the epilogue: 76 and 36 on GB300 from 116 KB up.
+int resident_clusters(int dev, int ks) {
+  static std::atomic<int> known[64][2];  // the answer + 1; dev < 64: allow_smem
+  int n = known[dev][ks - 1].load(std::memory_order_relaxed) - 1;
+  if (n >= 0) return n;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * ks * 128));
   cfg.blockDim = dim3(smallm::NUM_THREADS);
-  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg.dynamicSmemBytes = kSmemMax;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(2 * ks);
@@ -781,12 +778,11 @@ int resident_clusters(int dev, int ks, int smem) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel<smallm::EPI_STORE>, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    n = 0;
+    return 0;
   }
-  if (cache.size() < 256) cache.emplace_back(key, n);
+  known[dev][ks - 1].store(n + 1, std::memory_order_relaxed);
   return n;
 }
 
@@ -823,15 +819,15 @@ int box_of(int epi) { return epi == smallm::EPI_SWIGLU ? 128 : 64; }
 // (2 (seg + bn / 2)), and a wave `per_wave` clocks of set-up, first loads and drain.
 double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, double per_wave, Config* best) {
   const int64_t kb = (K + smallm::BK - 1) / smallm::BK;
+  const int fit = resident_clusters(dev, s.ks);
   double best_t = 1e30;
+  if (fit < 1) return best_t;
   for (int bn : {256, 224, 192, 160, 128, 96, 64}) {
     if (s.ks == 2 && bn % (s.paired ? 128 : 64) != 0) continue;  // whole chunks for each slice
     if (s.paired && bn / 2 / gcd(bn / 2, box_of(epi)) > smallm::kMaxBoxes) continue;
     if (epi == smallm::EPI_LOGSOFTMAX && bn != 256) continue;
     Config c{};
     if (!lay_out(s, bn, &c)) continue;
-    const int fit = resident_clusters(dev, s.ks, c.smem);
-    if (fit < 1) continue;
     const int fill = 2 * (s.seg + bn / 2), mma = 2 * bn;
     const double item = 2.0 * (fill > mma ? fill : mma);
     const int64_t waves = (tiles_of(s, N, epi, bn) + fit - 1) / fit;

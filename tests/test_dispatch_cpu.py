@@ -93,3 +93,18 @@ def test_every_compiled_attention_form_is_taken_by_some_shape(fake):
     taken = {fake.attention(nseq, p, heads)[0] for nseq in (1, 2, 3, 8, 13, 16, 20, 27, 40)
              for p in (97, 128, 300, 384, 390, 640, 700, 768, 900, 1000, 1024) for heads in (1, 5, 12, 32)}
     assert forms == taken
+
+
+def test_occupancy_is_asked_once_per_device_and_a_failed_query_is_not_kept(fake):
+    fake.device(error=1)
+    (v,) = fake.linear(97, 4096, 12288)
+    assert "dual_lora_gemm_kernel" in v[0]
+    before = fake.lib.fake_cluster_queries()
+    for device in range(3):
+        fake.device(device=device)
+        for m in range(1, 513, 8):
+            for n in (520, 1032, 4096, 12288):
+                for r in (0, 16):
+                    assert all(_small(v) for v in fake.linear(min(m, 128), 4096, n, 2, r))
+                    fake.linear(m, 4096, n, 1, r), fake.linear(m, 4096, n, 3, r)
+    assert fake.lib.fake_cluster_queries() - before <= 6  # one and two K slices
