@@ -98,8 +98,10 @@ hydra_status lora_linear_impl(const void* x_off, const void* x_on, int64_t M, in
   if (err == nullptr) return HYDRA_ERR_CUDA;
 
   const void* xo = shared_x ? x_off : x_on;
+  const bool use_gemv = (algo == 2) || (algo == 0 && rows <= hydra::kGemvMaxRows);
+  const bool settle = !use_gemv || hydra::gemv_beside_lora_down(rows, K, N);
   if (lora && !u_given) {
-    if (hydra::launch_lora_down(xo, M, K, A, r, s, workspace, st) != 0) return HYDRA_ERR_CUDA;
+    if (hydra::launch_lora_down(xo, M, K, A, r, s, workspace, settle, st) != 0) return HYDRA_ERR_CUDA;
   }
   hydra::GemmArgs g;
   g.x_off = x_off;
@@ -118,13 +120,12 @@ hydra_status lora_linear_impl(const void* x_off, const void* x_on, int64_t M, in
   g.err = err;
   g.epi = epi;
   g.single_cta = algo == 3;
-  g.x_settled = lora && !u_given;
+  g.x_settled = lora && !u_given && settle;
   if (epi == kEpiRope) {
     g.rope_P = rope->P;
     g.rope_cols = rope->cols;
     g.rope_table = rope->table;
   }
-  const bool use_gemv = (algo == 2) || (algo == 0 && rows <= hydra::kGemvMaxRows);
   const int rc = use_gemv ? hydra::launch_dual_lora_gemv(g, st) : hydra::launch_dual_lora_gemm_tc(g, st);
   return rc == 0 ? HYDRA_OK : HYDRA_ERR_CUDA;
 }
@@ -199,7 +200,7 @@ hydra_status hydra_lora_down(const void* x_on, int64_t M, int64_t K, const void*
   if (K % 8 != 0 || r % 8 != 0) return HYDRA_ERR_ALIGN;
   if (!aligned16(x_on) || !aligned16(A) || !aligned16(u)) return HYDRA_ERR_ALIGN;
   if (M == 0) return HYDRA_OK;
-  return hydra::launch_lora_down(x_on, M, K, A, r, s, u, static_cast<cudaStream_t>(stream)) == 0
+  return hydra::launch_lora_down(x_on, M, K, A, r, s, u, false, static_cast<cudaStream_t>(stream)) == 0
              ? HYDRA_OK
              : HYDRA_ERR_CUDA;
 }
@@ -333,8 +334,8 @@ hydra_status hydra_lora_linear_tri(const void* x_off, const void* x_act, const v
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   void* u_a = ws;
   void* u_c = lora_a || lora_c ? ws + round_up(static_cast<size_t>(M) * r * 2, 256) : nullptr;
-  if (lora_a && hydra::launch_lora_down(x_act, M, K, A_act, r, s, u_a, st) != 0) return HYDRA_ERR_CUDA;
-  if (lora_c && hydra::launch_lora_down(x_crit, M, K, A_crit, r, s, u_c, st) != 0) return HYDRA_ERR_CUDA;
+  if (lora_a && hydra::launch_lora_down(x_act, M, K, A_act, r, s, u_a, true, st) != 0) return HYDRA_ERR_CUDA;
+  if (lora_c && hydra::launch_lora_down(x_crit, M, K, A_crit, r, s, u_c, true, st) != 0) return HYDRA_ERR_CUDA;
   hydra::GemmArgs g;
   g.x_off = x_off;
   g.x_on = x_act;
@@ -398,7 +399,7 @@ hydra_status hydra_lm_head_logprobs(const void* h_off, const void* h_on, int64_t
   void* u = ws + round_up(2 * static_cast<size_t>(M) * nt * 8, 256) +
             round_up(2 * static_cast<size_t>(M) * 4, 256);
   const void* xo = shared_x ? h_off : h_on;
-  if (r > 0 && hydra::launch_lora_down(xo, M, d, A, r, s, u, st) != 0) return HYDRA_ERR_CUDA;
+  if (r > 0 && hydra::launch_lora_down(xo, M, d, A, r, s, u, true, st) != 0) return HYDRA_ERR_CUDA;
   hydra::GemmArgs g;
   g.x_off = h_off;
   g.x_on = xo;

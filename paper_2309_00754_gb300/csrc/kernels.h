@@ -70,6 +70,8 @@ struct GemmArgs {
   int64_t lsm_L = 1, lsm_ids_ld = 1, lsm_ids_off = 0;
 };
 
+// Multiprocessors of the current device (0 on failure), asked once per device.
+int sm_count();
 // Device address of the library's error word on the current device (NULL on failure).
 int* device_error_word();
 
@@ -89,6 +91,8 @@ bool make_tma_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols
 // written by a store
 bool make_tma_map_3d(CUtensorMap* map, const void* base, int64_t cols, int64_t rows,
                      int64_t planes, int64_t ld, int64_t plane_stride, int box_rows);
+// Whether the GEMV of these sizes runs beside its lora_down (GemmArgs::x_settled).
+bool gemv_beside_lora_down(int64_t rows, int64_t K, int64_t N);
 int launch_dual_lora_gemv(const GemmArgs& a, cudaStream_t stream);
 
 // Skinny linear (gemm_skinny.cu): y = x W^T for all M <= 128 rows of x, plus u B^T on rows
@@ -109,8 +113,10 @@ struct SkinnyArgs {
 };
 bool skinny_gemm_supported(int64_t M, int64_t K, int64_t N, int64_t r);
 int launch_skinny_gemm_tc(const SkinnyArgs& a, cudaStream_t stream);
+// settle: the kernel lets its dependents start only once everything before it is complete, so that the
+// linear launched right after it may be told x_settled. Without it they start at once, and wait.
 int launch_lora_down(const void* x, int64_t M, int64_t K, const void* A, int64_t r, float s,
-                     void* u, cudaStream_t stream);
+                     void* u, bool settle, cudaStream_t stream);
 // ids of sequence s start at ids + s * ids_ld (ids_ld = L for a dense [S, L] array)
 // merge the per-tile (max, sum exp) partials [rows][n_tiles] (float2) of the reference and
 // actor heads and their sampled-token logits [rows] into logp / reward (as

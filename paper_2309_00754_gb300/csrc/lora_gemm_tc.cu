@@ -977,7 +977,7 @@ static bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t c
   return make_tma_map(map, base, rows, cols, cols, box_rows, f32);
 }
 
-static int sm_count() {
+int sm_count() {
   static int cached[64] = {0};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;

@@ -48,11 +48,12 @@ template <int NT>  // NT n-tiles of 8 ranks
 __global__ void __launch_bounds__(32 * kDownWarps)
     lora_down_kernel(const __nv_bfloat16* __restrict__ x, int M, int K,
                      const __nv_bfloat16* __restrict__ A, int r, float s,
-                     __nv_bfloat16* __restrict__ u, int ck) {
+                     __nv_bfloat16* __restrict__ u, int ck, int settle) {
   __shared__ float red[kDownWarps][16][NT * 8 + 1];
   __shared__ float tile[16][NT * 8];  // this CTA's sum over its warps
+  if (!settle) pdl_launch_dependents();
   pdl_wait();  // x is written by the preceding kernel
-  pdl_launch_dependents();  // after the wait: a dependent may take x as final
+  if (settle) pdl_launch_dependents();  // after the wait, in every CTA: a dependent takes x as final
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, c = lane & 3;
@@ -226,7 +227,7 @@ template <int NT>
 __global__ void __launch_bounds__(kThreads)
     lora_down_stream_kernel(const __grid_constant__ CUtensorMap tm_x,
                             const __grid_constant__ CUtensorMap tm_a, int M, int K, int r, float s,
-                            __nv_bfloat16* __restrict__ u, int ck, int* err) {
+                            __nv_bfloat16* __restrict__ u, int ck, int settle, int* err) {
   using C = Cfg<NT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -259,8 +260,9 @@ __global__ void __launch_bounds__(kThreads)
   // first half of a cluster barrier: its wait, before the first store to another CTA's shared
   // memory, ensures every CTA of the cluster has started
   if (ck > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (!settle) pdl_launch_dependents();
   pdl_wait();  // x is written by the preceding kernel, which may also still read u
-  pdl_launch_dependents();  // after the wait: a dependent may take x as final
+  if (settle) pdl_launch_dependents();  // after the wait, in every CTA: a dependent takes x as final
 
   float d[4][NT][4];
 #pragma unroll
@@ -431,6 +433,15 @@ __device__ __forceinline__ void gv_ldsm_x4(uint32_t addr, uint32_t (&a)[4]) {
                : "r"(addr));
 }
 
+// 16 bytes that another kernel wrote during this one (before pdl_wait()): not a read-only load, which
+// the compiler may move up, but through L1, as every CTA reads the same few lines (8 rows of one
+// input, 256 x 10000: 5.25 us with ld.global.cg, 4.9 so)
+__device__ __forceinline__ uint4 ld_written(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 template <int NT, int kGvWarps, bool kAlias = false>  // kAlias: partial tiles in the ring
 __global__ void __launch_bounds__(32 * kGvWarps)
     dual_lora_gemv_kernel(const __nv_bfloat16* __restrict__ x_off,
@@ -577,7 +588,7 @@ __global__ void __launch_bounds__(32 * kGvWarps)
         const uint4* up = reinterpret_cast<const uint4*>(u + static_cast<size_t>(m) * r);
         const uint4* bp = reinterpret_cast<const uint4*>(B + static_cast<size_t>(n) * r);
         for (int j = 0; j < r / 8; ++j) {
-          const uint4 a4 = __ldcg(up + j), b4 = __ldg(bp + j);  // u may be younger than this launch
+          const uint4 a4 = ld_written(up + j), b4 = __ldg(bp + j);
           const uint32_t* ap = &a4.x;
           const uint32_t* bq = &b4.x;
 #pragma unroll
@@ -634,7 +645,7 @@ void launch_gemv_t(const GemmArgs& a, int nsm, cudaStream_t stream) {
 // still lets every CTA of the launch be resident at once, and at least one k-block per CTA.
 template <int NT>
 int launch_lora_down_stream(const void* x, int64_t M, int64_t K, const void* A, int64_t r,
-                            float s, void* u, int nsm, cudaStream_t stream) {
+                            float s, void* u, bool settle, int nsm, cudaStream_t stream) {
   using C = lds::Cfg<NT>;
   static bool attr = false;
   if (!attr) {
@@ -672,14 +683,14 @@ int launch_lora_down_stream(const void* x, int64_t M, int64_t K, const void* A, 
   const cudaError_t e = cudaLaunchKernelEx(&cfg, lds::lora_down_stream_kernel<NT>, mx, ma,
                                            static_cast<int>(M), static_cast<int>(K),
                                            static_cast<int>(r), s, static_cast<__nv_bfloat16*>(u),
-                                           ck, err);
+                                           ck, settle ? 1 : 0, err);
   return e == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace
 
 int launch_lora_down(const void* x, int64_t M, int64_t K, const void* A, int64_t r, float s,
-                     void* u, cudaStream_t stream) {
+                     void* u, bool settle, cudaStream_t stream) {
   if (M == 0 || r == 0) return 0;
   static int nsm = 0;
   if (nsm == 0) {
@@ -692,10 +703,10 @@ int launch_lora_down(const void* x, int64_t M, int64_t K, const void* A, int64_t
   const auto* ap = static_cast<const __nv_bfloat16*>(A);
   auto* up = static_cast<__nv_bfloat16*>(u);
   if (M >= lds::kBM && K >= 64) {
-    if (r <= 8) return launch_lora_down_stream<1>(x, M, K, A, r, s, u, nsm, stream);
-    if (r <= 16) return launch_lora_down_stream<2>(x, M, K, A, r, s, u, nsm, stream);
-    if (r <= 32) return launch_lora_down_stream<4>(x, M, K, A, r, s, u, nsm, stream);
-    return launch_lora_down_stream<8>(x, M, K, A, r, s, u, nsm, stream);
+    if (r <= 8) return launch_lora_down_stream<1>(x, M, K, A, r, s, u, settle, nsm, stream);
+    if (r <= 16) return launch_lora_down_stream<2>(x, M, K, A, r, s, u, settle, nsm, stream);
+    if (r <= 32) return launch_lora_down_stream<4>(x, M, K, A, r, s, u, settle, nsm, stream);
+    return launch_lora_down_stream<8>(x, M, K, A, r, s, u, settle, nsm, stream);
   }
   const int64_t tiles = (M + 15) / 16;
   const int64_t ny = r <= 32 ? 1 : (r + 63) / 64;
@@ -711,22 +722,30 @@ int launch_lora_down(const void* x, int64_t M, int64_t K, const void* A, int64_t
   const int cki = static_cast<int>(ck);
   cudaError_t e;
   if (r <= 8)
-    e = launch_down(lora_down_kernel<1>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki);
+    e = launch_down(lora_down_kernel<1>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki, settle ? 1 : 0);
   else if (r <= 16)
-    e = launch_down(lora_down_kernel<2>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki);
+    e = launch_down(lora_down_kernel<2>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki, settle ? 1 : 0);
   else if (r <= 32)
-    e = launch_down(lora_down_kernel<4>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki);
+    e = launch_down(lora_down_kernel<4>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki, settle ? 1 : 0);
   else
-    e = launch_down(lora_down_kernel<8>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki);
+    e = launch_down(lora_down_kernel<8>, grid, cki, stream, xp, Mi, Ki, ap, ri, s, up, cki, settle ? 1 : 0);
   return e == cudaSuccess ? 0 : -3;
+}
+
+// Beside its lora_down, the GEMV streams W while u is formed, but is let in only when x is final. With
+// a short K there is little of W to stream, and one wave of 4-warp CTAs does better to be there early
+// (let in at once / beside, us for the two launches: 1 row x 256 x 12288 4.6 / 5.0, 8 x 256 x 10000
+// 4.7 / 4.9, 1 x 512 x 12288 5.9 / 6.0; but 1 x 256 x 4096 3.7 / 3.4, 1 x 512 x 22016 8.8 / 8.6,
+// 1 x 768 x 12288 7.1 / 6.8, 16 rows x 512 x 12288 9.1 / 8.7).
+bool gemv_beside_lora_down(int64_t rows, int64_t K, int64_t N) {
+  const int64_t nsm = sm_count(), blocks = (N + 15) / 16;
+  return !(rows <= 8 && K <= 512 && blocks >= 4 * nsm && blocks <= 6 * nsm);
 }
 
 int launch_dual_lora_gemv(const GemmArgs& a, cudaStream_t stream) {
   const int64_t rows = a.shared_x ? a.M : 2 * a.M;
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return -1;
+  const int nsm = sm_count();
+  if (nsm <= 0) return -1;
   const bool narrow = (a.N + 15) / 16 >= 4LL * nsm;  // enough row blocks for 4-warp CTAs
   if (rows <= 8) {
     if (narrow)

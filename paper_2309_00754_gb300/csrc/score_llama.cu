@@ -120,8 +120,8 @@ int stacked_linear_impl(int prof_class, const void* x, int64_t T, int64_t K, int
   const void* x_crit = static_cast<const uint8_t*>(x) + 2 * xs;
   if (r > 0) {
     ProfScope ps(HYDRA_PROF_LORA_DOWN, st);
-    int e = hydra::launch_lora_down(x_on, T, K, A, r, s, u, st);
-    if (e == 0 && ns == 3) e = hydra::launch_lora_down(x_crit, T, K, A2, r, s, u2, st);
+    int e = hydra::launch_lora_down(x_on, T, K, A, r, s, u, true, st);
+    if (e == 0 && ns == 3) e = hydra::launch_lora_down(x_crit, T, K, A2, r, s, u2, true, st);
     if (e != 0) return e;
   }
   ProfScope ps(prof_class, st);
@@ -378,7 +378,7 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
       // then the LoRA k-blocks accumulated on top for the on stream), the same bits as the
       // stacked form for half the products (§3 Dynamic LoRA: one frozen W, LoRA switched)
       HY_PROF(HYDRA_PROF_ELEMENTWISE, hydra::launch_rmsnorm(h, ly.norm_attn, T, d, c.rms_eps, ident, a, st));
-      HY_PROF(HYDRA_PROF_LORA_DOWN, hydra::launch_lora_down(a, T, d, ly.a_qv, 2 * r, s, u, st));
+      HY_PROF(HYDRA_PROF_LORA_DOWN, hydra::launch_lora_down(a, T, d, ly.a_qv, 2 * r, s, u, true, st));
       ProfScope ps(HYDRA_PROF_GEMM_QKV, st);
       hydra::GemmArgs g;
       g.x_off = a;

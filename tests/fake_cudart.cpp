@@ -14,10 +14,18 @@ std::string g_log;
 int g_device, g_sms = 152, g_clusters[2] = {76, 36}, g_cluster_error, g_cluster_queries;
 char g_symbol[256];
 
-void record(const void* fn, dim3 grid, unsigned cluster) {
+// a kernel's flag on the order of dependent launches: lora_down's `settle`, the GEMV's `x_settled`
+int order_flag(const std::string& name, void** args) {
+  if (name.find("lora_down") != std::string::npos) return *static_cast<int*>(args[8]);
+  if (name.find("dual_lora_gemv") != std::string::npos) return *static_cast<int*>(args[13]);
+  return -1;
+}
+
+void record(const void* fn, dim3 grid, unsigned cluster, void** args) {
   auto it = g_names.find(fn);
-  g_log += (it == g_names.end() ? std::string("?") : it->second) + " " + std::to_string(grid.x) + " " +
-           std::to_string(grid.y) + " " + std::to_string(grid.z) + " " + std::to_string(cluster) + "\n";
+  const std::string name = it == g_names.end() ? "?" : it->second;
+  g_log += name + " " + std::to_string(grid.x) + " " + std::to_string(grid.y) + " " + std::to_string(grid.z) + " " +
+           std::to_string(cluster) + " " + std::to_string(order_flag(name, args)) + "\n";
 }
 
 CUresult encode_tiled(CUtensorMap* map, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -80,11 +88,11 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** fn, unsigned, u
   if (q) *q = cudaDriverEntryPointSuccess;
   return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* fn, void**) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* fn, void** args) {
   unsigned cluster = 1;
   for (unsigned i = 0; i < cfg->numAttrs; ++i)
     if (cfg->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = cfg->attrs[i].val.clusterDim.x;
-  return record(fn, cfg->gridDim, cluster), cudaSuccess;
+  return record(fn, cfg->gridDim, cluster, args), cudaSuccess;
 }
 
 // what the compiler's registration and launch stubs call
@@ -105,7 +113,7 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* smem, vo
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* fn) {
   return *k = static_cast<cudaKernel_t>(const_cast<void*>(fn)), cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void**, size_t, cudaStream_t) {
-  return record(k, grid, 1), cudaSuccess;
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void** args, size_t, cudaStream_t) {
+  return record(k, grid, 1, args), cudaSuccess;
 }
 }

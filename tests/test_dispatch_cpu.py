@@ -40,7 +40,7 @@ class Fake:
         self.lib.fake_device(device, sms, pairs, quads, error)
 
     def launches(self):
-        """[(kernel, grid x, y, z, cluster)] since the last call."""
+        """[(kernel, grid x, y, z, cluster, order flag)] since the last call."""
         out = [line.split() for line in self.lib.fake_launches().decode().splitlines()]
         self.lib.fake_clear()
         return [(v[0], *map(int, v[1:])) for v in out]
@@ -108,3 +108,24 @@ def test_occupancy_is_asked_once_per_device_and_a_failed_query_is_not_kept(fake)
                     assert all(_small(v) for v in fake.linear(min(m, 128), 4096, n, 2, r))
                     fake.linear(m, 4096, n, 1, r), fake.linear(m, 4096, n, 3, r)
     assert fake.lib.fake_cluster_queries() - before <= 6  # one and two K slices
+
+
+def test_gemv_takes_x_as_final_only_after_a_lora_down_that_settles(fake):
+    """`x_settled` of the GEMV and `settle` of the lora_down launched right before it go together; few
+    rows of a short K in one wave of 4-warp CTAs are let in at once."""
+    early = set()
+    for m in range(1, 9):
+        for k in (8, 256, 512, 520, 4096):
+            for n in (8, 776, 4096, 9712, 9728, 12288, 14592, 14600, 22016):
+                for shared in (True, False):
+                    assert fake.lib.hydra_lora_linear(P, None if shared else 2 * P, m, k, n, P, P, P, 8, 1.0, P, P, 0, P,
+                                                      BIG, None) == 0
+                    down, gemv = fake.launches()
+                    assert "lora_down" in down[0] and "gemv" in gemv[0] and down[5] == gemv[5]
+                    if not gemv[5]:
+                        early.add((m if shared else 2 * m, k, n))
+    assert early == {(m, k, n) for m in range(1, 9) for k in (8, 256, 512) for n in (9728, 12288, 14592)}
+    # the two calls apart: the GEMV waits
+    assert fake.lib.hydra_lora_down(P, 1, 4096, P, 8, 1.0, P, None) == 0
+    assert fake.lib.hydra_dual_linear(P, 2 * P, 1, 4096, 4096, P, P, P, 8, P, P, 0, 0, None) == 0
+    assert [v[5] for v in fake.launches()] == [0, 0]
