@@ -15,9 +15,10 @@
 // Larger ones take two launches, the second a programmatic dependent launch:
 //   moments:  per block, the valid count n and (with whitening) the sums of a - c and
 //             (a - c)^2 over the valid advantages, c = adv[0] a common shift;
-//   loss:     every block merges those partials (or takes the caller's moments) into
-//             (mean, 1 / std, 1 / n), all in the same order, while its first loads are in
-//             flight; streams float4 chunks of the flattened [S, L] batch; chunks without a
+//             The caller's moments, if given, take the place of this pass: one thread turns
+//             them into (mean, 1 / std, 1 / n);
+//   loss:     every block merges those partials into (mean, 1 / std, 1 / n), all in the same
+//             order, while its first loads are in flight; streams float4 chunks of the flattened [S, L] batch; chunks without a
 //             valid token are written as zero gradients without reading the inputs; per-block
 //             sums go to the workspace, and the block that finishes last merges them, in a
 //             fixed order, into the statistics. (A launch of its own for either merge cost
@@ -360,6 +361,12 @@ struct Moments {
   double n, mean, m2;
   float c_mean, inv_std, inv_n;
 };
+static_assert(sizeof(Moments) <= sizeof(MomPart) * kPpoMaxMomentBlocks, "ppo_ext_kernel writes it there");
+
+__device__ __forceinline__ Moments load_moments(const Moments* p) {
+  return Moments{__ldcg(&p->n),      __ldcg(&p->mean),    __ldcg(&p->m2),
+                 __ldcg(&p->c_mean), __ldcg(&p->inv_std), __ldcg(&p->inv_n)};
+}
 
 __device__ __forceinline__ Moments moments_from_ext(const double* ext) {
   Moments m;
@@ -430,6 +437,16 @@ __global__ void __launch_bounds__(kPpoThreads)
     moments[1] = m.mean;
     moments[2] = m.m2;
   }
+  pdl_launch_dependents();
+}
+
+// The caller's moments for the loss pass, in the place of the moments partials. (With
+// the fp64 root and quotients in every thread of the loss pass 16384 x 400 tokens took 27.3 us, with
+// every thread reading one thread's results 26.1, with one thread of each block 22.1.)
+__global__ void ppo_ext_kernel(const double* __restrict__ ext, Moments* __restrict__ out, unsigned* ticket) {
+  pdl_wait();
+  *out = moments_from_ext(ext);
+  *ticket = 0;
   pdl_launch_dependents();
 }
 
@@ -512,7 +529,15 @@ __device__ __forceinline__ void loss_compute(const LossChunk<VEC>& x, float mean
   }
 }
 
-// The statistics of a batch from its loss sums.
+// The moments among the statistics.
+__device__ __forceinline__ void write_moment_stats(double* stats, const Moments& m) {
+  stats[4] = m.mean;
+  stats[5] = m.n > 0.0 ? sqrt(m.m2 / m.n) : 0.0;
+  stats[6] = m.n;
+}
+
+// The statistics of a batch from its loss sums (kMomentsDone: all but the moments).
+template <bool kMomentsDone = false>
 __device__ __forceinline__ void write_stats(double* stats, const float (&v)[kLossSums], int nclip,
                                             const Moments& m, bool report_moments) {
   const double n = m.n, inv = n > 0.0 ? 1.0 / n : 0.0;
@@ -520,6 +545,7 @@ __device__ __forceinline__ void write_stats(double* stats, const float (&v)[kLos
   stats[1] = static_cast<double>(v[1]) * inv;
   stats[2] = static_cast<double>(nclip) * inv;
   stats[3] = static_cast<double>(v[2]) * inv;
+  if (kMomentsDone) return;
   if (report_moments) {
     stats[4] = m.mean;
     stats[5] = n > 0.0 ? sqrt(m.m2 * inv) : 0.0;
@@ -538,7 +564,7 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
                     const float* __restrict__ adv, const float* __restrict__ ret,
                     const float* __restrict__ val, const int32_t* __restrict__ lengths, int S,
                     int L, float eps, const MomPart* __restrict__ mpart, int Gm,
-                    const double* __restrict__ ext, int report_moments, LossPart* __restrict__ lpart,
+                    const Moments* __restrict__ ext, int report_moments, LossPart* __restrict__ lpart,
                     unsigned* ticket, float* __restrict__ grad_logp, float* __restrict__ grad_val,
                     double* __restrict__ stats, int* err) {
   __shared__ float sh[kLossSums][kPpoWarps];
@@ -554,9 +580,17 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
   LossAcc acc;
   LossChunk<VEC> x, y;
   loss_load<VEC, ODD>(x, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
-  const Moments mom = ext != nullptr ? moments_from_ext(ext)
-                                     : merge_moments(mpart, Gm, WHITEN ? __ldg(adv) : 0.f, sh, shk);
+  Moments mom;
+  if (ext != nullptr) {  // one thread: every thread of the grid at the same line took 2 us
+    __shared__ Moments given;
+    if (threadIdx.x == 0) given = load_moments(ext);
+    __syncthreads();
+    mom = given;
+  } else {
+    mom = merge_moments(mpart, Gm, WHITEN ? __ldg(adv) : 0.f, sh, shk);
+  }
   const float mean = mom.c_mean, inv_std = mom.inv_std, inv_n = mom.inv_n;
+  if (WHITEN && tid == 0) write_moment_stats(stats, mom);  // the fp64 root off the end of the launch
   while (true) {
     if (cur.s >= S) {
       loss_compute<VEC, ODD, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
@@ -603,7 +637,7 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
 #pragma unroll
     for (int q = 0; q < kLossSums; ++q) v[q] = k[q].s;
     block_sums<kLossSums>(v, nclip, sh, shk);
-    if (threadIdx.x == 0) write_stats(stats, v, nclip, mom, report_moments != 0);
+    if (threadIdx.x == 0) write_stats<WHITEN>(stats, v, nclip, mom, report_moments != 0);
   }
   pdl_launch_dependents();
 }
@@ -653,7 +687,10 @@ __global__ void __launch_bounds__(kPpoThreads)
   loss_load<VEC, ODD>(x, cur, logp_new, logp_old, adv, ret, val, S, L, ds, dt, lengths, err);
   Moments mom;
   if (ext != nullptr) {
-    mom = moments_from_ext(ext);
+    __shared__ Moments given;
+    if (threadIdx.x == 0) given = moments_from_ext(ext);
+    __syncthreads();
+    mom = given;
     if (c > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   } else {
     int n = 0;
@@ -855,14 +892,20 @@ int launch_ppo_loss(const float* logp_new, const float* logp_old, const float* a
     else e = whiten ? go(ppo_small_kernel<1, false, true>) : go(ppo_small_kernel<1, false, false>);
     return e == cudaSuccess ? 0 : -3;
   }
-  // the caller's moments need no pass over the batch: an empty one clears the ticket
   const WsLayout w = layout(ws);
-  const int Gm = launch_moments(adv, lengths, ext_moments != nullptr ? 0 : Si, Li, whiten, w, err, st);
-  if (Gm < 0) return Gm;
+  Moments* ext = nullptr;
+  int Gm = 0;
+  if (ext_moments != nullptr) {
+    ext = reinterpret_cast<Moments*>(w.mom);
+    if (launch_pdl(ppo_ext_kernel, dim3(1), dim3(1), 0, st, ext_moments, ext, w.ticket) != cudaSuccess) return -3;
+  } else {
+    Gm = launch_moments(adv, lengths, Si, Li, whiten, w, err, st);
+    if (Gm < 0) return Gm;
+  }
   auto go = [&](auto kernel) {
     const int G = one_wave(kernel, items, kPpoMaxLossBlocks);
     return launch_pdl(kernel, dim3(G), dim3(kPpoThreads), 0, st, logp_new, logp_old, adv, ret, val,
-                      lengths, Si, Li, eps, static_cast<const MomPart*>(w.mom), Gm, ext_moments,
+                      lengths, Si, Li, eps, static_cast<const MomPart*>(w.mom), Gm, static_cast<const Moments*>(ext),
                       report, w.loss, w.ticket, grad_logp, grad_val, stats, err);
   };
   if (v4 && L % 4 == 0) e = whiten ? go(ppo_loss_kernel<4, false, true>) : go(ppo_loss_kernel<4, false, false>);

@@ -129,3 +129,11 @@ def test_gemv_takes_x_as_final_only_after_a_lora_down_that_settles(fake):
     assert fake.lib.hydra_lora_down(P, 1, 4096, P, 8, 1.0, P, None) == 0
     assert fake.lib.hydra_dual_linear(P, 2 * P, 1, 4096, 4096, P, P, P, 8, P, P, 0, 0, None) == 0
     assert [v[5] for v in fake.launches()] == [0, 0]
+
+
+@pytest.mark.parametrize("whiten", [0, 1])
+def test_losses_with_the_callers_moments_make_no_pass_over_the_batch_for_them(fake, whiten):
+    """One thread turns them into the loss pass's coefficients, once for all its blocks."""
+    assert fake.lib.hydra_ppo_loss(P, P, P, P, P, None, 1000, 400, 0.2, whiten, P, P, P, P, P, BIG, None) == 0
+    first, second = fake.launches()
+    assert "ppo_ext_kernel" in first[0] and first[1:4] == (1, 1, 1) and "ppo_loss_kernel" in second[0]
