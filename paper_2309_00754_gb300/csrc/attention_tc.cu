@@ -195,10 +195,6 @@ __device__ __forceinline__ void tc_st_x32(uint32_t taddr, const uint32_t (&u)[32
       : "memory");
 }
 
-__device__ __forceinline__ void tc_wait_st() {
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
 // D[tmem] (+)= A[tmem] * B[smem]^T, bf16 inputs, fp32 accumulation: A is M rows (TMEM lanes)
 // by K = 16 elements, two bf16 per 32-bit column (8 columns from a_tmem)
 __device__ __forceinline__ void tc_mma_ts_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,

@@ -76,11 +76,13 @@ int sm_count();
 int* device_error_word();
 
 int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream);
-// The same linear for few token rows per stream (lora_gemm_small.cu), which
-// launch_dual_lora_gemm_tc takes where small_gemm_wanted. kSmallGemmNoFit: nothing was launched, since
-// the device (a partition of it) holds no cluster of the kernel; the tile kernel serves the call.
-constexpr int kSmallGemmNoFit = 1;
-bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams);
+// The same linear for few token rows per stream (lora_gemm_small.cu), which launch_dual_lora_gemm_tc takes
+// for some sizes. It sums in the tile kernel's order, so either may serve a call; except where it adds
+// the sums of two halves of K (few_rows_halves), which is up to M, K and N alone, so that every call of
+// those sizes takes it: equal rows give equal bits whatever the streams and the epilogue.
+bool few_rows_halves(int64_t M, int64_t K, int64_t N);
+// Which of the two kernels is the faster one otherwise.
+bool few_rows_kernel_wins(int64_t M, int64_t K, int64_t N, int streams);
 int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream);
 // TMA map over a row-major [rows, cols] bf16 (or fp32) matrix with row stride ld elements:
 // 128-byte swizzle, boxes of [box_rows x 128 bytes], zero fill out of bounds

@@ -9,17 +9,20 @@
 //    accumulator rows, 2 i + 1 the second's. Up to 128 rows, a pair holds the off and the on
 //    stream of the same rows, so one pass over a W tile serves both; three segments per stream
 //    make three pairs, not four.
-//  * Columns and K. bn (a multiple of 32 up to 256) and the split of K over ks pairs of a cluster
-//    (1 or 2) are chosen so that the pairs fill the SMs. ks depends on M, K and N alone, so that
-//    every output element is one sum in one order whatever the streams, the epilogue and the tile
-//    width: shared, stacked and three-stream calls that come here agree bit for bit. (Four slices measured
-//    slower: only 15 clusters of eight CTAs fit on the chip, 36 of four.)
+//  * Columns and K. bn (a multiple of 32 from 64 to 256) and the split of K over ks pairs of a cluster
+//    (1 or 2) are chosen so that the pairs fill the SMs. With one slice the sums are the tile kernel's,
+//    in its order, so that the faster kernel may serve each call. With two they are not, and M, K and N
+//    alone decide (few_rows_halves): shared, stacked and three-stream calls and every epilogue
+//    agree bit for bit. (Four slices measured slower: only 15 clusters of eight CTAs fit on the chip,
+//    36 of four.)
 //  * Ring items are two k-blocks of 64, and x and W have a TMA warp each. What a warp executes
 //    per item is the limit at these sizes: one warp and 64-wide items took 570 clocks each, more
-//    than the products of a tile (97 x 4096 x 12288: 44.8 us, then 26.5).
-//  * LoRA. The k-blocks of u B^T go to the last K slice and accumulate in TMEM columns of their
-//    own; y_on's partial sum there is main + lora. No drain waits for them, and a pair with an
-//    off segment never mixes B into the off rows (their part of that accumulator is not read).
+//    than the products of a tile (97 x 4096 x 12288: 44.8 us, then 26).
+//  * LoRA. The k-blocks of u B^T follow x W^T into the accumulator of y_on. The rows of a CTA without
+//    LoRA are masked out of those products, so that B, whatever it holds, never meets an off row. One
+//    input with both outputs: y_off's sums are copied in TMEM first and drained beside the LoRA
+//    products. Two K slices: the last one accumulates u B^T apart, and y_on's partial sum there is
+//    main + lora.
 //  * Reduction and epilogue. Each of two K slices finishes half of the tile's columns: it takes
 //    the other slice's fp32 sums of those columns, pushed into its drained ring through
 //    distributed shared memory. Once the products are done all twelve warps drain, three per
@@ -34,7 +37,7 @@
 // What bounds it: HBM for W, and an SM's fill from L2 (64 B per clock: a k-block of 64 costs
 // 2 (seg + bn / 2) clocks of fill for 2 bn clocks of products), which is why the x boxes are as
 // high as the segment and not 128 rows. 97 rows x 4096 x 12288 (two streams): the main loop runs
-// at 6.6 TB/s of W; about 6 us of the 25.6 are set-up, first loads, drain and stores.
+// at 6.6 TB/s of W; about 6 us of the 26 are set-up, first loads, drain and stores.
 #include <float.h>
 
 #include <atomic>
@@ -50,7 +53,7 @@ constexpr int BK = 128;  // a ring item: two k-blocks of 64 (128-byte swizzle ea
 constexpr int NUM_THREADS = 384;
 constexpr int kMaxStages = 12;
 constexpr int kSmemMax = 232448;  // dynamic shared memory of one CTA (227 KiB)
-constexpr int kBarBytes = (2 * kMaxStages + 1) * 8 + 16;
+constexpr int kBarBytes = (2 * kMaxStages + 2) * 8 + 16;
 
 // Epilogues. The kernel is compiled for each: a launch then fetches about 40 KB of code and not its
 // parts of 82 KB (a 3-layer scoring pass of 97 rows 500 -> 495 us).
@@ -76,9 +79,11 @@ struct Params {
   int has_on, has_crit;
   int b_box;     // rows of a W / B box
   int x_settled; // x is final before the preceding kernel of the stream ends
-  int lcol;      // TMEM column of the LoRA accumulator
+  int lcol;      // TMEM column of a second accumulator, 0: none. Two K slices: the LoRA sums; one, with
+                 // `both`: a copy of the sums, for y_on
   uint32_t tmem_cols;
   int stg_off;   // byte offset of the drain warps' staging buffers (over the drained ring)
+  int lora_first;  // `both`, one K slice: the buffers overlap the LoRA items
   int bar_off;
   void* y[3];
   int rope_P, rope_cols;
@@ -108,6 +113,16 @@ __device__ __forceinline__ void prefetch_box(const CUtensorMap* map, int x, int 
                "r"(x), "r"(y)
                : "memory");
 }
+// tc_mma2_bf16 that leaves the accumulator lanes of a CTA alone whose `skip` is all ones (0: not)
+__device__ __forceinline__ void tc_mma2_bf16_masked(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                    uint32_t accumulate, uint32_t skip0, uint32_t skip1) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5, %6, %6, %6, %6}, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(skip0), "r"(skip1)
+      : "memory");
+}
 __device__ __forceinline__ float bf16_round(float v) {
   return __bfloat162float(__float2bfloat16_rn(v));
 }
@@ -133,8 +148,9 @@ __device__ __forceinline__ void ld_cols(uint32_t taddr, uint32_t (&v)[16]) { tc_
 // An epilogue thread's accumulator row: its sums, a chunk of tile columns at a time.
 struct RowSums {
   uint32_t taddr;  // TMEM address of the thread's lane, column 0 of the main accumulator
-  int lcol;        // columns from there to the LoRA accumulator
-  bool own_lora;   // this CTA holds the LoRA sums
+  int on_col;      // columns from there to the sums of y_on, if they are apart (one K slice)
+  int lcol;        // columns from there to the LoRA sums, to be added to y_on's (two slices)
+  bool own_lora;   // this CTA holds LoRA sums
   const float4* recv;  // the other K slice's sums of this CTA's columns (ks == 2), else NULL
   int lplane;      // float4 from there to the LoRA sums sent along (shared input, slice 0), or 0
   int row;         // row of the tile (TMEM lane)
@@ -144,7 +160,7 @@ struct RowSums {
   template <int n>
   __device__ __forceinline__ void get(int c, int pos, bool lora, float (&v)[n]) const {
     uint32_t a[n];
-    ld_cols(taddr + c, a);
+    ld_cols(taddr + c + (lora ? on_col : 0), a);
     if (lora && own_lora) {
       uint32_t l[n];
       ld_cols(taddr + lcol + c, l);
@@ -342,14 +358,16 @@ __device__ __forceinline__ void emit_lsm(const Params& p, const RowSums& r, int 
   asm volatile("bar.sync %0, 96;" ::"r"(1 + q) : "memory");  // the buffer serves the next output
 }
 
-template <int kEpi>
+// kCopy: one input with LoRA and both outputs wanted, one K slice (see `both`). In a kernel of its own:
+// as a run-time flag it cost the others 0.3 us a launch.
+template <int kEpi, bool kCopy>
 __global__ void __launch_bounds__(NUM_THREADS)
     lora_gemm_small_kernel(const __grid_constant__ Maps mp, const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.bar_off);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
@@ -358,6 +376,7 @@ __global__ void __launch_bounds__(NUM_THREADS)
   auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
   auto empty_bar = [&](int s) { return smem_u32(&bars[kMaxStages + s]); };
   const uint32_t acc_full = smem_u32(&bars[2 * kMaxStages]);
+  const uint32_t copied = smem_u32(&bars[2 * kMaxStages + 1]);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
@@ -371,6 +390,7 @@ __global__ void __launch_bounds__(NUM_THREADS)
     }
     if (lane == 0) {
       mbar_init(acc_full, 1);
+      mbar_init(copied, 2 * (NUM_THREADS / 32));
       *abort_flag = 0;
     }
     __syncwarp();
@@ -459,6 +479,22 @@ __global__ void __launch_bounds__(NUM_THREADS)
   // 97-row scoring pass 457 us, let in at once 465).
   constexpr bool kEarly = kEpi == EPI_STORE || kEpi == EPI_STORE_F32;
   if (kEarly) pdl_launch_dependents();
+  int loaded = 0;  // items that a producer has asked for
+  // products of LoRA item i, from stage s. With one K slice they go on in y_on's accumulator, past the
+  // lanes of a CTA whose rows have none; with two they have their own.
+  auto lora_products = [&](int i, int s) {
+    const uint32_t st = smem_base + s * stage_bytes;
+    const int nsub = min(BK / 16, (p.r - i * BK + 15) / 16);
+    const bool one = p.ks == 1;
+#pragma unroll 1
+    for (int k = 0; k < nsub; ++k) {
+      const uint32_t at = static_cast<uint32_t>(k & 3) * 32;
+      tc_mma2_bf16_masked(tmem_acc + p.lcol, smem_desc_sw128(st + (k < 4 ? 0 : a_bytes) + at),
+                          smem_desc_sw128(st + 2 * a_bytes + (k < 4 ? 0 : b_bytes) + at), idesc_bf16_f32(256, p.bn),
+                          one || i > 0 || k > 0 ? 1u : 0u, one && !lora0 ? ~0u : 0u, one && !lora1 ? ~0u : 0u);
+    }
+    commit_pair_mask(empty_bar(s), pair_mask);
+  };
   if (warp == 0 || warp == 2) {
     // ------------------------------------------------------------------ TMA producers: warp 0
     // moves W (and B), warp 2 x (and u). Everything an item needs is a running value, an item is
@@ -525,9 +561,10 @@ __global__ void __launch_bounds__(NUM_THREADS)
         }
       }
     }
+    loaded = it;
     // copies in flight land before shared memory is reused: a stage's empty barrier is
     // committed after the products that read it
-    for (int k = (it > p.stages ? it - p.stages : 0); k < it; ++k) {
+    for (int k = (it > p.stages ? it - p.stages : 0); k < (kCopy ? min(it, n_main) : it); ++k) {
       volatile int no_abort = 0;
       warp_wait_bounded(empty_bar(k % p.stages), (k / p.stages) & 1, &no_abort, p.err, kDevTimeoutDrain);
     }
@@ -537,27 +574,24 @@ __global__ void __launch_bounds__(NUM_THREADS)
       const uint32_t idesc = idesc_bf16_f32(256, p.bn);
       int s = 0;
       uint32_t ph = 0;
-      for (int it = 0; it < items; ++it) {
+      for (int it = 0; it < (kCopy ? n_main : items); ++it) {
         if (!warp_wait_bounded(full_bar(s), ph, abort_flag, p.err, kDevTimeoutMma)) break;
         tc_fence_after();
         if (elect_one()) {
-          const uint32_t st = smem_base + s * stage_bytes;
-          const uint64_t a0 = smem_desc_sw128(st), a1 = smem_desc_sw128(st + a_bytes);
-          const uint64_t b0 = smem_desc_sw128(st + 2 * a_bytes);
-          const uint64_t b1 = smem_desc_sw128(st + 2 * a_bytes + b_bytes);
           if (it < n_main) {
+            const uint32_t st = smem_base + s * stage_bytes;
+            const uint64_t a0 = smem_desc_sw128(st), a1 = smem_desc_sw128(st + a_bytes);
+            const uint64_t b0 = smem_desc_sw128(st + 2 * a_bytes);
+            const uint64_t b1 = smem_desc_sw128(st + 2 * a_bytes + b_bytes);
 #pragma unroll
             for (int k = 0; k < 4; ++k)  // + 32 bytes per k-step: 2 in the address field
               tc_mma2_bf16(tmem_acc, a0 + 2 * k, b0 + 2 * k, idesc, (it > 0 || k > 0) ? 1u : 0u);
 #pragma unroll
             for (int k = 0; k < 4; ++k) tc_mma2_bf16(tmem_acc, a1 + 2 * k, b1 + 2 * k, idesc, 1u);
+            commit_pair_mask(empty_bar(s), pair_mask);
           } else {
-            const int nsub = min(BK / 16, (p.r - (it - n_main) * BK + 15) / 16);
-            for (int k = 0; k < nsub; ++k)
-              tc_mma2_bf16(tmem_acc + p.lcol, (k < 4 ? a0 : a1) + 2 * (k & 3),
-                           (k < 4 ? b0 : b1) + 2 * (k & 3), idesc, (it > n_main || k > 0) ? 1u : 0u);
+            lora_products(it - n_main, s);
           }
-          commit_pair_mask(empty_bar(s), pair_mask);
         }
         __syncwarp();
         if (++s == p.stages) {
@@ -572,10 +606,43 @@ __global__ void __launch_bounds__(NUM_THREADS)
     volatile int no_abort = 0;
     warp_wait_bounded(acc_full, 0, &no_abort, p.err, kDevTimeoutDrain);
   }
+  // (waited for once: with kCopy the barrier may have completed again by the next look)
+  bool epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
+  if constexpr (kCopy) {
+    // y_on's sums go on from y_off's, which stay: every warp copies its part (three per quarter of
+    // the TMEM lanes), then the LoRA products accumulate on the copy while y_off is drained
+    tc_fence_after();
+    if (__all_sync(0xffffffffu, epi_ok) && (warp & 3) * 32 < nrow) {
+      const uint32_t from = tmem_acc + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+#pragma unroll 1
+      for (int c = 16 * (warp >> 2); c < p.bn; c += 48) {
+        uint32_t v[16];
+        tc_ld_32x32b_x16(from + c, v);
+        tc_wait_ld();
+        tc_st_32x32b_x16(from + p.lcol + c, v);
+      }
+      tc_wait_st();
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive_cluster(map_to_rank(copied, lead_rank));
+    if (warp == 1 && leader) {
+      const bool all = warp_wait_cluster_bounded(copied, 0, abort_flag, p.err, kDevTimeoutMma);
+      tc_fence_after();
+      for (int it = n_main; all && it < items; ++it) {
+        const int s = it % p.stages;
+        if (!warp_wait_bounded(full_bar(s), (it / p.stages) & 1, abort_flag, p.err, kDevTimeoutMma)) break;
+        tc_fence_after();
+        if (elect_one()) lora_products(it - n_main, s);
+        __syncwarp();
+      }
+      if (elect_one()) commit_pair_mask(acc_full, pair_mask);
+      __syncwarp();
+    }
+  }
   // ---------------------------------------------------------------------- drain: every warp,
   // three per quarter of the TMEM lanes
   constexpr int kDrainers = 3;
-  bool epi_ok = mbar_wait_bounded(acc_full, 0, abort_flag, p.err, kDevTimeoutEpilogue);
   epi_ok = __all_sync(0xffffffffu, epi_ok) && *abort_flag == 0;
   if (kEpi == EPI_LOGSOFTMAX) epi_ok = __syncthreads_and(epi_ok);  // a quarter's warps meet again
   tc_fence_after();
@@ -583,7 +650,8 @@ __global__ void __launch_bounds__(NUM_THREADS)
 
   const int q = warp & 3;             // TMEM lanes 32 q .. of a drain warp
   const int trow = q * 32 + lane;     // row of the segment
-  const int par = warp >> 2;          // which of the warps of its lanes
+  // which of the warps of its lanes; the first ones, which have had the main loop, take the fewer chunks
+  const int par = kDrainers - 1 - (warp >> 2);
   const bool drain = epi_ok && q * 32 < nrow;
   const bool last = slice == p.ks - 1;
   constexpr int kChunk = chunk_of(kEpi);
@@ -598,8 +666,9 @@ __global__ void __launch_bounds__(NUM_THREADS)
   };
   RowSums rs;
   rs.taddr = tmem_acc + (static_cast<uint32_t>(q * 32) << 16);
+  rs.on_col = kCopy ? p.lcol : 0;
   rs.lcol = p.lcol;
-  rs.own_lora = last && lora_me;
+  rs.own_lora = p.ks == 2 && last && lora_me;
   rs.row = trow;
   rs.recv = nullptr;
   rs.lplane = 0;
@@ -654,6 +723,10 @@ __global__ void __launch_bounds__(NUM_THREADS)
         lora = true;
       }
       if (y == nullptr) continue;
+      if (kCopy && (o == 1 || p.lora_first)) {  // the LoRA products are done
+        if (!warp_wait_bounded(acc_full, 1, abort_flag, p.err, kDevTimeoutEpilogue)) break;
+        tc_fence_after();
+      }
       if constexpr (kEpi == EPI_LOGSOFTMAX) {
         emit_lsm(p, rs, row, live, n0, static_cast<float2*>(y),
                  p.lsm_target + ((p.shared_x ? o : stream) == 0 ? 0 : p.M), lora, par, q,
@@ -675,6 +748,12 @@ __global__ void __launch_bounds__(NUM_THREADS)
         }
       }
     }
+  }
+  if (kCopy && warp < 3) {  // the LoRA items, as above
+    volatile int no_abort = 0;
+    if (warp == 1) warp_wait_bounded(acc_full, 1, &no_abort, p.err, kDevTimeoutDrain);
+    for (int k = n_main; warp != 1 && k < loaded; ++k)
+      warp_wait_bounded(empty_bar(k % p.stages), (k / p.stages) & 1, &no_abort, p.err, kDevTimeoutDrain);
   }
   tc_fence_before();
   // no CTA leaves while a peer may touch its barriers or shared memory. Relaxed: nothing is
@@ -738,14 +817,15 @@ bool lay_out(const Shape& s, int bn, Config* c) {
 }
 
 using Kernel = void (*)(smallm::Maps, smallm::Params);
+template <bool kCopy>
 Kernel kernel_of(int epi) {
   switch (epi) {
-    case smallm::EPI_SWIGLU: return smallm::lora_gemm_small_kernel<smallm::EPI_SWIGLU>;
-    case smallm::EPI_RESIDUAL: return smallm::lora_gemm_small_kernel<smallm::EPI_RESIDUAL>;
-    case smallm::EPI_ROPE: return smallm::lora_gemm_small_kernel<smallm::EPI_ROPE>;
-    case smallm::EPI_LOGSOFTMAX: return smallm::lora_gemm_small_kernel<smallm::EPI_LOGSOFTMAX>;
-    case smallm::EPI_STORE_F32: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE_F32>;
-    default: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE>;
+    case smallm::EPI_SWIGLU: return smallm::lora_gemm_small_kernel<smallm::EPI_SWIGLU, kCopy>;
+    case smallm::EPI_RESIDUAL: return smallm::lora_gemm_small_kernel<smallm::EPI_RESIDUAL, kCopy>;
+    case smallm::EPI_ROPE: return smallm::lora_gemm_small_kernel<smallm::EPI_ROPE, kCopy>;
+    case smallm::EPI_LOGSOFTMAX: return smallm::lora_gemm_small_kernel<smallm::EPI_LOGSOFTMAX, false>;
+    case smallm::EPI_STORE_F32: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE_F32, kCopy>;
+    default: return smallm::lora_gemm_small_kernel<smallm::EPI_STORE, kCopy>;
   }
 }
 
@@ -755,8 +835,8 @@ bool allow_smem(int dev) {
   if (dev < 0 || dev >= 64) return false;
   if (done[dev]) return true;
   for (int e = smallm::EPI_STORE; e <= smallm::EPI_STORE_F32; ++e)
-    if (cudaFuncSetAttribute(kernel_of(e), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
-      return false;
+    for (Kernel k : {kernel_of<false>(e), kernel_of<true>(e)})
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return false;
   return done[dev] = true;
 }
 
@@ -778,7 +858,7 @@ int resident_clusters(int dev, int ks) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel<smallm::EPI_STORE>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, smallm::lora_gemm_small_kernel<smallm::EPI_STORE, false>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -786,20 +866,24 @@ int resident_clusters(int dev, int ks) {
   return n;
 }
 
-Shape shape_of(int64_t M, int64_t K, int64_t N, int streams, int epi) {
+// Split of K between the two pairs of a cluster (36 of these fit on the chip) where 256-column
+// tiles of two streams leave most pairs idle and half of K is worth the exchange of the sums,
+// about 3 us. Measured, one slice against two, us, two streams: 4 to 12 tiles, 20 x 1024 x 776
+// -4 % to 200 x 1024 x 1536 +18 %, 200 x 2048 x 1536 +4 %, 97 x 3200 x 3000 -5 %; 16 tiles,
+// 128 x 2048 x 4096 +6 %, 97 x 4096 x 4096 -9 %; 24 tiles, 449 x 3200 x 1536 +26 %,
+// 200 x 6000 x 3000 -1 %; 32 tiles, 200 x 4096 x 4096 +21 %, 200 x 11008 x 4096 +8 %.
+int k_slices(int64_t M, int64_t K, int64_t N) {
+  const int64_t kb = (K + smallm::BK - 1) / smallm::BK;
+  const int64_t tiles = (M + 127) / 128 * ((N + 255) / 256);
+  const int64_t kb_min = tiles <= 12 ? 16 : (tiles <= 18 ? 20 : 40);
+  return tiles <= 24 && kb >= kb_min ? 2 : 1;
+}
+
+Shape shape_of(int64_t M, int streams, int epi, int ks) {
   Shape s{};
   s.streams = streams;
   s.nseg = static_cast<int>((M + 127) / 128);
-  const int64_t kb = (K + smallm::BK - 1) / smallm::BK;
-  // Split of K between the two pairs of a cluster (36 of these fit on the chip) where 256-column
-  // tiles of two streams leave most pairs idle and half of K is worth the exchange of the sums,
-  // about 3 us. Measured, one slice against two, us, two streams: 4 to 12 tiles, 20 x 1024 x 776
-  // -4 % to 200 x 1024 x 1536 +18 %, 200 x 2048 x 1536 +4 %, 97 x 3200 x 3000 -5 %; 16 tiles,
-  // 128 x 2048 x 4096 +6 %, 97 x 4096 x 4096 -9 %; 24 tiles, 449 x 3200 x 1536 +26 %,
-  // 200 x 6000 x 3000 -1 %; 32 tiles, 200 x 4096 x 4096 +21 %, 200 x 11008 x 4096 +8 %.
-  const int64_t tiles = s.nseg * ((N + 255) / 256);
-  const int64_t kb_min = tiles <= 12 ? 16 : (tiles <= 18 ? 20 : 40);
-  s.ks = epi != smallm::EPI_LOGSOFTMAX && tiles <= 24 && kb >= kb_min ? 2 : 1;
+  s.ks = ks;
   if (s.streams == 1 && (s.nseg & 1)) ++s.nseg;
   s.seg = static_cast<int>(((M + s.nseg - 1) / s.nseg + 7) / 8 * 8);
   s.row_tiles = (s.streams * s.nseg + 1) / 2;
@@ -842,8 +926,13 @@ double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, doub
 
 }  // namespace
 
-// Sizes alone decide, not the epilogue, nor whether one or two streams are given: the sums of one
-// (M, K, N) have one order. Above 128 rows the tile kernel of lora_gemm_tc.cu takes over where its
+bool few_rows_halves(int64_t M, int64_t K, int64_t N) {
+  if (M < 1 || M > 512 || (M > 448 && K > 4096) || K >= (1LL << 28) || k_slices(M, K, N) != 2) return false;
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && allow_smem(dev) && resident_clusters(dev, 2) > 0;
+}
+
+// Above 128 rows the tile kernel of lora_gemm_tc.cu takes over where its
 // 256-column tiles fill the chip (measured on GB300, us, this kernel / that one; rows x K x N, two
 // streams):
 //  * up to 128 rows: 97 x 4096 x 4096 12.3 / 30.4, x 12288 25.6 / 35.3, x 22016 43.9 / 80.3;
@@ -861,17 +950,16 @@ double choose_width(const Shape& s, int64_t K, int64_t N, int epi, int dev, doub
 // 81.5, 100 x 4096 x 4096 23.5 / 35.7): the clocks of both are estimated, with shares per wave
 // and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
 // 12288), four of which are then slower, by 2 to 3 %.
-bool small_gemm_wanted(int64_t M, int64_t K, int64_t N, int streams) {
+bool few_rows_kernel_wins(int64_t M, int64_t K, int64_t N, int streams) {
   if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
   const bool wanted = M <= 128 || (M <= 256 && (N <= 11264 || (N <= 14336 && K >= 2048))) ||
                       (M <= 384 && M > 256 && N <= 16384) || (M <= 448 && N <= 5120) ||
                       (M <= 512 && N <= 5120 && K <= 4096);
-  if (!wanted || streams < 3) return wanted;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || !allow_smem(dev)) return false;
+  if (!wanted || cudaGetDevice(&dev) != cudaSuccess || !allow_smem(dev) || resident_clusters(dev, 1) < 1) return false;
+  if (streams < 3) return true;
   Config c{};
-  const double here = choose_width(shape_of(M, K, N, streams, smallm::EPI_STORE), K, N, smallm::EPI_STORE, dev,
-                                   10000.0, &c);
+  const double here = choose_width(shape_of(M, streams, smallm::EPI_STORE, 1), K, N, smallm::EPI_STORE, dev, 10000.0, &c);
   const int64_t kb = (K + 63) / 64, cols = (N + 255) / 256;
   // that kernel: 128-row tiles, 704 clocks of fill per k-block, on 152 SMs; 256-row tiles, 512 of
   // products, on 76 pairs
@@ -889,13 +977,18 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   const int M = static_cast<int>(a.M), N = static_cast<int>(a.N);
   const int kb = static_cast<int>((a.K + BK - 1) / BK);
   const bool lora_on = a.r > 0 && a.u != nullptr && a.B != nullptr && a.y_on != nullptr;
+  // Up to 128 rows of one input with LoRA go as two streams: a CTA has one output to drain, and the
+  // sums of y_on need no copy (40 x 1024 x 4096 8.6 us as one stream, 7.6 as two; 97 x 4096 x 12288
+  // 25.9, 25.6).
+  const int ks = a.epi != EPI_LOGSOFTMAX && few_rows_halves(a.M, a.K, a.N) ? 2 : 1;
+  const bool shared = a.shared_x && !(a.M <= 128 && lora_on && a.y_off != nullptr && ks == 1);
   const bool lora_crit = tri && a.r > 0 && a.u_crit != nullptr && a.B_crit != nullptr && a.y_crit != nullptr;
-  Shape s = shape_of(a.M, a.K, a.N, a.shared_x ? 1 : (tri ? 3 : 2), a.epi);
+  Shape s = shape_of(a.M, shared ? 1 : (tri ? 3 : 2), a.epi, ks);
   s.lora = lora_on || lora_crit;
-  s.both = a.shared_x && lora_on && a.y_off != nullptr;
+  s.both = shared && lora_on && a.y_off != nullptr;
   Config best{};
   choose_width(s, a.K, a.N, a.epi, dev, 6000.0, &best);
-  if (best.bn == 0) return kSmallGemmNoFit;
+  if (best.bn == 0) return -4;
   const int bn = best.bn;
 
   Params p{};
@@ -928,14 +1021,25 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   p.bn = bn;
   p.ks = s.ks;
   p.stages = best.stages;
-  p.shared_x = a.shared_x ? 1 : 0;
+  p.shared_x = shared ? 1 : 0;
   p.both = s.both ? 1 : 0;
   p.has_on = lora_on ? 1 : 0;
   p.has_crit = lora_crit ? 1 : 0;
   p.x_settled = a.x_settled ? 1 : 0;
-  p.lcol = pow2_at_least(bn);
-  p.tmem_cols = static_cast<uint32_t>(s.lora ? 2 * p.lcol : p.lcol);
+  const bool second = s.ks == 2 ? s.lora : s.both;
+  p.lcol = second ? pow2_at_least(bn) : 0;
+  p.tmem_cols = static_cast<uint32_t>(pow2_at_least(bn) * (second ? 2 : 1));
   p.stg_off = best.stg_off;
+  if (s.both && s.ks == 1) {
+    // y_off is drained while the LoRA items are still read: through the stages before or after them
+    const int stage = 2 * (s.seg * 128 + bn * 64), first = kb % best.stages;
+    const int staging = NUM_THREADS / 32 * 4096, wrapped = first + p.kb_lora > best.stages ? stage : 0;
+    p.stg_off = first * stage - wrapped >= staging ? wrapped : (first + p.kb_lora) * stage;
+    if (p.stg_off + staging > best.stages * stage) {  // two items in the middle of a short ring
+      p.stg_off = best.stg_off;
+      p.lora_first = 1;
+    }
+  }
   p.bar_off = best.bar_off;
   p.y[0] = a.y_off;
   p.y[1] = a.y_on;
@@ -968,7 +1072,7 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const int epi = a.epi == EPI_STORE && a.out_f32 ? EPI_STORE_F32 : a.epi;
-  return cudaLaunchKernelEx(&cfg, kernel_of(epi), mp, p) == cudaSuccess ? 0 : -3;
+  return cudaLaunchKernelEx(&cfg, s.both && s.ks == 1 ? kernel_of<true>(epi) : kernel_of<false>(epi), mp, p) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace hydra

@@ -1028,10 +1028,9 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   const bool packed = a.epi == EPI_LOGSOFTMAX && !a.shared_x && a.x_crit == nullptr && a.r == 0 && a.M <= BM / 2 &&
                       a.y_off != nullptr && a.y_on != nullptr;
   const int streams = a.shared_x ? 1 : (a.x_crit != nullptr ? 3 : 2);
-  if (!packed && !a.single_cta && lsm_ok && small_gemm_wanted(a.M, a.K, a.N, streams)) {
-    const int rc = launch_dual_lora_gemm_small(a, stream);
-    if (rc != kSmallGemmNoFit) return rc;
-  }
+  if (!packed && !a.single_cta && lsm_ok &&
+      ((a.epi != EPI_LOGSOFTMAX && few_rows_halves(a.M, a.K, a.N)) || few_rows_kernel_wins(a.M, a.K, a.N, streams)))
+    return launch_dual_lora_gemm_small(a, stream);
   static bool attr_set = false;
   if (!attr_set) {
     if (cudaFuncSetAttribute(dual_lora_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

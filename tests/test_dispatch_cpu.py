@@ -79,8 +79,8 @@ def test_linear_falls_back_where_no_cluster_fits(fake):
     """A partition that holds no cluster of four CTAs (or none at all): the tile kernel serves the call."""
     assert all(_small(v) for v in fake.linear(97, 4096, 4096) + fake.linear(97, 4096, 12288))
     fake.device(device=1, quads=0)
-    (two,), (one,) = fake.linear(97, 4096, 4096), fake.linear(97, 4096, 12288)
-    assert "dual_lora_gemm_kernel" in two[0] and _small(one)  # two K slices and one
+    for (v,) in (fake.linear(97, 4096, 4096), fake.linear(97, 4096, 12288)):  # otherwise two K slices, and one
+        assert _small(v) and v[4] == 2
     fake.device(device=2, pairs=0, quads=0)
     for streams in (1, 2, 3):
         for m, kernel in ((1, "dual_lora_gemm_kernel"), (128, "dual_lora_gemm_kernel"), (200, "dual_lora_gemm_2cta_kernel")):
@@ -137,3 +137,16 @@ def test_losses_with_the_callers_moments_make_no_pass_over_the_batch_for_them(fa
     assert fake.lib.hydra_ppo_loss(P, P, P, P, P, None, 1000, 400, 0.2, whiten, P, P, P, P, P, BIG, None) == 0
     first, second = fake.launches()
     assert "ppo_ext_kernel" in first[0] and first[1:4] == (1, 1, 1) and "ppo_loss_kernel" in second[0]
+
+
+def test_kernel_with_its_own_order_of_sums_is_up_to_the_sizes_alone(fake):
+    """Two K slices (clusters of four) add the halves of K apart: one, two and three streams all take
+    them, or none does. Any other size has the tile kernel's order in either kernel."""
+    halves = 0
+    for m in (1, 20, 64, 128, 129, 200, 300, 384, 448, 449, 512, 513):
+        for k in (8, 1024, 2048, 2560, 4096, 5120, 11008):
+            for n in (8, 776, 1536, 3000, 4096, 5120, 8192, 12288, 22016):
+                split = {_small(v) and v[4] == 4 for st in (1, 2, 3) for r in (0, 16) for v in fake.linear(m, k, n, st, r)}
+                assert len(split) == 1
+                halves += split.pop()
+    assert halves > 50
