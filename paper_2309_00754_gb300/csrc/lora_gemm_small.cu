@@ -961,10 +961,12 @@ bool few_rows_kernel_wins(int64_t M, int64_t K, int64_t N, int streams) {
   Config c{};
   const double here = choose_width(shape_of(M, streams, smallm::EPI_STORE, 1), K, N, smallm::EPI_STORE, dev, 10000.0, &c);
   const int64_t kb = (K + 63) / 64, cols = (N + 255) / 256;
-  // that kernel: 128-row tiles, 704 clocks of fill per k-block, on 152 SMs; 256-row tiles, 512 of
-  // products, on 76 pairs
+  // that kernel: 128-row tiles, 704 clocks of fill per k-block, on the SMs; 256-row tiles, 512 of
+  // products, on pairs of them
+  const int64_t nsm = sm_count(), units = M <= 128 ? nsm : nsm / 2;
+  if (units < 1) return false;
   const int64_t tiles = streams * cols * (M <= 128 ? 1 : (M + 255) / 256);
-  const int64_t waves = M <= 128 ? (tiles + 151) / 152 : (tiles + 75) / 76;
+  const int64_t waves = (tiles + units - 1) / units;
   const double there = static_cast<double>(waves * kb) * (M <= 128 ? 704 : 512) + 12000.0 + 1000.0 * (waves - 1);
   return c.bn != 0 && 1.1 * here < there;
 }

@@ -150,3 +150,14 @@ def test_kernel_with_its_own_order_of_sums_is_up_to_the_sizes_alone(fake):
                 assert len(split) == 1
                 halves += split.pop()
     assert halves > 50
+
+
+def test_three_stream_estimate_counts_the_devices_multiprocessors(fake):
+    """The same tiles per multiprocessor, the same choice: half the columns on half the device."""
+    def choice(device, sms, n):
+        fake.device(device, sms, sms // 2, 36 * sms // 152)
+        (v,) = fake.linear(100, 4096, n, 3)
+        return _small(v)
+    for n in (4096, 6144, 8192):
+        assert choice(0, 152, 2 * n) == choice(1, 76, n), n
+    assert choice(1, 76, 8192) and not choice(1, 76, 6144)
