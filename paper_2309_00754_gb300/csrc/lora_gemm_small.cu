@@ -932,29 +932,41 @@ bool few_rows_halves(int64_t M, int64_t K, int64_t N) {
   return cudaGetDevice(&dev) == cudaSuccess && allow_smem(dev) && resident_clusters(dev, 2) > 0;
 }
 
-// Above 128 rows the tile kernel of lora_gemm_tc.cu takes over where its
-// 256-column tiles fill the chip (measured on GB300, us, this kernel / that one; rows x K x N, two
-// streams):
-//  * up to 128 rows: 97 x 4096 x 4096 12.3 / 30.4, x 12288 25.6 / 35.3, x 22016 43.9 / 80.3;
-//    97 x 11008 x 4096 22.5 / 69.3;
-//  * up to 256, where a stream is one 256-row tile there: 200 x 4096 x 8192 22.9 / 24.7, x 11008
-//    35.3 / 39.5, x 14336 40.6 / 41.0, x 16384 45.4 / 44.1, x 22016 79.4 / 71.2 (above 11264
-//    columns with a long K only: 200 x 512 x 12288 15.4 / 14.9);
-//  * up to 384, where it is two and the second half empty: 300 x 4096 x 4096 18.8 / 23.8 (shared
-//    input 15.9 / 24.5), x 12288 58.9 / 63.3, x 16384 66.7 / 74.1, x 22016 105.1 / 104.0;
-//  * up to 512, while few columns leave it less than one wave or little more: 512 x 4096 x 2048
-//    18.8 / 21.7, x 4096 22.9 / 24.7, x 5120 33.1 / 38.2, x 8192 46.6 / 42.9; a long K makes up
-//    for that: 448 x 11008 x 4096 51.9 / 54.2, 512 x 11008 x 4096 57.4 / 55.0.
-// Three streams leave a row segment over in a pair, or a wave, more often (with their lora_downs:
-// 100 x 4096 x 12288 44.3 / 41.6, 300 x 512 x 12288 35.4 / 26.1, but 100 x 11008 x 4096 43.0 /
-// 81.5, 100 x 4096 x 4096 23.5 / 35.7): the clocks of both are estimated, with shares per wave
-// and a margin fitted to 360 measured sizes (20 to 512 rows, K 512 to 11008, N 1024 to
-// 12288), four of which are then slower, by 2 to 3 %.
+// Measured over 8 to 512 rows, K 256 to 11008 and N 1024 to 65536 (GB300, us in a graph with the call's
+// lora_down of rank 16, this kernel / the tile kernel of lora_gemm_tc.cu, two streams unless said):
+//  * up to 128 rows that kernel's 128 x 256 tiles leave most SMs idle until the columns fill them:
+//    97 x 4096 x 4096 13.7 / 31.2, x 12288 26.4 / 35.0, x 16384 32.1 / 37.4; but 40 x 256 x 22016 13.0 /
+//    10.3, x 65536 28.5 / 17.5. A long K is worth a second wave: 97 x 1024 x 22016 20.7 / 22.7,
+//    97 x 2048 x 32000 38.0 / 38.8, 97 x 4096 x 65536 116 / 120. One stream has one of that kernel's
+//    tiles where two have one of these: 40 x 1024 x 22016 19.0 / 19.1, 97 x 2048 x 32000 36.4 / 33.2;
+//  * up to 256, where a stream is one 256-row tile there: 200 x 512 x 9216 11.1 / 11.5, x 11008 15.0 /
+//    13.5, 200 x 2048 x 11008 26.0 / 27.4, 200 x 4096 x 12288 42.0 / 43.9;
+//  * up to 384, where it is two and the second half empty: 300 x 1024 x 6144 13.8 / 17.4, x 8192 19.3 /
+//    19.0, x 12288 24.0 / 24.6, x 14336 30.1 / 25.4, 300 x 4096 x 16384 69.9 / 78.2;
+//  * up to 512: 448 x 1024 x 4096 13.7 / 14.2, x 5120 17.8 / 17.2, 448 x 4096 x 5120 37.1 / 43.3.
+// Three streams leave a row segment over in a pair, or a wave, more often (97 x 4096 x 12288 45.5 /
+// 40.2, 300 x 512 x 12288 35.7 / 25.0, but 97 x 4096 x 4096 23.7 / 34.9): the clocks of both are
+// estimated, with shares per wave and a margin that choose within 0.4 % of the better kernel over 875
+// sizes, 7 of them slower by more than 3 %.
 bool few_rows_kernel_wins(int64_t M, int64_t K, int64_t N, int streams) {
-  if (M < 1 || K >= (1LL << 28) || N > 64 * 65535) return false;
-  const bool wanted = M <= 128 || (M <= 256 && (N <= 11264 || (N <= 14336 && K >= 2048))) ||
-                      (M <= 384 && M > 256 && N <= 16384) || (M <= 448 && N <= 5120) ||
-                      (M <= 512 && N <= 5120 && K <= 4096);
+  if (M < 1 || M > 512 || K >= (1LL << 28) || N > 64 * 65535) return false;
+  const bool up_to_5k = N <= 5632 && (M <= 448 || K <= 4096);
+  bool wanted;
+  if (streams == 1)
+    wanted = M <= 128   ? N <= 16384 || (K >= 4096 && N <= 24000)
+             : M <= 256 ? N <= 14336
+             : M <= 384 ? N <= 11264 || (K >= 4096 && N <= 13824)
+                        : up_to_5k;
+  else if (streams == 2)
+    wanted = M <= 128   ? N <= 16384 || K >= 4096 || (K >= 2048 && N <= 40000) || (K >= 1024 && N <= 24000)
+             : M <= 256 ? N <= 9600 || (K >= 2048 && N <= 11264) || (K >= 4096 && N <= 13824)
+             : M <= 384 ? N <= 7168 || (N > 10240 && N <= 12800) || (K >= 2048 && N <= 12800) || (K >= 4096 && N <= 16384)
+                        : up_to_5k && (N <= 4608 || K >= 2048);
+  else
+    wanted = M <= 128   ? true
+             : M <= 256 ? N <= 11264 || (K >= 2048 && N <= 14336)
+             : M <= 384 ? N <= 16384
+                        : N <= 5120 && (M <= 448 || K <= 4096);
   int dev = 0;
   if (!wanted || cudaGetDevice(&dev) != cudaSuccess || !allow_smem(dev) || resident_clusters(dev, 1) < 1) return false;
   if (streams < 3) return true;

@@ -152,6 +152,17 @@ def test_kernel_with_its_own_order_of_sums_is_up_to_the_sizes_alone(fake):
     assert halves > 50
 
 
+def test_many_columns_take_the_tile_kernel(fake):
+    """Sizes whose 128 x 256 tiles fill the chip: the few-rows kernel took up to twice the time."""
+    for m, k, n, streams in ((40, 256, 65536, 1), (40, 256, 65536, 2), (97, 512, 32000, 2), (128, 1024, 22016, 1),
+                             (300, 512, 14336, 2), (200, 512, 11008, 2)):
+        (v,) = fake.linear(m, k, n, streams)
+        assert "dual_lora_gemm" in v[0]
+    for m, k, n, streams in ((97, 4096, 22016, 2), (97, 4096, 12288, 1), (300, 4096, 4096, 1), (40, 4096, 11008, 2)):
+        (v,) = fake.linear(m, k, n, streams)
+        assert _small(v)
+
+
 def test_three_stream_estimate_counts_the_devices_multiprocessors(fake):
     """The same tiles per multiprocessor, the same choice: half the columns on half the device."""
     def choice(device, sms, n):
