@@ -992,8 +992,8 @@ int launch_dual_lora_gemm_small(const GemmArgs& a, cudaStream_t stream) {
   const int kb = static_cast<int>((a.K + BK - 1) / BK);
   const bool lora_on = a.r > 0 && a.u != nullptr && a.B != nullptr && a.y_on != nullptr;
   // Up to 128 rows of one input with LoRA go as two streams: a CTA has one output to drain, and the
-  // sums of y_on need no copy (40 x 1024 x 4096 8.6 us as one stream, 7.6 as two; 97 x 4096 x 12288
-  // 25.9, 25.6).
+  // sums of y_on need no copy (40 x 1024 x 4096 8.9 us as one stream, 8.0 as two; 97 x 4096 x 12288
+  // 26.3, 25.9).
   const int ks = a.epi != EPI_LOGSOFTMAX && few_rows_halves(a.M, a.K, a.N) ? 2 : 1;
   const bool shared = a.shared_x && !(a.M <= 128 && lora_on && a.y_off != nullptr && ks == 1);
   const bool lora_crit = tri && a.r > 0 && a.u_crit != nullptr && a.B_crit != nullptr && a.y_crit != nullptr;
