@@ -442,16 +442,6 @@ __global__ void __launch_bounds__(kPpoThreads)
   pdl_launch_dependents();
 }
 
-// The caller's moments for the loss pass, in the place of the moments partials. (With
-// the fp64 root and quotients in every thread of the loss pass 16384 x 400 tokens took 27.3 us, with
-// every thread reading one thread's results 26.1, with one thread of each block 22.1.)
-__global__ void ppo_ext_kernel(const double* __restrict__ ext, Moments* __restrict__ out, unsigned* ticket) {
-  pdl_wait();
-  *out = moments_from_ext(ext);
-  *ticket = 0;
-  pdl_launch_dependents();
-}
-
 // Pass 2: per-token terms and gradients. Each thread holds two chunks: the next chunk's
 // five loads are issued before the current chunk is computed and stored.
 template <int VEC>
@@ -538,16 +528,15 @@ __device__ __forceinline__ void write_moment_stats(double* stats, const Moments&
   stats[6] = m.n;
 }
 
-// The statistics of a batch from its loss sums (kMomentsDone: all but the moments).
-template <bool kMomentsDone = false>
+// The statistics of a batch from its loss sums (moments_done: all but the moments).
 __device__ __forceinline__ void write_stats(double* stats, const float (&v)[kLossSums], int nclip,
-                                            const Moments& m, bool report_moments) {
+                                            const Moments& m, bool report_moments, bool moments_done = false) {
   const double n = m.n, inv = n > 0.0 ? 1.0 / n : 0.0;
   stats[0] = -static_cast<double>(v[0]) * inv;
   stats[1] = static_cast<double>(v[1]) * inv;
   stats[2] = static_cast<double>(nclip) * inv;
   stats[3] = static_cast<double>(v[2]) * inv;
-  if (kMomentsDone) return;
+  if (moments_done) return;
   if (report_moments) {
     stats[4] = m.mean;
     stats[5] = n > 0.0 ? sqrt(m.m2 * inv) : 0.0;
@@ -557,6 +546,27 @@ __device__ __forceinline__ void write_stats(double* stats, const float (&v)[kLos
     stats[5] = n > 0.0 ? sqrt(fmax(static_cast<double>(v[4]) * inv - a * a, 0.0)) : 0.0;
   }
   stats[6] = n;
+}
+
+// The caller's moments for the loss pass, in the place of the moments partials, and among the
+// statistics. One thread of a warp for each: the fp64 root and quotients are slow (in every thread
+// of the loss pass 16384 x 400 tokens took 27.3 us, with every thread reading one thread's
+// results 26.1, with one thread of each block 22.1; 700 x 1500 tokens unwhitened 10.0 with the
+// statistics at the loss pass's end, 9.55 so).
+__global__ void ppo_ext_kernel(const double* __restrict__ ext, Moments* __restrict__ out, unsigned* ticket,
+                               double* __restrict__ stats) {
+  pdl_wait();
+  if (threadIdx.x == 0) {
+    *out = moments_from_ext(ext);
+    *ticket = 0;
+  } else if (threadIdx.x == 32) {
+    Moments m;
+    m.n = __ldcg(ext);
+    m.mean = __ldcg(ext + 1);
+    m.m2 = __ldcg(ext + 2);
+    write_moment_stats(stats, m);
+  }
+  pdl_launch_dependents();
 }
 
 // Pass 2 over the grid, and the statistics by the block that finishes last.
@@ -592,7 +602,7 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
     mom = merge_moments(mpart, Gm, WHITEN ? __ldg(adv) : 0.f, sh, shk);
   }
   const float mean = mom.c_mean, inv_std = mom.inv_std, inv_n = mom.inv_n;
-  if (WHITEN && tid == 0) write_moment_stats(stats, mom);  // the fp64 root off the end of the launch
+  if (WHITEN && ext == nullptr && tid == 0) write_moment_stats(stats, mom);  // the fp64 root off the end of the launch
   while (true) {
     if (cur.s >= S) {
       loss_compute<VEC, ODD, WHITEN>(x, mean, inv_std, inv_n, eps, acc, grad_logp, grad_val);
@@ -639,7 +649,7 @@ __global__ void __launch_bounds__(kPpoThreads, 3)
 #pragma unroll
     for (int q = 0; q < kLossSums; ++q) v[q] = k[q].s;
     block_sums<kLossSums>(v, nclip, sh, shk);
-    if (threadIdx.x == 0) write_stats<WHITEN>(stats, v, nclip, mom, report_moments != 0);
+    if (threadIdx.x == 0) write_stats(stats, v, nclip, mom, report_moments != 0, WHITEN || ext != nullptr);
   }
   pdl_launch_dependents();
 }
@@ -922,7 +932,7 @@ int launch_ppo_loss(const float* logp_new, const float* logp_old, const float* a
   int Gm = 0;
   if (ext_moments != nullptr) {
     ext = reinterpret_cast<Moments*>(w.mom);
-    if (launch_pdl(ppo_ext_kernel, dim3(1), dim3(1), 0, st, ext_moments, ext, w.ticket) != cudaSuccess) return -3;
+    if (launch_pdl(ppo_ext_kernel, dim3(1), dim3(64), 0, st, ext_moments, ext, w.ticket, stats) != cudaSuccess) return -3;
   } else {
     Gm = launch_moments(adv, lengths, Si, Li, whiten, w, err, st);
     if (Gm < 0) return Gm;
