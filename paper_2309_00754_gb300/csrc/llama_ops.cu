@@ -60,8 +60,11 @@ __global__ void embed_kernel(const __nv_bfloat16* __restrict__ table, int V, int
 // ---------------------------------------------------------------- RMSNorm
 
 // y[i] = bf16( x[map(i)] / sqrt(mean(x^2) + eps) * w ), one CTA of 128 threads per row. The first
-// 4096 elements stay in registers between the two uses, and their loads go out together (194 rows
-// of 4096: 2.8 us back to back with the row read twice, 2.0 so; 6144 rows 25.2, 22.2).
+// 512 kKeep elements (up to 4096) stay in registers between the two uses, and their loads go out
+// together (194 rows of 4096: 2.8 us back to back with the row read twice, 2.0 so; 6144 rows 25.2,
+// 22.2). Short rows have a kernel with fewer: with room for 4096 elements 3000 rows of 128 took 5.2
+// us, read twice 3.7, 4.0 so (3000 of 1024: 5.4, 4.9, 4.2).
+template <int kKeep>
 __global__ void __launch_bounds__(128)
     rmsnorm_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w, int d,
                    float eps, RowMap map, __nv_bfloat16* __restrict__ y) {
@@ -70,7 +73,6 @@ __global__ void __launch_bounds__(128)
   const long long i = blockIdx.x;
   const float4* xr = reinterpret_cast<const float4*>(x + static_cast<size_t>(map_row(i, map)) * d);
   const int n4 = d / 4;
-  constexpr int kKeep = 8;
   float4 keep[kKeep];
 #pragma unroll
   for (int i = 0; i < kKeep; ++i) {
@@ -391,7 +393,11 @@ int launch_embed(const void* table, int64_t V, int64_t d, const int32_t* ids, in
 int launch_rmsnorm(const float* x, const void* w, int64_t rows, int64_t d, float eps,
                    const RowMap& map, void* y, cudaStream_t st) {
   if (rows == 0) return 0;
-  return launch_pdl(rmsnorm_kernel, dim3(static_cast<unsigned>(rows)), dim3(128), 0, st, x,
+  auto* kernel = d <= 512    ? rmsnorm_kernel<1>
+                 : d <= 1024 ? rmsnorm_kernel<2>
+                 : d <= 2048 ? rmsnorm_kernel<4>
+                             : rmsnorm_kernel<8>;
+  return launch_pdl(kernel, dim3(static_cast<unsigned>(rows)), dim3(128), 0, st, x,
                     static_cast<const __nv_bfloat16*>(w), static_cast<int>(d), eps, map,
                     static_cast<__nv_bfloat16*>(y)) == cudaSuccess
              ? 0

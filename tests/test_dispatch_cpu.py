@@ -172,3 +172,14 @@ def test_three_stream_estimate_counts_the_devices_multiprocessors(fake):
     for n in (4096, 6144, 8192):
         assert choice(0, 152, 2 * n) == choice(1, 76, n), n
     assert choice(1, 76, 8192) and not choice(1, 76, 6144)
+
+
+def test_rmsnorm_keeps_no_more_of_a_row_than_there_is(fake):
+    """The kernel by how many elements a thread keeps: a short row with the longest one's took 1.4
+    times its former time."""
+    keep = {}
+    for d in (8, 128, 512, 520, 1024, 1032, 2048, 2056, 4096, 11008):
+        assert fake.lib.hydra_rmsnorm(P, P, 5, d, 1e-6, 5, 5, 0, P, None) == 0
+        ((name, *_),) = fake.launches()
+        keep[d] = int(name.split("rmsnorm_kernelILi")[1].split("E")[0])
+    assert keep == {8: 1, 128: 1, 512: 1, 520: 2, 1024: 2, 1032: 4, 2048: 4, 2056: 8, 4096: 8, 11008: 8}

@@ -50,6 +50,18 @@ def test_rmsnorm_with_row_gather():
     assert_rel(host_f64(y), ref, TOL_LINEAR, "rmsnorm")
 
 
+@pytest.mark.parametrize("d", [8, 512, 520, 1024, 1032, 2048, 2056, 4096, 4104, 11008])
+def test_rmsnorm_by_row_length(d):
+    """The edges of what the kernels keep of a row in registers."""
+    x = synth.normal_f32(515 + d, (7, d), 2.0)
+    w = synth.normal_bf16(516 + d, (d,), 0.5)
+    y = torch.full((7, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    H.hydra_rmsnorm(dev_f32(x), dev_bf16(w), 1e-6, y)
+    x64 = x.astype(np.float64)
+    ref = x64 / np.sqrt(np.mean(x64 * x64, axis=1, keepdims=True) + 1e-6) * f64(w)
+    assert_rel(host_f64(y), ref, 2.0 ** -8 + 1e-6, "rmsnorm")  # one bf16 rounding
+
+
 def test_rope_q_k_rotated_v_untouched():
     H_, Dh, S, P = 3, 128, 2, 70
     d = H_ * Dh
