@@ -516,14 +516,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     if (p.deferred && n_local > 0)
       for (int kl = 0; kl < prev.n_lora && ok; ++kl)
         load(&mp.u[prev.stream == 2 ? 1 : 0], kl * BK, prev.m0, &mp.b[prev.stream == 2 ? 1 : 0], kl * BK, prev.n0);
-    pdl_launch_dependents();
     // copies still in flight must land before the CTA's shared memory is released
     for (int k = (it > STAGES ? it - STAGES : 0); k < it; ++k) {
       volatile int no_abort = 0;
       warp_wait_bounded(full_bar(k % STAGES), (k / STAGES) & 1, &no_abort, p.err, kDevTimeoutDrain);
     }
   } else if (warp == 1) {
-    pdl_launch_dependents();  // the dependents start once every warp has said so
     // ------------------------------------------------------------ MMA issuer (whole warp,
     // one elected lane issues; the same lane issues every MMA and commit, so each commit
     // covers all MMAs before it)
@@ -611,6 +609,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       if (p.deferred) {
         if (!mbar_wait_bounded(acc_full(b), 0, abort_flag, p.err, kDevTimeoutEpilogue)) break;
         tc_fence_after();
+        if (j == n_local - 1) pdl_launch_dependents();
         drain(acc, q, lane, staging, chunk_ctr, p, tl.m0, tl.n0, y_off, nullptr, py_off, nullptr);
         tc_fence_before();
         mbar_arrive(acc_mid(b));
@@ -621,6 +620,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (!mbar_wait_bounded(acc_full(b), (j >> 1) & 1, abort_flag, p.err, kDevTimeoutEpilogue))
           break;
         tc_fence_after();
+        // A CTA has let its dependents in once any thread of it says so: here, when the products of
+        // its last tile are done. (At its start: 128 rows x 1024 x 32000, two streams, with the
+        // combining launch 29.6 us, 25.9 so, 26.3 without; 144 LM heads of up to 128 rows 0.8 %.)
         if (j == n_local - 1) pdl_launch_dependents();
         if (p.shared_x)
           drain(acc, q, lane, staging, chunk_ctr, p, tl.m0, tl.n0, tl.n_lora > 0 ? nullptr : y_off, y_on,
