@@ -110,7 +110,13 @@ size_t hydra_lora_linear_workspace_size(int64_t M, int64_t r);
  *           reused as soon as the call's work on `stream` has completed.
  * Requirements: K % 8 == 0 and N % 8 == 0 (16-byte rows), all pointers 16-byte aligned,
  * M, N, K < 2^31. M == 0 is a no-op. Up to 16 token rows over both streams take the
- * memory-bound GEMV kernel; larger M the tcgen05 tensor-core kernel.
+ * memory-bound GEMV kernel; larger M the tcgen05 tensor-core kernels.
+ * Bits: sums are fp32. On the tensor-core kernels equal rows of x give equal bits in every call of one
+ * (M, K, N), whatever the streams, the outputs wanted and the epilogue, and for any M as well where K is
+ * summed in one piece. For up to 512 rows of a long K and few columns (K > 1920 and at most 24
+ * blocks of 128 rows x 256 columns in a stream) two halves of K are summed apart, and the GEMV sums
+ * four or eight parts: there a row's bits depend on M. algo 3 of hydra_lora_linear_algo always sums
+ * in one piece.
  */
 hydra_status hydra_lora_linear(const void* x_off, const void* x_on, int64_t M, int64_t K,
                                int64_t N, const void* W, const void* A, const void* B, int64_t r,
@@ -170,7 +176,8 @@ hydra_status hydra_skinny_linear(const void* x, int64_t M, int64_t K, int64_t N,
  * tile comes from HBM once and again from L2. Inputs may alias one another (the first
  * layer of a pass); any output may be NULL (not all three), and a NULL output's LoRA set may
  * be NULL. With A_crit = A_act, B_crit = B_act and x_crit = x_act, y_crit equals y_act bit
- * for bit (J-Hydra's single LoRA set). Layouts, alignment and errors as hydra_lora_linear;
+ * for bit (J-Hydra's single LoRA set), and y_off and y_act those of hydra_lora_linear (algo 1).
+ * Layouts, alignment and errors as hydra_lora_linear;
  * workspace: hydra_lora_linear_tri_workspace_size(M, r) bytes (both u).
  */
 size_t hydra_lora_linear_tri_workspace_size(int64_t M, int64_t r);
@@ -577,7 +584,7 @@ hydra_status hydra_score_llama(const hydra_llama_config* cfg, const hydra_llama_
  * the actor's LoRA set w->layers (logp_actor) and the critic's LoRA set critic[l] (a HOST
  * array of n_layers entries, same rank r), whose final hidden states give the values through
  * the reward head (r_phi <- LO(V)): values_t = w_rm . h_critic[P0 + t - 1]. With critic equal
- * to the actor's LoRA pointers the outputs equal hydra_score_llama's (J-Hydra-PPO).
+ * to the actor's LoRA pointers the outputs equal hydra_score_llama's (J-Hydra-PPO) bit for bit.
  * Workspace: hydra_score_llama_hydra_workspace_size(cfg, S); other arguments and errors as
  * hydra_score_llama; NULL critic -> HYDRA_ERR_NULL.
  */

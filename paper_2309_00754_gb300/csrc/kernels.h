@@ -15,7 +15,7 @@ namespace hydra {
 
 // Launch with programmatic stream serialisation: the kernel may begin while the preceding
 // kernel of the stream finishes, and must call pdl_wait() (common.cuh) before reading
-// anything that work may write or writing anything.
+// anything that work may write or writing anything (one exception there: GemmArgs::x_settled).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t stream, Args&&... args) {
@@ -54,8 +54,9 @@ struct GemmArgs {
   int epi = 0;        // tcgen05 epilogue: 0 store, 1 SwiGLU, 2 residual add (fp32), 3 rotary,
                       // 4 log-softmax partials
   bool single_cta = false;  // tcgen05: never use the CTA-pair (cta_group::2) kernel
-  // the kernel launched just before on the stream is this call's lora_down: the inputs x were
-  // final before it let its dependents start (only u is still being written)
+  // the kernel launched just before on the stream is this call's lora_down, with `settle`: x, W and all
+  // else that is older were final before it let its dependents start (only u is still being
+  // written), so the linear may read them before pdl_wait() (see there)
   bool x_settled = false;
   // epi 3 (rotary): columns [0, rope_cols) rotate in heads of 128 at position row % rope_P,
   // by the (cos, sin) pairs of rope_table [rope_P][64] (launch_rope_table)

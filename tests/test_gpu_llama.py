@@ -715,3 +715,29 @@ def test_score_llama_hydra_one_lora_set_is_j_hydra():
     jh = run_pass(cfg, sep, ids, lengths)
     for k in got:
         assert np.array_equal(got[k], jh[k]), k
+
+
+@pytest.mark.parametrize("S,P0,L", [(1, 37, 60), (3, 50, 50), (2, 100, 90)])
+def test_score_llama_hydra_one_lora_set_is_j_hydra_at_7b_width(S, P0, L):
+    """The same at the sizes where two and three streams take different kernels (97, 150 and 190 rows
+    of 4096 columns by 12288 and 22016), first and last layer included."""
+    cfg = dict(n_layers=2, d_model=4096, n_heads=32, head_dim=128, ffn=11008, vocab=1024, prompt_len=P0,
+               response_len=L, lora_rank=16, lora_scale=2.0, rms_eps=1e-6, rope_theta=10000.0, beta=0.1,
+               gamma=1.0, lam=0.95)
+    w = llama.random_device_weights(cfg, 5, "cuda")
+    ids = dev_i32(synth.randint(673, (S, P0 + L), 0, 1024))
+    lengths = dev_i32(np.array([L, L - 7, 3], dtype=np.int32)[:S])
+    out = []
+    for critic in (None, {k: w[k] for k in llama.LORA_KEYS}):
+        o = llama.alloc_outputs(S, L, "cuda")
+        if critic is None:
+            ws = torch.empty(H.score_llama_workspace_size(cfg, S), dtype=torch.uint8, device="cuda")
+            H.hydra_score_llama(cfg, w, ids, lengths, ws, o)
+        else:
+            ws = torch.empty(H.score_llama_hydra_workspace_size(cfg, S), dtype=torch.uint8, device="cuda")
+            H.hydra_score_llama_hydra(cfg, w, critic, ids, lengths, ws, o)
+        torch.cuda.synchronize()
+        out.append(o)
+    for k in out[0]:
+        assert torch.equal(out[0][k], out[1][k]), k
+    assert H.device_error(clear=True) == 0
