@@ -1026,7 +1026,10 @@ int launch_dual_lora_gemm_tc(const GemmArgs& a, cudaStream_t stream) {
   const bool lsm_ok = a.epi != EPI_LOGSOFTMAX || (!a.shared_x && a.M <= BM);
   // Log-softmax of up to 64 rows of two streams without LoRA: both fit one 128-row tile here, and
   // 32000 columns are 125 of these tiles on 152 SMs where the few-rows kernel has two waves of
-  // pairs (60 rows x 4096 x 32000, with the combining launch: 52.6 us, 60.2 there).
+  // pairs (60 rows x 4096 x 32000, with the combining launch: 52.6 us, 60.2 there; 24000 columns
+  // 42.9, 55.6). Up to 19456 columns it has one wave and is the faster one (16000 columns 36.7,
+  // 30.7; 4000 30.8, 25.5), but merges a row's partial sums in another order than the tiles do for
+  // more rows, so they are not sent there.
   const bool packed = a.epi == EPI_LOGSOFTMAX && !a.shared_x && a.x_crit == nullptr && a.r == 0 && a.M <= BM / 2 &&
                       a.y_off != nullptr && a.y_on != nullptr;
   const int streams = a.shared_x ? 1 : (a.x_crit != nullptr ? 3 : 2);
