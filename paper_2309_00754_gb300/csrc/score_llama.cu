@@ -346,8 +346,8 @@ static hydra_status score_pass(const hydra_llama_config* cfg, const hydra_llama_
   // score, at the last valid token). Its q/k/v projection and attention run over every
   // position (the prompt's keys and values); from the o projection on it runs on those
   // Lc = L + 1 rows of each sequence, gathered into compact buffers: per row the same
-  // arithmetic, and the same bits where both row counts take the same kernel (the few-rows
-  // linear adds a sum's two halves of K apart).
+  // arithmetic, and the same bits unless the few-rows linear adds a sum's two halves of K
+  // apart for one of the row counts.
   const int64_t Lc = L + 1, Tc = S * Lc;
   const bool compact = Lc < P;
   const hydra::RowMap pick{Lc, P, c.prompt_len - 1};  // compact row -> row of the full stream
